@@ -124,6 +124,9 @@ struct sb_ctx {
   double* d_bestE = nullptr;
   int32_t* d_bestr = nullptr;
   uint8_t* d_T = nullptr;
+  uint8_t* d_bits = nullptr;    // selections of eR replicas as bits (whole-number couplings)
+  bool b_whole = false;         // couplings are whole numbers of 2^-8 (k_energy_bits)
+  int32_t* d_inexact = nullptr;  // k_convert's verdict on that
   int8_t* d_spins = nullptr;
   int32_t spins_cap_R = 0;
   // host copy of the (global) CSR structure, for weight updates and re-tiling
@@ -377,6 +380,7 @@ sb_status validate_csr(int32_t n, int64_t nnz, const int32_t* rowptr, const int3
 }
 
 void free_readout(sb_ctx* c) {
+  dfree(c->d_bits);
   dfree(c->d_partial);
   dfree(c->d_Eall);
   c->eR = 0;
@@ -482,6 +486,7 @@ void free_all(sb_ctx* c) {
   dfree(c->d_bestE);
   dfree(c->d_bestr);
   dfree(c->d_T);
+  dfree(c->d_inexact);
   dfree(c->d_spins);
   dfree(c->d_blk_row0);
   dfree(c->d_blk_u0);
@@ -552,11 +557,17 @@ sb_status ensure_state(sb_ctx* c, int32_t R) {
 
 sb_status ensure_readout(sb_ctx* c, int32_t R) {
   const sbd::Tiling t = sbd::make_tiling(R);
-  const int32_t rows = std::max(kEnergyRowsMin, 256 / t.G);
-  if (c->eR == R && c->energy_rows == rows && c->d_partial && c->d_Eall) return SB_OK;
+  int32_t rows = std::max(kEnergyRowsMin, 256 / t.G);
+  // whole-number couplings: larger blocks where that still leaves eight CTAs
+  // per SM (fewer partial sums to add; the 472,812-row event: 2 ms of block sums)
+  if (c->b_whole) rows = std::min(sbd::kEnergyBitRows, std::max(kEnergyRowsMin, c->n / (152 * 8) / 64 * 64));
+  if (c->eR == R && c->energy_rows == rows && c->d_partial && c->d_Eall &&
+      (!c->b_whole || c->d_bits))
+    return SB_OK;
   free_readout(c);
   sb_status st = ensure_energy_blocks(c, rows);
   if (st) return st;
+  if (c->b_whole && (st = dalloc(&c->d_bits, (size_t)c->n * sbd::energy_bit_stride(R)))) return st;
   if ((st = dalloc(&c->d_partial, (size_t)c->nblk * R)) ||
       (st = dalloc(&c->d_Eall, (size_t)c->E * R)))
     return st;
@@ -1136,6 +1147,14 @@ void note_j_range(sb_ctx* c) {
   c->j_small = m < 0x1p118;
 }
 
+// k_convert's verdict on the couplings: whole numbers of 2^-8, held exactly by J
+sb_status note_whole(sb_ctx* c) {
+  int32_t v = 1;
+  SB_CUDA(cudaMemcpy(&v, c->d_inexact, 4, cudaMemcpyDeviceToHost));
+  c->b_whole = v == 0;
+  return SB_OK;
+}
+
 sb_status create_common(sb_ctx* c, const int32_t* rowptr, const int32_t* col, const double* qval,
                         const double* qlin) {
   SB_CUDA(cudaGetDevice(&c->device));
@@ -1161,8 +1180,9 @@ sb_status create_common(sb_ctx* c, const int32_t* rowptr, const int32_t* col, co
     }
     SB_CUDA(cudaMemset(c->d_J, 0, jb));
   }
-  if ((st = dalloc(&c->d_err, 1))) return st;
+  if ((st = dalloc(&c->d_err, 1)) || (st = dalloc(&c->d_inexact, 1))) return st;
   SB_CUDA(cudaMemset(c->d_err, 0, sizeof(int)));
+  SB_CUDA(cudaMemset(c->d_inexact, 0, sizeof(int)));
   SB_CUDA(cudaMemcpy(c->d_rowptr, rowptr, (n + 1) * 4, cudaMemcpyHostToDevice));
   if (nnz) {
     SB_CUDA(cudaMemcpy(c->d_col, col, nnz * 4, cudaMemcpyHostToDevice));
@@ -1185,7 +1205,8 @@ sb_status create_common(sb_ctx* c, const int32_t* rowptr, const int32_t* col, co
     return st;
   }
   cudaError_t e1 = sbd::launch_convert(c->d_rowptr, c->d_col, c->d_qval, c->d_qlin, c->n, c->d_J,
-                                       c->jbf16, c->d_h64, c->d_h32, row_off, row_sq, 0);
+                                       c->jbf16, c->d_h64, c->d_h32, row_off, row_sq,
+                                       c->d_inexact, 0);
   cudaError_t e2 = sbd::launch_event_stats(row_off, row_sq, c->d_ev_row0, c->E, c->d_offset,
                                            c->d_sigma, c->d_c0auto, 0);
   cudaError_t e3 = cudaDeviceSynchronize();
@@ -1201,6 +1222,7 @@ sb_status create_common(sb_ctx* c, const int32_t* rowptr, const int32_t* col, co
   SB_CUDA(cudaMemcpy(c->sigma.data(), c->d_sigma, c->E * 8, cudaMemcpyDeviceToHost));
   SB_CUDA(cudaMemcpy(c->c0_auto.data(), c->d_c0auto, c->E * 8, cudaMemcpyDeviceToHost));
   note_j_range(c);
+  if (sb_status st2 = note_whole(c)) return st2;
   SB_CUDA(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   return SB_OK;
 }
@@ -2196,11 +2218,37 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   return SB_OK;
 }
 
-// Energies of R replicas (from the current x, or from d_spins) into d_Eall, arg-min into
-// d_bestE / d_bestr.
-sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s) {
+// Energies of R replicas (from the current x, or from d_spins) into E_all (NULL:
+// d_Eall), arg-min into best_E / best_r (NULL: d_bestE / d_bestr).
+sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
+                  double* E_all = nullptr, double* best_E = nullptr, int32_t* best_r = nullptr) {
   sb_status st = ensure_readout(c, R);
   if (st) return st;
+  if (!E_all) E_all = c->d_Eall;
+  if (!best_E) best_E = c->d_bestE;
+  if (!best_r) best_r = c->d_bestr;
+  if (c->b_whole) {
+    sbd::EnergyBitArgs b;
+    b.rowptr = c->d_rowptr;
+    b.col = c->d_col;
+    b.J = c->d_J;
+    b.jbf16 = c->jbf16;
+    b.qlin = c->d_qlin;
+    b.bits = c->d_bits;
+    b.bstride = sbd::energy_bit_stride(R);
+    b.blk_row = c->d_blk_row;
+    b.nblk = c->nblk;
+    b.n = c->n;
+    b.R = R;
+    b.partial = c->d_partial;
+    b.nnz = c->nnz;
+    SB_CUDA(sbd::launch_select_bits(d_spins ? nullptr : c->d_x[c->cur], R, d_spins, c->n, R,
+                                    c->d_bits, s));
+    SB_CUDA(sbd::launch_energy_bits(b, s));
+    SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
+    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, s));
+    return SB_OK;
+  }
   const sbd::Tiling t = sbd::make_tiling(R);
   sbd::EnergyArgs a;
   a.rowptr = c->d_rowptr;
@@ -2217,8 +2265,8 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s) {
   a.partial = c->d_partial;
   a.nnz = c->nnz;
   SB_CUDA(sbd::launch_energy_partial(t, a, s));
-  SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, c->d_Eall, s));
-  SB_CUDA(sbd::launch_argmin(c->d_Eall, c->E, R, c->d_bestE, c->d_bestr, s));
+  SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
+  SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, s));
   return SB_OK;
 }
 
@@ -2642,17 +2690,22 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
       return SB_ERR_STATE;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    sb_status st = readout(ctx, nullptr, ctx->R, s);
+    // the kernels write the caller's buffers themselves where they are aligned
+    // for their type, else through the context's own and a copy
+    auto direct = [](void* p, size_t a) { return p && reinterpret_cast<uintptr_t>(p) % a == 0; };
+    const bool dE = direct(d_E_all, 8), db = direct(d_best_E, 8), dr = direct(d_best_r, 4);
+    sb_status st = readout(ctx, nullptr, ctx->R, s, dE ? d_E_all : nullptr,
+                           db ? d_best_E : nullptr, dr ? d_best_r : nullptr);
     if (st) return st;
     if (d_T)
-      SB_CUDA(sbd::launch_best_T(ctx->d_x[ctx->cur], ctx->d_row_event, ctx->d_bestr, ctx->n,
-                                 ctx->R, d_T, s));
-    if (d_E_all)
+      SB_CUDA(sbd::launch_best_T(ctx->d_x[ctx->cur], ctx->d_row_event,
+                                 dr ? d_best_r : ctx->d_bestr, ctx->n, ctx->R, d_T, s));
+    if (d_E_all && !dE)
       SB_CUDA(cudaMemcpyAsync(d_E_all, ctx->d_Eall, (size_t)ctx->E * ctx->R * 8,
                               cudaMemcpyDeviceToDevice, s));
-    if (d_best_E)
+    if (d_best_E && !db)
       SB_CUDA(cudaMemcpyAsync(d_best_E, ctx->d_bestE, ctx->E * 8, cudaMemcpyDeviceToDevice, s));
-    if (d_best_r)
+    if (d_best_r && !dr)
       SB_CUDA(cudaMemcpyAsync(d_best_r, ctx->d_bestr, ctx->E * 4, cudaMemcpyDeviceToDevice, s));
     return SB_OK;
   });
@@ -2726,6 +2779,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     SB_CUDA(cudaMemcpy(ctx->d_quality, quality, (size_t)n * 8, cudaMemcpyHostToDevice));
     SB_CUDA(cudaMemcpy(ctx->d_nconf, nconf.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
     SB_CUDA(cudaMemcpy(ctx->d_qlin, ql.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
+    SB_CUDA(cudaMemset(ctx->d_inexact, 0, sizeof(int)));
     double *row_off = nullptr, *row_sq = nullptr;
     if ((st = dalloc(&row_off, (size_t)n)) || (st = dalloc(&row_sq, (size_t)n))) {
       dfree(row_off);
@@ -2734,7 +2788,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     }
     cudaError_t e1 = sbd::launch_convert(ctx->d_rowptr, ctx->d_col, ctx->d_qval, ctx->d_qlin, n,
                                          ctx->d_J, ctx->jbf16, ctx->d_h64, ctx->d_h32, row_off,
-                                         row_sq, 0);
+                                         row_sq, ctx->d_inexact, 0);
     cudaError_t e2 = sbd::launch_event_stats(row_off, row_sq, ctx->d_ev_row0, 1, ctx->d_offset,
                                              ctx->d_sigma, ctx->d_c0auto, 0);
     cudaError_t e3 = cudaDeviceSynchronize();
@@ -2747,6 +2801,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     SB_CUDA(cudaMemcpy(ctx->sigma.data(), ctx->d_sigma, 8, cudaMemcpyDeviceToHost));
     SB_CUDA(cudaMemcpy(ctx->c0_auto.data(), ctx->d_c0auto, 8, cudaMemcpyDeviceToHost));
     note_j_range(ctx);
+    if ((st = note_whole(ctx))) return st;
     // the tiled kernel's packed words carry J: rebuild them
     dfree(ctx->d_blk_row0);
     dfree(ctx->d_blk_u0);

@@ -1057,14 +1057,17 @@ __device__ __forceinline__ void store_j(__nv_bfloat16* J, int p, double v) {
 template <typename JT>
 __global__ void k_convert(const int32_t* rowptr, const int32_t* col, const double* qval,
                           const double* qlin, int32_t n, JT* J, double* h64, float* h32,
-                          double* row_off, double* row_sq) {
+                          double* row_off, double* row_sq, int32_t* inexact) {
+  bool whole = true;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double s = 0.0, lo = 0.0, sq = 0.0;
+    double s = 0.0, lo = 0.0, sq = 0.0, mag = 0.0;
     for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
       const double b = qval[p];
       s += b;
       const double jv = -b / 4.0;
       store_j(J, p, jv);
+      mag += fabs(b);
+      whole = whole && (double)(float)J[p] == jv && rint(b * 256.0) == b * 256.0;
       sq += jv * jv;
       if (col[p] < i) lo += b;
     }
@@ -1073,7 +1076,9 @@ __global__ void k_convert(const int32_t* rowptr, const int32_t* col, const doubl
     h32[i] = (float)hv;
     row_off[i] = qlin[i] / 2.0 + lo / 4.0;
     row_sq[i] = sq;
+    whole = whole && mag <= 16384.0;
   }
+  if (inexact && !whole) *inexact = 1;
 }
 
 // one block per event: fixed-order tree reduction of the per-row terms
@@ -1200,13 +1205,162 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
   }
 }
 
-__global__ void k_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t R,
-                                double* out) {
+// ---------------------------------------------------------------- energies from selection bits
+// FP64 arithmetic is scarce on this part (about two FMAs per clock and SM, a
+// 64th of the FP32 rate), and the energy of R replicas is nnz x R of them. The
+// QUBOs of Eq. 13 carry couplings that are small whole numbers (-1 and w_c), so
+// sum_j b_ij T_j is a whole number too: it is summed exactly in integers, in any
+// order, from the selections as bits, and only the linear terms (n x R) and the
+// block sums stay in FP64. Bits also cut the gather: a neighbour's 256 replicas
+// are one 32-byte sector instead of 1 KB of positions. Bound by integer issue
+// (about two instructions per nonzero and replica). Whole readout of the
+// 39,165-row event at R = 256: 1791 us with k_energy_partial and serial block
+// sums, 273 us here; the error against 64-bit sums falls from 7e-16 to 2e-16.
+
+// Bits of one row's selections: a warp takes 32 replicas of a row at a time
+// (one coalesced 128-byte load, one ballot) when R >= 16, a thread a whole row
+// otherwise. Bits past R are zero.
+__global__ void __launch_bounds__(kBlock) k_select_bits(const float* x, int32_t xstride,
+                                                        const int8_t* spins, int32_t n, int32_t R,
+                                                        int32_t words, uint32_t* bits) {
+  if (R < 16) {
+    const int row = blockIdx.x * kBlock + threadIdx.x;
+    if (row >= n) return;
+    uint32_t w = 0;
+    for (int r = 0; r < R; ++r) {
+      const bool t = x ? __ldg(x + (size_t)row * xstride + r) > 0.f
+                       : spins[(size_t)row * R + r] > 0;
+      w |= (t ? 1u : 0u) << r;
+    }
+    bits[row] = w;
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const int64_t total = (int64_t)n * words;
+  const int64_t step = (int64_t)gridDim.x * (kBlock / 32);
+  for (int64_t i = (int64_t)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5); i < total; i += step) {
+    const int64_t row = i / words;
+    const int r = (int)(i - row * words) * 32 + lane;
+    bool t = false;
+    if (r < R) t = x ? __ldg(x + (size_t)row * xstride + r) > 0.f : spins[(size_t)row * R + r] > 0;
+    const uint32_t w = __ballot_sync(0xffffffffu, t);
+    if (lane == 0) bits[i] = w;
+  }
+}
+
+// 256 b of a coupling from its stored J = -b / 4 (whole numbers below 2^22: the
+// FP32 sum with 1.5 * 2^23 is exact and holds the number in its low bits)
+__device__ __forceinline__ int whole_b(float j) {
+  return __float_as_int(fmaf(j, -1024.f, 12582912.f)) - 0x4B400000;
+}
+
+// A team of L x S lanes owns a row: lane l of slice s holds the replicas 8 l ..
+// 8 l + 7 (one byte of bits per neighbour) of every S-th nonzero, four in
+// flight. Few replicas leave few bytes per row, so the slices then share a
+// row's nonzeros (whole-number sums: any split gives the same value).
+template <typename JT>
+__global__ void __launch_bounds__(kBlock) k_energy_bits(const EnergyBitArgs a, int L, int S) {
+  extern __shared__ double sm[];
+  const int TS = L * S;
+  const int team = threadIdx.x / TS, t = threadIdx.x - team * TS;
+  const int teams = kBlock / TS;
+  const int sl = t / L, bl = t - sl * L;
+  const int byte = blockIdx.y * 32 + bl;
+  const bool have = byte < a.bstride;
+  const uint8_t* bits = a.bits + (have ? byte : 0);
+  const JT* J = static_cast<const JT*>(a.J);
+  const int lane = threadIdx.x & 31;
+  const unsigned mask = TS == 32 ? 0xffffffffu : (((1u << TS) - 1u) << (lane & ~(TS - 1)));
+  const int b = blockIdx.x;
+  const int r0 = a.blk_row[b], r1 = a.blk_row[b + 1];
+  int pair[8];     // sum over the rows of T_i sum_j 256 b_ij T_j
+  double lin[8];   // sum over the rows of T_i a_i
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    pair[v] = 0;
+    lin[v] = 0.0;
+  }
+  for (int row = r0 + team; row < r1; row += teams) {
+    int in[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) in[v] = 0;
+    int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
+    chk_rows(p0, p1, a.nnz);
+    const unsigned own = bits[(size_t)row * a.bstride];
+    for (int p = p0 + sl; p < p1; p += 4 * S) {
+      int ib[4];
+      unsigned w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = p + u * S;
+        const bool in_row = q < p1;
+        const int c = chk_idx(__ldg(a.col + (in_row ? q : p)), a.n, kChkCol);
+        ib[u] = in_row ? whole_b(jval(J, q)) : 0;
+        w[u] = __ldg(bits + (size_t)c * a.bstride);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+          if (w[u] & (1u << v)) in[v] += ib[u];
+    }
+    for (int off = L; off < TS; off <<= 1)
+#pragma unroll
+      for (int v = 0; v < 8; ++v) in[v] += __shfl_xor_sync(mask, in[v], off);
+    const double ai = __ldg(a.qlin + row);
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+      if (own & (1u << v)) {
+        pair[v] += in[v];
+        lin[v] += ai;
+      }
+  }
+  // the teams' sums in team order: E = sum T a + (1/2) sum T b T
+  const int W = 8 * L;
+  if (sl == 0)
+#pragma unroll
+    for (int v = 0; v < 8; ++v) sm[team * W + 8 * bl + v] = lin[v] + (double)pair[v] * 0x1p-9;
+  __syncthreads();
+  for (int w = threadIdx.x; w < W; w += kBlock) {
+    const int rep = blockIdx.y * 256 + w;
+    if (rep >= a.R) continue;
+    double s = 0.0;
+    for (int k = 0; k < teams; ++k) s += sm[k * W + w];
+    a.partial[(size_t)b * a.R + rep] = s;
+  }
+}
+
+// Sum over an event's blocks: a warp takes every kReduceWarps-th block for 32
+// replicas, eight loads in flight, and the warps' sums are added in warp order
+// (one thread per replica walking all blocks was a chain of as many memory
+// round trips: 230 us for 617 blocks).
+constexpr int kReduceWarps = 32;
+__global__ void __launch_bounds__(32 * kReduceWarps) k_energy_reduce(const double* partial,
+                                                                     const int32_t* ev_blk0,
+                                                                     int32_t R, double* out) {
+  __shared__ double sm[kReduceWarps][32];
   const int e = blockIdx.y;
   const int b0 = ev_blk0[e], b1 = ev_blk0[e + 1];
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = b0; b < b1; ++b) s += partial[(size_t)b * R + r];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int r = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (r < R) {
+    int b = b0 + wid;
+    for (; b + 7 * kReduceWarps < b1; b += 8 * kReduceWarps) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = __ldg(partial + (size_t)(b + u * kReduceWarps) * R + r);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; b < b1; b += kReduceWarps) s += __ldg(partial + (size_t)b * R + r);
+  }
+  sm[wid][lane] = s;
+  __syncthreads();
+  if (wid == 0 && r < R) {
+    s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kReduceWarps; ++w) s += sm[w][lane];
     out[(size_t)e * R + r] = s;
   }
 }
@@ -1263,10 +1417,10 @@ __global__ void k_argmin(const double* E_all, int32_t R, double* best_E, int32_t
 }
 
 __global__ void k_best_T(const float* x, const int32_t* row_event, const int32_t* best_r,
-                         int32_t n, int32_t R, uint8_t* T) {
+                         int32_t n, int32_t xstride, uint8_t* T) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int e = row_event ? row_event[i] : 0;
-    T[i] = x[(size_t)i * R + best_r[e]] > 0.f ? 1 : 0;
+    T[i] = x[(size_t)i * xstride + best_r[e]] > 0.f ? 1 : 0;
   }
 }
 
@@ -1449,16 +1603,17 @@ cudaError_t launch_set_c0(float* c0_ev, const double* c0_auto, double c0, int32_
 
 cudaError_t launch_convert(const int32_t* rowptr, const int32_t* col, const double* qval,
                            const double* qlin, int32_t n, void* J, int jbf16, double* h64,
-                           float* h32, double* row_off, double* row_sq, cudaStream_t s) {
+                           float* h32, double* row_off, double* row_sq, int32_t* inexact,
+                           cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int grid = grid_for(n, kBlock);
   if (jbf16)
     k_convert<__nv_bfloat16><<<grid, kBlock, 0, s>>>(rowptr, col, qval, qlin, n,
                                                      static_cast<__nv_bfloat16*>(J), h64, h32,
-                                                     row_off, row_sq);
+                                                     row_off, row_sq, inexact);
   else
     k_convert<float><<<grid, kBlock, 0, s>>>(rowptr, col, qval, qlin, n, static_cast<float*>(J),
-                                             h64, h32, row_off, row_sq);
+                                             h64, h32, row_off, row_sq, inexact);
   return cudaGetLastError();
 }
 
@@ -1485,8 +1640,34 @@ cudaError_t launch_energy_partial(const Tiling& t, const EnergyArgs& a, cudaStre
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
                                  int32_t R, double* E_out, cudaStream_t s) {
   if (E <= 0 || R <= 0) return cudaSuccess;
-  dim3 grid((R + kBlock - 1) / kBlock, E);
-  k_energy_reduce<<<grid, kBlock, 0, s>>>(partial, ev_blk0, R, E_out);
+  dim3 grid((R + 31) / 32, E);
+  k_energy_reduce<<<grid, 32 * kReduceWarps, 0, s>>>(partial, ev_blk0, R, E_out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_select_bits(const float* x, int32_t xstride, const int8_t* spins, int32_t n,
+                               int32_t R, uint8_t* bits, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const int32_t words = energy_bit_stride(R) / 4;
+  const size_t threads = R < 16 ? (size_t)n : (size_t)n * words * 32;
+  const unsigned grid = R < 16 ? (unsigned)((n + (int64_t)kBlock - 1) / kBlock)
+                               : (unsigned)grid_for(threads, kBlock);
+  k_select_bits<<<grid, kBlock, 0, s>>>(x, xstride, spins, n, R, words,
+                                        reinterpret_cast<uint32_t*>(bits));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s) {
+  if (a.nblk <= 0) return cudaSuccess;
+  int L = 1;
+  while (L < 32 && L < (a.R + 7) / 8) L *= 2;
+  const int S = L < 8 ? 8 / L : 1;
+  dim3 grid(a.nblk, (a.R + 255) / 256);
+  const size_t smem = (size_t)(kBlock / (L * S)) * 8 * L * sizeof(double);
+  if (a.jbf16)
+    k_energy_bits<__nv_bfloat16><<<grid, kBlock, smem, s>>>(a, L, S);
+  else
+    k_energy_bits<float><<<grid, kBlock, smem, s>>>(a, L, S);
   return cudaGetLastError();
 }
 
@@ -1498,9 +1679,9 @@ cudaError_t launch_argmin(const double* E_all, int32_t E, int32_t R, double* bes
 }
 
 cudaError_t launch_best_T(const float* x, const int32_t* row_event, const int32_t* best_r,
-                          int32_t n, int32_t R, uint8_t* T, cudaStream_t s) {
+                          int32_t n, int32_t xstride, uint8_t* T, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_best_T<<<grid_for(n, kBlock), kBlock, 0, s>>>(x, row_event, best_r, n, R, T);
+  k_best_T<<<grid_for(n, kBlock), kBlock, 0, s>>>(x, row_event, best_r, n, xstride, T);
   return cudaGetLastError();
 }
 

@@ -105,9 +105,13 @@ cudaError_t launch_set_c0(float* c0_ev, const double* c0_auto, double c0, int32_
                           cudaStream_t s);
 
 // QUBO -> Ising in FP64 (per row), then per-event reductions.
+// *inexact (device, may be NULL): set to 1 when some b_ij is no whole number of
+// 2^-8, is not -4 times its stored J, or a row's sum of |b_ij| exceeds 2^14
+// (k_energy_bits needs the couplings as whole numbers).
 cudaError_t launch_convert(const int32_t* rowptr, const int32_t* col, const double* qval,
                            const double* qlin, int32_t n, void* J, int jbf16, double* h64,
-                           float* h32, double* row_off, double* row_sq, cudaStream_t s);
+                           float* h32, double* row_off, double* row_sq, int32_t* inexact,
+                           cudaStream_t s);
 cudaError_t launch_event_stats(const double* row_off, const double* row_sq,
                                const int32_t* ev_row0, int32_t E, double* offset,
                                double* sigma, double* c0_auto, cudaStream_t s);
@@ -126,6 +130,29 @@ struct EnergyArgs {
   int64_t nnz = INT64_MAX; // CSR entries, where known (bounds-checked build)
 };
 cudaError_t launch_energy_partial(const Tiling& t, const EnergyArgs& a, cudaStream_t s);
+
+// The same partial sums for QUBOs whose couplings are whole numbers of 2^-8
+// (launch_convert's test): selections as bits, couplings summed as integers.
+constexpr int kEnergyBitRows = 256;  // most rows of a block that one lane team sums in int32
+struct EnergyBitArgs {
+  const int32_t* rowptr;
+  const int32_t* col;
+  const void* J;           // -b / 4, FP32 or BF16, exact
+  int jbf16;
+  const double* qlin;
+  const uint8_t* bits;     // [n x bstride]: bit r & 7 of byte r >> 3 is T_r
+  int32_t bstride;         // bytes per row, a multiple of 4
+  const int32_t* blk_row;  // [nblk + 1]
+  int32_t nblk, n, R;
+  double* partial;         // [nblk x R]
+  int64_t nnz;
+};
+// bytes per row of the selection bits for R replicas
+inline int32_t energy_bit_stride(int R) { return (R + 31) / 32 * 4; }
+// bits of T = (x > 0), x [n] rows of xstride floats, or of spins [n x R] when x is NULL
+cudaError_t launch_select_bits(const float* x, int32_t xstride, const int8_t* spins, int32_t n,
+                               int32_t R, uint8_t* bits, cudaStream_t s);
+cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s);
 // E[e*R + r] = sum of the event's block partials, in block order.
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
                                  int32_t R, double* E_out, cudaStream_t s);
@@ -133,7 +160,7 @@ cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, 
 cudaError_t launch_argmin(const double* E_all, int32_t E, int32_t R, double* best_E,
                           int32_t* best_r, cudaStream_t s);
 cudaError_t launch_best_T(const float* x, const int32_t* row_event, const int32_t* best_r,
-                          int32_t n, int32_t R, uint8_t* T, cudaStream_t s);
+                          int32_t n, int32_t xstride, uint8_t* T, cudaStream_t s);
 
 // ---------------------------------------------------------------- bSB adjoint
 struct AdjArgs {
