@@ -107,6 +107,10 @@ struct sb_ctx {
   float* d_c0ev = nullptr;
   // device: state
   int32_t R = 0;
+  // replicas as stored: rows of x, y and the sign bytes are Rs >= R values
+  // apart, and the step kernels run all Rs (padded_replicas); replicas R .. Rs
+  // - 1 start from whatever their slots hold and are never read out
+  int32_t Rs = 0;
   float* d_x[2] = {nullptr, nullptr};
   float* d_y = nullptr;
   int cur = 0;
@@ -394,6 +398,7 @@ void free_state(sb_ctx* c) {
   dfree(c->d_sgn[0]);
   dfree(c->d_sgn[1]);
   c->R = 0;
+  c->Rs = 0;
   c->have_state = false;
   c->graph.reset();
 }
@@ -538,16 +543,35 @@ sb_status ensure_energy_blocks(sb_ctx* c, int32_t rows) {
   return SB_OK;
 }
 
+// Replicas as stored. Counts that are no multiple of 4 (the paper's 50 shots)
+// cannot take 16-byte loads, and dSB cannot take its sign bytes, so their rows
+// are padded: to the next power of two where that adds at most a third (50 ->
+// 64: the widest kernels of every variant), else to the next multiple of 4. Each
+// replica is computed as before, so the results are the same. Measured at 50
+// shots, us per step, unpadded / padded: 67,445 rows dSB 61 / 21, 10,214
+// rows bSB 8.2 / 4.9. Multiples of 4 stay as they are, and so does R = 1.
+int32_t padded_replicas(int32_t R) {
+  if (R == 1 || R % 4 == 0) return R;
+  int32_t p = 4;
+  while (p < R) p *= 2;
+  return (int64_t)3 * p <= (int64_t)4 * R ? p : (R + 3) / 4 * 4;
+}
+
 sb_status ensure_state(sb_ctx* c, int32_t R) {
   if (c->R == R && c->d_y) return SB_OK;
   free_state(c);
-  const size_t cnt = (size_t)c->n * R;
   // with a factor, the x buffers also hold the U rows after the n state rows
   const int64_t xr = (int64_t)c->n + (c->fac_set ? c->fac_urows : 0);
-  sb_status st;
-  if ((st = dalloc(&c->d_x[0], (size_t)xr * R)) || (st = dalloc(&c->d_x[1], (size_t)xr * R)) ||
-      (st = dalloc(&c->d_y, cnt)))
-    return st;
+  sb_status st = SB_OK;
+  // a padded state that does not fit is tried again without padding
+  for (int32_t Rs : {padded_replicas(R), R}) {
+    c->Rs = Rs;
+    if ((st = dalloc(&c->d_x[0], (size_t)xr * Rs)) || (st = dalloc(&c->d_x[1], (size_t)xr * Rs)) ||
+        (st = dalloc(&c->d_y, (size_t)c->n * Rs)))
+      free_state(c);
+    if (st != SB_ERR_OOM) break;
+  }
+  if (st) return st;
   c->x_rows = xr;
   c->R = R;
   c->cur = 0;
@@ -1741,7 +1765,7 @@ sb_status ensure_frw(sb_ctx* c, int RW) {
 // the n state rows.
 sb_status ensure_x_rows(sb_ctx* c, int64_t rows) {
   if (c->x_rows >= rows) return SB_OK;
-  const size_t cnt = (size_t)rows * c->R, keep = (size_t)c->n * c->R;
+  const size_t cnt = (size_t)rows * c->Rs, keep = (size_t)c->n * c->Rs;
   float* nx[2] = {nullptr, nullptr};
   sb_status st;
   if ((st = dalloc(&nx[0], cnt)) || (st = dalloc(&nx[1], cnt))) {
@@ -1780,12 +1804,12 @@ sb_status check_run_args(sb_ctx* c, sb_variant variant, double a0, double c0, do
 
 // Enqueue `steps` SB steps reading x from c->d_x[c->cur]; flips c->cur.
 sbd::Tiling step_tiling(const sb_ctx* c) {
-  if (c->groups > 1 && c->R % (4 * c->groups) == 0) {
-    const int rt = c->R / c->groups;
-    if (rt <= 128 && ((rt / 4) & (rt / 4 - 1)) == 0) return sbd::make_tiling_rt(c->R, rt);
+  if (c->groups > 1 && c->Rs % (4 * c->groups) == 0) {
+    const int rt = c->Rs / c->groups;
+    if (rt <= 128 && ((rt / 4) & (rt / 4 - 1)) == 0) return sbd::make_tiling_rt(c->Rs, rt);
   }
-  if (c->step_rt > 0 && c->R % c->step_rt == 0) return sbd::make_tiling_rt(c->R, c->step_rt);
-  return sbd::make_tiling(c->R);
+  if (c->step_rt > 0 && c->Rs % c->step_rt == 0) return sbd::make_tiling_rt(c->Rs, c->step_rt);
+  return sbd::make_tiling(c->Rs);
 }
 
 sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
@@ -1795,7 +1819,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     sb_status st0 = ensure_stream(c);
     if (st0) return st0;
   }
-  if (c->use_tiled && c->R % sbd::kTileRT == 0) {
+  if (c->use_tiled && c->Rs % sbd::kTileRT == 0) {
     sb_status st0 = ensure_tiles(c);
     if (st0) return st0;
   }
@@ -1803,8 +1827,9 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   // dSB needs the sign bytes and U sums that BF16 holds exactly
   int fG = 0, fNCH = 0, ftiles = 0;
   const int fac = (c->fac_set && c->fac_use != 0 && c->groups == 1 &&
-                   sbd::fac_tiling(variant, c->R, &fG, &fNCH, &ftiles) &&
-                   (variant != SB_DSB || (c->dsb_signs && c->j_small)))
+                   sbd::fac_tiling(variant, c->Rs, &fG, &fNCH, &ftiles) &&
+                   (variant != SB_DSB || (c->dsb_signs && c->j_small)) &&
+                   (c->Rs == c->R || (variant == SB_DSB && c->b_whole)))
                       ? 1 : 0;
   // dSB: BF16 U rows hold sums of at most 256 members exactly; larger blocks
   // take FP32 U rows (the dSB kernels' NCH = 2 instances)
@@ -1814,7 +1839,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   // aSB / bSB with R a multiple of 128: the row-group kernel over the extended
   // CSR, the U rows written into the x buffer after the n state rows
   int frw = 0;
-  if (fac && variant != SB_DSB && c->R % 128 == 0 && c->rw_rows != 0 && c->step_rt == 0) {
+  if (fac && variant != SB_DSB && c->Rs % 128 == 0 && c->rw_rows != 0 && c->step_rt == 0) {
     sb_status st0 = ensure_frw(c, 2);
     if (st0) return st0;
     if (c->frw_built == 2) {
@@ -1823,7 +1848,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     }
   }
   if (fac && !frw) {
-    const size_t ub = (size_t)std::max(c->fac_urows, 1) * c->R * (variant == SB_DSB && fNCH == 1 ? 2 : 4);
+    const size_t ub = (size_t)std::max(c->fac_urows, 1) * c->Rs * (variant == SB_DSB && fNCH == 1 ? 2 : 4);
     if (ub > c->f_U_bytes) {
       if (c->d_f_U) cudaFree(c->d_f_U);
       c->d_f_U = nullptr;
@@ -1851,7 +1876,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
       c->f_cnt_count = cnt_need;
       c->graph.reset();
     }
-    const size_t scr_need = (size_t)std::max(c->fac_nslots, 1) * c->fac_K * c->R;
+    const size_t scr_need = (size_t)std::max(c->fac_nslots, 1) * c->fac_K * c->Rs;
     if (scr_need > c->f_scr_count) {
       dfree(c->d_f_scr);
       c->f_scr_count = 0;
@@ -1873,7 +1898,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     fs.K = c->fac_K;
     fs.couple = c->fac_couple;
     fs.U = c->d_f_U;
-    fs.R = c->R;
+    fs.R = c->Rs;
     fs.G = fG;
     fs.NCH = fNCH;
     fs.tiles = ftiles;
@@ -1897,7 +1922,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     fa.dta0 = (float)(dt * a0);
     fa.y = c->d_y;
     fa.n = c->n;
-    fa.R = c->R;
+    fa.R = c->Rs;
     fa.G = fG;
     fa.NCH = fNCH;
     fa.tiles = ftiles;
@@ -1906,7 +1931,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   sbd::StreamArgs sa{};
   size_t s_smem = 0;
   if (!fac && c->use_stream && c->stream_ok && c->groups == 1) {
-    sa.W = sbd::stream_tile_width(c->R);
+    sa.W = sbd::stream_tile_width(c->Rs);
     if (sa.W) s_smem = sbd::stream_smem(sa.W, c->stream_jbuf, &sa.nst);
   }
   const int streamed = s_smem ? 1 : 0;
@@ -1917,12 +1942,12 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   // dSB keeps its sign-byte kernel (fewer instructions per neighbour)
   const int rw_want = c->rw_rows < 0 ? (variant == SB_DSB ? 0 : 2) : c->rw_rows;
   const bool rw_auto_ok = c->rw_rows >= 0 || (!c->use_tiled && c->step_rt == 0);
-  if (!fac && !streamed && rw_want && rw_auto_ok && c->groups == 1 && c->R % 128 == 0) {
+  if (!fac && !streamed && rw_want && rw_auto_ok && c->groups == 1 && c->Rs % 128 == 0) {
     sb_status st0 = ensure_rw(c, rw_want);
     if (st0) return st0;
     if (c->rw_built == rw_want) {
       rw = rw_want;
-      rw_nch = (c->R % 256 == 0 && c->step_rt != 128) ? 2 : 1;
+      rw_nch = (c->Rs % 256 == 0 && c->step_rt != 128) ? 2 : 1;
       ra.gptr = c->d_rw_gptr;
       ra.grows = c->d_rw_rows;
       ra.ent = c->d_rw_ent;
@@ -1936,13 +1961,13 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
       ra.dta0 = (float)(dt * a0);
       ra.y = c->d_y;
       ra.n = c->n;
-      ra.R = c->R;
+      ra.R = c->Rs;
       ra.ngroups = c->rw_ngroups;
       ra.gpc = std::max(sbd::kRwBlock / 32, c->step_rpc > 0 ? c->step_rpc / rw : 0);
       ra.cta_order = nullptr;
       const bool sgn_rw = variant == SB_DSB && c->dsb_signs && c->j_small;
       const int64_t ctas = ((int64_t)c->rw_ngroups + ra.gpc - 1) / ra.gpc;
-      if (heavy_first(c, (size_t)c->n * c->R * (sgn_rw ? 1 : 4), ctas)) {
+      if (heavy_first(c, (size_t)c->n * c->Rs * (sgn_rw ? 1 : 4), ctas)) {
         st0 = ensure_rw_order(c, ra.gpc);
         if (st0) return st0;
         ra.cta_order = c->d_rw_order;
@@ -1951,7 +1976,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   }
   if (frw) {
     rw = 2;
-    rw_nch = c->R % 256 == 0 ? 2 : 1;
+    rw_nch = c->Rs % 256 == 0 ? 2 : 1;
     ra.gptr = c->d_frw_gptr;
     ra.grows = c->d_frw_rows;
     ra.ent = c->d_frw_ent;
@@ -1965,7 +1990,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     ra.dta0 = (float)(dt * a0);
     ra.y = c->d_y;
     ra.n = c->n;
-    ra.R = c->R;
+    ra.R = c->Rs;
     ra.xrows = c->n + c->fac_urows;  // the extended CSR's columns n + u are U rows
     ra.ngroups = c->frw_ngroups;
     ra.gpc = std::max(sbd::kRwBlock / 32, c->step_rpc > 0 ? c->step_rpc / 2 : 0);
@@ -1985,14 +2010,14 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     sa.dta0 = (float)(dt * a0);
     sa.y = c->d_y;
     sa.n = c->n;
-    sa.R = c->R;
+    sa.R = c->Rs;
     sa.cta_blk0 = c->d_s_cta;
     sa.blk = reinterpret_cast<const int4*>(c->d_s_blk);
     sa.rjo = c->d_s_rjo;
     sa.ucol = c->d_s_ucol;
     sa.umask = c->d_s_umask;
     sa.grid = c->stream_grid;
-    sa.tiles = c->R / sa.W;
+    sa.tiles = c->Rs / sa.W;
     sa.jbuf_bytes = c->stream_jbuf;
     sa.err = c->d_err;
     sa.wait_ns = c->wait_ns;
@@ -2002,9 +2027,9 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   // byte condition below must agree
   const bool dsb16 = !fac && !streamed && !rw && variant == SB_DSB && c->dsb_signs && c->j_small &&
                      c->step_rt == 0 &&
-                     c->groups == 1 && sbd::dsb16_ok(c->R) &&
-                     !(c->tiled_ok && c->use_tiled && c->R % sbd::kTileRT == 0);
-  const sbd::Tiling t = dsb16 ? sbd::make_tiling_dsb16(c->R) : step_tiling(c);
+                     c->groups == 1 && sbd::dsb16_ok(c->Rs) && (int64_t)c->n * c->Rs > sbd::kDsb16Spins &&
+                     !(c->tiled_ok && c->use_tiled && c->Rs % sbd::kTileRT == 0);
+  const sbd::Tiling t = dsb16 ? sbd::make_tiling_dsb16(c->Rs) : step_tiling(c);
   sbd::StepArgs a;
   a.rowptr = c->d_rowptr;
   a.col = c->d_col;
@@ -2018,7 +2043,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   a.dta0 = (float)(dt * a0);
   a.y = c->d_y;
   a.n = c->n;
-  a.R = c->R;
+  a.R = c->Rs;
   a.G = t.G;
   a.unroll = c->step_unroll;
   a.tile0 = 0;
@@ -2040,14 +2065,14 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   a.r1_lanes = r1_lanes_for(c);
   if (dsb16) {
     const int rpc16 = sbd::dsb16_rows_per_cta(a.rpc);
-    if (heavy_first(c, (size_t)c->n * c->R, ((int64_t)c->n + rpc16 - 1) / rpc16)) {
+    if (heavy_first(c, (size_t)c->n * c->Rs, ((int64_t)c->n + rpc16 - 1) / rpc16)) {
       sb_status st2 = ensure_row_order(c, rpc16);
       if (st2) return st2;
       a.cta_order = c->d_row_order;
     }
   }
   const int tiled =
-      (!fac && !streamed && !rw && c->tiled_ok && c->use_tiled && c->R % sbd::kTileRT == 0) ? 1 : 0;
+      (!fac && !streamed && !rw && c->tiled_ok && c->use_tiled && c->Rs % sbd::kTileRT == 0) ? 1 : 0;
   sbd::TiledArgs ta;
   ta.blk_row0 = c->d_blk_row0;
   ta.blk_u0 = c->d_blk_u0;
@@ -2064,15 +2089,15 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   ta.dta0 = a.dta0;
   ta.y = c->d_y;
   ta.n = c->n;
-  ta.R = c->R;
+  ta.R = c->Rs;
   ta.nb = c->nb;
   const int sgn = (variant == SB_DSB && c->dsb_signs && c->j_small && !tiled && !streamed &&
-                   c->R % 4 == 0) ? 1 : 0;
+                   c->Rs % 4 == 0) ? 1 : 0;
   if (sgn && !(c->d_sgn[0] && c->d_sgn[1])) {
     dfree(c->d_sgn[0]);  // a failed earlier attempt may have left one of the pair
     dfree(c->d_sgn[1]);
     sb_status st2;
-    const size_t cnt = (size_t)c->n * c->R;
+    const size_t cnt = (size_t)c->n * c->Rs;
     if ((st2 = dalloc(&c->d_sgn[0], cnt)) || (st2 = dalloc(&c->d_sgn[1], cnt))) return st2;
   }
 
@@ -2086,7 +2111,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     if (!c->l2_persist || !win_max) return cudaSuccess;
     cudaStreamAttrValue v = {};
     v.accessPolicyWindow.base_ptr = const_cast<void*>(base);
-    v.accessPolicyWindow.num_bytes = std::min(win_max, (size_t)c->n * c->R * sizeof(float));
+    v.accessPolicyWindow.num_bytes = std::min(win_max, (size_t)c->n * c->Rs * sizeof(float));
     v.accessPolicyWindow.hitRatio = 1.0f;
     v.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
     v.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
@@ -2110,7 +2135,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     if (fac) {
       fs.xin = xi;
       fs.sgn_in = sgn ? c->d_sgn[cur] : nullptr;
-      if (frw) fs.U = c->d_x[cur] + (size_t)c->n * c->R;
+      if (frw) fs.U = c->d_x[cur] + (size_t)c->n * c->Rs;
       cudaError_t ef = sbd::launch_fac_sum(variant, fs, st);
       if (ef != cudaSuccess || frw) {
         if (ef != cudaSuccess) return ef;
@@ -2151,7 +2176,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     a.xout = xo;
     return sbd::launch_step(variant, c->jbf16, t, a, st);
   };
-  const size_t NR = (size_t)c->n * c->R;
+  const size_t NR = (size_t)c->n * c->Rs;
   sbd::Tiling tg = t;
   if (ngroups > 1) tg.tiles = 1;
   // all steps for replica group g (tiles g), then the next group: each group's
@@ -2182,7 +2207,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
     int32_t a0b = 0, dtb = 0;
     memcpy(&a0b, &a.a0, 4);
     memcpy(&dtb, &a.dt, 4);
-    key = {variant, steps, c->R, c->cur, a0b, dtb, (int64_t)(intptr_t)sched, t.G, tiled, a.rpc,
+    key = {variant, steps, c->Rs, c->cur, a0b, dtb, (int64_t)(intptr_t)sched, t.G, tiled, a.rpc,
            t.tiles, a.unroll, sgn, ngroups, streamed, rw, rw_nch, ra.cta_order != nullptr,
            a.cta_order != nullptr, a.r1_lanes, fac, frw};
   }
@@ -2242,7 +2267,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
     b.R = R;
     b.partial = c->d_partial;
     b.nnz = c->nnz;
-    SB_CUDA(sbd::launch_select_bits(d_spins ? nullptr : c->d_x[c->cur], R, d_spins, c->n, R,
+    SB_CUDA(sbd::launch_select_bits(d_spins ? nullptr : c->d_x[c->cur], c->Rs, d_spins, c->n, R,
                                     c->d_bits, s));
     SB_CUDA(sbd::launch_energy_bits(b, s));
     SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
@@ -2256,6 +2281,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   a.qval = c->d_qval;
   a.qlin = c->d_qlin;
   a.x = d_spins ? nullptr : c->d_x[c->cur];
+  a.xstride = c->Rs;
   a.spins = d_spins;
   a.blk_row = c->d_blk_row;
   a.nblk = c->nblk;
@@ -2586,7 +2612,7 @@ sb_status sb_run(sb_ctx* ctx, sb_variant variant, double a0, double c0, double d
     SB_CUDA(sbd::launch_set_c0(ctx->d_c0ev, ctx->d_c0auto, c0, ctx->E, s));
     ctx->cur = 0;
     SB_CUDA(sbd::launch_init(ctx->d_x[0], ctx->d_y, ctx->d_row_event, ctx->d_ev_row0, ctx->n,
-                             ctx->R, seed, s));
+                             ctx->Rs, seed, s));
     ctx->have_state = true;
     return enqueue_steps(ctx, variant, a0, dt, steps, sched, s);
   });
@@ -2624,8 +2650,17 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     SB_CUDA(cudaDeviceSynchronize());
     ctx->cur = 0;
-    SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
-    SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
+    if (ctx->Rs == replicas) {
+      SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
+      SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
+    } else {  // through the second x buffer, then into the padded rows
+      for (int q = 0; q < 2; ++q) {
+        SB_CUDA(cudaMemcpy(ctx->d_x[1], q ? y : x, bytes, k));
+        SB_CUDA(sbd::launch_repitch(ctx->d_x[1], replicas, q ? ctx->d_y : ctx->d_x[0], ctx->Rs,
+                                    ctx->n, replicas, 0));
+      }
+      SB_CUDA(cudaDeviceSynchronize());
+    }
     ctx->have_state = true;
     return SB_OK;
   });
@@ -2645,8 +2680,17 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
   SB_CUDA(cudaDeviceSynchronize());
   sb_status st = check_wait_flag(ctx);
   if (st) return st;
-  if (x) SB_CUDA(cudaMemcpy(x, ctx->d_x[ctx->cur], bytes, k));
-  if (y) SB_CUDA(cudaMemcpy(y, ctx->d_y, bytes, k));
+  for (int q = 0; q < 2; ++q) {
+    float* const out = q ? y : x;
+    const float* src = q ? ctx->d_y : ctx->d_x[ctx->cur];
+    if (!out) continue;
+    if (ctx->Rs != ctx->R) {  // padded rows: gathered in the other x buffer first
+      float* const tmp = ctx->d_x[ctx->cur ^ 1];
+      SB_CUDA(sbd::launch_repitch(src, ctx->Rs, tmp, ctx->R, ctx->n, ctx->R, 0));
+      src = tmp;
+    }
+    SB_CUDA(cudaMemcpy(out, src, bytes, k));
+  }
   return SB_OK;
 }
 
@@ -2699,7 +2743,7 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
     if (st) return st;
     if (d_T)
       SB_CUDA(sbd::launch_best_T(ctx->d_x[ctx->cur], ctx->d_row_event,
-                                 dr ? d_best_r : ctx->d_bestr, ctx->n, ctx->R, d_T, s));
+                                 dr ? d_best_r : ctx->d_bestr, ctx->n, ctx->Rs, d_T, s));
     if (d_E_all && !dE)
       SB_CUDA(cudaMemcpyAsync(d_E_all, ctx->d_Eall, (size_t)ctx->E * ctx->R * 8,
                               cudaMemcpyDeviceToDevice, s));

@@ -97,18 +97,23 @@ struct Vec<1> {
   __device__ __forceinline__ void st(float* p) const { *p = v[0]; }
 };
 
-// V sign bytes of one chunk as the floats 2^-7 sgn
+// One chunk of a neighbour row as loaded: V positions, or V sign bytes
+// (unpacked to 2^-7 sgn only when used, so a chunk in flight holds one register)
+template <int V, bool SGN>
+struct Gathered {
+  Vec<V> t;
+  __device__ __forceinline__ void ld(const StepArgs& a, size_t off) { t.ldg(a.xin + off); }
+  __device__ __forceinline__ float get(int v) const { return t.v[v]; }
+};
 template <int V>
-__device__ __forceinline__ void ld_signs(const uint8_t* p, float (&out)[V]) {
-  if (V == 4) {
-    const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
-#pragma unroll
-    for (int v = 0; v < V; ++v) out[v] = scaled_sign_of_byte(w, v);
-  } else {
-#pragma unroll
-    for (int v = 0; v < V; ++v) out[v] = scaled_sign_of_byte(__ldg(p + v), 0);
+struct Gathered<V, true> {
+  uint32_t t;
+  __device__ __forceinline__ void ld(const StepArgs& a, size_t off) {
+    t = V == 4 ? __ldg(reinterpret_cast<const uint32_t*>(a.sgn_in + off))
+               : (uint32_t)__ldg(a.sgn_in + off);
   }
-}
+  __device__ __forceinline__ float get(int v) const { return scaled_sign_of_byte(t, v); }
+};
 
 __device__ __forceinline__ float jval(const float* J, int p) { return __ldg(J + p); }
 __device__ __forceinline__ float jval(const __nv_bfloat16* J, int p) {
@@ -123,35 +128,40 @@ __device__ __forceinline__ unsigned group_mask(int G) {
 }
 
 // ---------------------------------------------------------------- SB step
-// One row per group of G threads; the group loads G (col, J) pairs of the row
-// at a time (coalesced) and broadcasts them with shuffles; every thread then
-// gathers its replica chunks of the neighbour rows with 16-byte loads, four
-// neighbours in flight at once.
+// One row per group of G threads; every thread of the group reads the row's
+// (col, J) pairs itself (the group's lanes read the same word, one sector) and
+// gathers its replica chunks of U neighbour rows with 16-byte loads, all U in
+// flight at once, while the next U pairs are on their way. The row's own x, y,
+// h and c0 are asked for before the walk. What bounds a step of a small or
+// middling problem is not bytes but the longest chain: the heaviest row takes
+// degree / U rounds of an L2 latency whatever the other rows do. (Pairs loaded
+// G at a time and broadcast by shuffles, four neighbours in flight, took
+// degree / min(G, 4) rounds of two latencies: 34 us per step for 10,878 rows of
+// at most 105 nonzeros at R = 8, 10 us at R = 64.)
 // MODE: 0 aSB, 1 bSB, 2 dSB gathering x (sgn at use), 3 dSB gathering int8
 // signs, 4 bSB also recording the pre-wall momentum and the wall mask.
-// CTAs per SM the compiler is asked to fit: with two or four chunks per thread
-// the free choice takes 101 / 168 registers (two / one CTA per SM); bounding it
-// gives 80 / 128 registers and three / two CTAs without spills
-template <int NCH>
-struct StepMinBlocks {
-  static constexpr int value = NCH == 2 ? 3 : (NCH == 4 ? 2 : 1);
-};
-template <int V, int NCH, int MODE, typename JT>
-__global__ void __launch_bounds__(kBlock, StepMinBlocks<NCH>::value) k_step(const StepArgs a) {
+// CTAs per SM the compiler is asked to fit (64, 80 or 128 registers)
+constexpr int step_blocks(int V, int NCH, int U) {
+  return V == 1 ? (NCH == 1 ? 4 : 3) : (NCH * U <= 4 ? 3 : 2);
+}
+template <int V, int NCH, int U, int MODE, typename JT>
+__global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const StepArgs a) {
   constexpr int VARIANT = MODE == 3 ? 2 : (MODE == 4 ? 1 : MODE);
   constexpr bool use_sgn = MODE == 3;
   constexpr bool record = MODE == 4;
-  constexpr int U = 4;
   const int G = a.G;
   const int gid = threadIdx.x / G;
   const int g = threadIdx.x - gid * G;
   const int groups = blockDim.x / G;
-  const unsigned mask = group_mask(G);
   const int R = a.R;
   const int C = R / V;
   const int ch0 = (blockIdx.y + a.tile0) * (G * NCH) + g;
   const JT* J = static_cast<const JT*>(a.J);
   const int row_end = min(a.n, (blockIdx.x + 1) * a.rpc);
+  const float pa = a.a0 - __ldg(a.sched + a.k);
+  int chl[NCH];  // chunk to load: a lane past the row's last chunk reads it again, unused
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) chl[j] = min(ch0 + j * G, C - 1);
   // a CTA walks a contiguous chunk of rows, so rows in flight together share
   // neighbour rows in L1; the group count is uniform, so a group leaves whole
   for (int row = blockIdx.x * a.rpc + gid; row < row_end; row += groups) {
@@ -163,86 +173,81 @@ __global__ void __launch_bounds__(kBlock, StepMinBlocks<NCH>::value) k_step(cons
 
   int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
   chk_rows(p0, p1, a.nnz);
-  for (int pb = p0; pb < p1; pb += G) {
-    const int cnt = min(G, p1 - pb);
-    int mc = 0;
-    float mv = 0.f;
-    if (g < cnt) {
-      mc = chk_idx(__ldg(a.col + pb + g), a.n, kChkCol);
-      mv = jval(J, pb + g);
-      if (use_sgn) mv *= kSignScale;  // 2^7 J: sign bytes read as 2^-7 sgn
-    }
-    int q = 0;
-    for (; q + U <= cnt; q += U) {
-      int c[U];
-      float w[U];
+  Vec<V> xo[NCH], yo[NCH];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        c[u] = __shfl_sync(mask, mc, q + u, G);
-        w[u] = __shfl_sync(mask, mv, q + u, G);
-      }
-      float xv[U][NCH][V];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {
-          const int ch = ch0 + j * G;
-          if (ch < C) {
-            const size_t off = (size_t)c[u] * R + (size_t)ch * V;
-            if (use_sgn) {
-              ld_signs<V>(a.sgn_in + off, xv[u][j]);
-            } else {
-              Vec<V> t;
-              t.ldg(a.xin + off);
-#pragma unroll
-              for (int v = 0; v < V; ++v) xv[u][j][v] = VARIANT == 2 ? sgnf(t.v[v]) : t.v[v];
-            }
-          }
-        }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int j = 0; j < NCH; ++j)
-#pragma unroll
-          for (int v = 0; v < V; ++v) acc[j][v] = fmaf(w[u], xv[u][j][v], acc[j][v]);
-    }
-    for (; q < cnt; ++q) {
-      const int c = __shfl_sync(mask, mc, q, G);
-      const float w = __shfl_sync(mask, mv, q, G);
-#pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const int ch = ch0 + j * G;
-        if (ch < C) {
-          const size_t off = (size_t)c * R + (size_t)ch * V;
-          float xs[V];
-          if (use_sgn) {
-            ld_signs<V>(a.sgn_in + off, xs);
-          } else {
-            Vec<V> t;
-            t.ldg(a.xin + off);
-#pragma unroll
-            for (int v = 0; v < V; ++v) xs[v] = VARIANT == 2 ? sgnf(t.v[v]) : t.v[v];
-          }
-#pragma unroll
-          for (int v = 0; v < V; ++v) acc[j][v] = fmaf(w, xs[v], acc[j][v]);
-        }
-      }
-    }
+  for (int j = 0; j < NCH; ++j) {
+    xo[j].ldg(a.xin + (size_t)row * R + (size_t)chl[j] * V);
+    if (ch0 + j * G < C) yo[j].ld(a.y + (size_t)row * R + (size_t)chl[j] * V);
   }
-
-  // symplectic Euler: momentum with the old position, then position, then wall
-  const float pa = a.a0 - __ldg(a.sched + a.k);
   const int e = a.row_event ? __ldg(a.row_event + row) : 0;
   const float c0 = __ldg(a.c0_ev + e);
   const float hi = __ldg(a.h + row);
+
+  int c[U];
+  float w[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    c[u] = 0;
+    w[u] = 0.f;
+    if (p0 + u < p1) {
+      c[u] = chk_idx(__ldg(a.col + p0 + u), a.n, kChkCol);
+      w[u] = jval(J, p0 + u);
+    }
+  }
+  int p = p0;
+  for (; p + U <= p1; p += U) {
+    Gathered<V, use_sgn> xv[U][NCH];
+    float wc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < NCH; ++j) xv[u][j].ld(a, (size_t)c[u] * R + (size_t)chl[j] * V);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      wc[u] = use_sgn ? w[u] * kSignScale : w[u];  // 2^7 J: sign bytes read as 2^-7 sgn
+      if (p + U + u < p1) {
+        c[u] = chk_idx(__ldg(a.col + p + U + u), a.n, kChkCol);
+        w[u] = jval(J, p + U + u);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < NCH; ++j)
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const float xs = xv[u][j].get(v);
+          acc[j][v] = fmaf(wc[u], VARIANT == 2 && !use_sgn ? sgnf(xs) : xs, acc[j][v]);
+        }
+  }
+  if (p < p1) {  // the last 1 .. U - 1 neighbours, also in one batch
+    Gathered<V, use_sgn> xv[U - 1][NCH];
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+#pragma unroll
+      for (int j = 0; j < NCH; ++j)
+        if (p + u < p1) xv[u][j].ld(a, (size_t)c[u] * R + (size_t)chl[j] * V);
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (p + u < p1) {
+        const float wc = use_sgn ? w[u] * kSignScale : w[u];
+#pragma unroll
+        for (int j = 0; j < NCH; ++j)
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            const float xs = xv[u][j].get(v);
+            acc[j][v] = fmaf(wc, VARIANT == 2 && !use_sgn ? sgnf(xs) : xs, acc[j][v]);
+          }
+      }
+  }
+
+  // symplectic Euler: momentum with the old position, then position, then wall
 #pragma unroll
   for (int j = 0; j < NCH; ++j) {
     const int ch = ch0 + j * G;
     if (ch >= C) continue;
     const size_t idx = (size_t)row * R + (size_t)ch * V;
-    Vec<V> xv, yv;
-    xv.ldg(a.xin + idx);
-    yv.ld(a.y + idx);
+    Vec<V> xv = xo[j], yv = yo[j];
     uint32_t sw = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -279,23 +284,49 @@ __global__ void __launch_bounds__(kBlock, StepMinBlocks<NCH>::value) k_step(cons
   }
 }
 
-template <int V, int NCH, int MODE>
-cudaError_t launch_step_t(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
+template <int V, int NCH, int U, int MODE>
+cudaError_t launch_step_u(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
   dim3 grid((a.n + a.rpc - 1) / a.rpc, t.tiles);
   if (jbf16)
-    k_step<V, NCH, MODE, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
+    k_step<V, NCH, U, MODE, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
   else
-    k_step<V, NCH, MODE, float><<<grid, kBlock, 0, s>>>(a);
+    k_step<V, NCH, U, MODE, float><<<grid, kBlock, 0, s>>>(a);
   return cudaGetLastError();
+}
+
+// Neighbours in flight. More shorten the chain of a heavy row and cost
+// resident CTAs; measured with BF16 J, us per step:
+//  one 16-byte chunk per lane, 4 / 8 in flight: 10,878 rows R = 32 7.8 / 6.6,
+//  R = 64 8.2 / 8.4; 39,165 rows R = 16 16.8 / 16.3, R = 64 32.7 / 37.0; 109,775
+//  rows R = 64 62 / 84. So 8 where the lanes (n R / 4) fill at most a third of the
+//  GPU's threads;
+//  two chunks per lane, 2 / 4 in flight: 10,878 rows R = 100 12.9 / 11.4, R = 192
+//  16.2 / 17.1; 109,775 rows R = 100 88 / 105. So 2 from 1.5 M spins on (4 with
+//  sign bytes, which hold a quarter of the registers: 89 / 84).
+template <int V, int NCH, int MODE>
+cudaError_t launch_step_t(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
+  const int64_t spins = (int64_t)a.n * a.R;
+  if constexpr (V == 1) {
+    return launch_step_u<V, NCH, NCH == 4 ? 4 : 8, MODE>(jbf16, t, a, s);
+  } else if constexpr (NCH == 1) {
+    return spins <= 400000 ? launch_step_u<V, NCH, 8, MODE>(jbf16, t, a, s)
+                           : launch_step_u<V, NCH, 4, MODE>(jbf16, t, a, s);
+  } else if constexpr (NCH == 2 && MODE != 3) {
+    return spins >= 1500000 ? launch_step_u<V, NCH, 2, MODE>(jbf16, t, a, s)
+                            : launch_step_u<V, NCH, 4, MODE>(jbf16, t, a, s);
+  } else {
+    return launch_step_u<V, NCH, NCH == 2 ? 4 : 2, MODE>(jbf16, t, a, s);
+  }
 }
 
 template <int V, int NCH, int MODE>
 int blocks_per_sm_t(int jbf16) {
+  constexpr int U = V == 1 ? (NCH == 4 ? 4 : 8) : (NCH == 4 ? 2 : 4);
   int b = 0;
   const cudaError_t e =
-      jbf16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step<V, NCH, MODE, __nv_bfloat16>,
-                                                            kBlock, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step<V, NCH, MODE, float>,
+      jbf16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                  &b, k_step<V, NCH, U, MODE, __nv_bfloat16>, kBlock, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step<V, NCH, U, MODE, float>,
                                                             kBlock, 0);
   return e == cudaSuccess && b > 0 ? b : 1;
 }
@@ -442,27 +473,33 @@ __global__ void __launch_bounds__(kBlock) k_step_r1g(const StepArgs a) {
 // ---------------------------------------------------------------- dSB, 16 signs per lane
 // dSB gathering int8 signs with 16 replicas per lane: one 16-byte load brings a
 // neighbour's signs for 16 replicas. G = R / 16 lanes own a row (R / 16 a power
-// of two, <= 32). Same CSR-order FMA sequence per replica as k_step.
+// of two, <= 32). Same CSR-order FMA sequence per replica as k_step, and the
+// same walk: each lane reads the (col, J) pairs itself, four neighbours in
+// flight without a predicate, the next four pairs on their way. Pairs loaded G
+// at a time and broadcast by shuffles left G = 1 .. 4 with as many neighbours in
+// flight: us per step before / now, 39,165 rows R = 16 81 / 21, R = 64 37 / 24.5,
+// R = 128 40.5 / 36; 67,445 rows R = 64 24.8 / 20.8; 109,775 rows R = 256 equal.
 
 #ifndef SB_DSB_BLOCK
 #define SB_DSB_BLOCK 128
 #endif
-// nine CTAs of 128 threads per SM: 56 registers, no spills (measured faster
-// than the unbounded 72 registers, seven CTAs; ten CTAs spill)
+// eight CTAs of 128 threads per SM: 64 registers, no spills (nine spill and take
+// twice the time, ten 42 registers 1.1 to 1.9 times)
 #ifndef SB_DSB_MINB
-#define SB_DSB_MINB 9
+#define SB_DSB_MINB 8
 #endif
 constexpr int kDsbBlock = SB_DSB_BLOCK;  // threads per CTA of k_step_dsb16
 
 template <typename JT>
 __global__ void __launch_bounds__(kDsbBlock, SB_DSB_MINB) k_step_dsb16(const StepArgs a) {
+  constexpr int U = 4;
   const int G = a.G;
   const int gid = threadIdx.x / G;
   const int g = threadIdx.x - gid * G;
   const int groups = blockDim.x / G;
-  const unsigned mask = group_mask(G);
   const int R = a.R;
   const JT* J = static_cast<const JT*>(a.J);
+  const uint8_t* sg = a.sgn_in + 16 * g;
   const int chunk = a.cta_order ? __ldg(a.cta_order + blockIdx.x) : (int)blockIdx.x;
   const int row_end = min(a.n, (chunk + 1) * a.rpc);
   for (int row = chunk * a.rpc + gid; row < row_end; row += groups) {
@@ -471,44 +508,53 @@ __global__ void __launch_bounds__(kDsbBlock, SB_DSB_MINB) k_step_dsb16(const Ste
     for (int v = 0; v < 16; ++v) acc[v] = 0.f;
     int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
     chk_rows(p0, p1, a.nnz);
-    for (int pb = p0; pb < p1; pb += G) {
-      const int cnt = min(G, p1 - pb);
-      int mc = 0;
-      float mv = 0.f;
-      if (g < cnt) {
-        mc = chk_idx(__ldg(a.col + pb + g), a.n, kChkCol);
-        mv = jval(J, pb + g);
-        mv *= kSignScale;  // 2^7 J: sign bytes read as 2^-7 sgn
+    int c[U];
+    float w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      c[u] = 0;
+      w[u] = 0.f;
+      if (p0 + u < p1) {
+        c[u] = chk_idx(__ldg(a.col + p0 + u), a.n, kChkCol);
+        w[u] = jval(J, p0 + u);
       }
-      int q = 0;
-      for (; q + 4 <= cnt; q += 4) {
-        int c[4];
-        float w[4];
-        uint4 sv[4];
+    }
+    int p = p0;
+    for (; p + U <= p1; p += U) {
+      uint4 sv[U];
+      float wc[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          c[u] = __shfl_sync(mask, mc, q + u, G);
-          w[u] = __shfl_sync(mask, mv, q + u, G);
+      for (int u = 0; u < U; ++u) sv[u] = __ldg(reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R));
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        wc[u] = w[u] * kSignScale;  // 2^7 J: sign bytes read as 2^-7 sgn
+        if (p + U + u < p1) {
+          c[u] = chk_idx(__ldg(a.col + p + U + u), a.n, kChkCol);
+          w[u] = jval(J, p + U + u);
         }
+      }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          sv[u] = __ldg(reinterpret_cast<const uint4*>(a.sgn_in + (size_t)c[u] * R + 16 * g));
+      for (int u = 0; u < U; ++u) {
+        const unsigned ww[4] = {sv[u].x, sv[u].y, sv[u].z, sv[u].w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int v = 0; v < 16; ++v)
+          acc[v] = fmaf(wc[u], scaled_sign_of_byte(ww[v >> 2], v & 3), acc[v]);
+      }
+    }
+    if (p < p1) {
+      uint4 sv[U - 1];
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (p + u < p1) sv[u] = __ldg(reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R));
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (p + u < p1) {
+          const float wc = w[u] * kSignScale;
           const unsigned ww[4] = {sv[u].x, sv[u].y, sv[u].z, sv[u].w};
 #pragma unroll
           for (int v = 0; v < 16; ++v)
-            acc[v] = fmaf(w[u], scaled_sign_of_byte(ww[v >> 2], v & 3), acc[v]);
+            acc[v] = fmaf(wc, scaled_sign_of_byte(ww[v >> 2], v & 3), acc[v]);
         }
-      }
-      for (; q < cnt; ++q) {
-        const int c = __shfl_sync(mask, mc, q, G);
-        const float w = __shfl_sync(mask, mv, q, G);
-        const uint4 s4 = __ldg(reinterpret_cast<const uint4*>(a.sgn_in + (size_t)c * R + 16 * g));
-        const unsigned ww[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-        for (int v = 0; v < 16; ++v) acc[v] = fmaf(w, scaled_sign_of_byte(ww[v >> 2], v & 3), acc[v]);
-      }
     }
     const float pa = a.a0 - __ldg(a.sched + a.k);
     const int e = a.row_event ? __ldg(a.row_event + row) : 0;
@@ -1136,7 +1182,7 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
   const int g = threadIdx.x - gid * G;
   const int groups = blockDim.x / G;
   const unsigned mask = group_mask(G);
-  const int R = a.R;
+  const int R = a.R, XS = a.x && a.xstride ? a.xstride : a.R;
   const int C = R / V;
   const int tile_base = blockIdx.y * (G * NCH);
   const int ch0 = tile_base + g;
@@ -1171,7 +1217,7 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
           const int ch = ch0 + j * G;
           if (ch < C) {
             double t[V];
-            load_T<V>(a, (size_t)c * R + (size_t)ch * V, t);
+            load_T<V>(a, (size_t)c * XS + (size_t)ch * V, t);
 #pragma unroll
             for (int v = 0; v < V; ++v) inner[j][v] += w * t[v];
           }
@@ -1184,7 +1230,7 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
       const int ch = ch0 + j * G;
       if (ch < C) {
         double t[V];
-        load_T<V>(a, (size_t)row * R + (size_t)ch * V, t);
+        load_T<V>(a, (size_t)row * XS + (size_t)ch * V, t);
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[j][v] += t[v] * (ai + 0.5 * inner[j][v]);
       }
@@ -1531,6 +1577,24 @@ __global__ void k_signs(const float* x, uint8_t* s, size_t count) {
 cudaError_t launch_signs(const float* x, uint8_t* s, size_t count, cudaStream_t st) {
   if (!count) return cudaSuccess;
   k_signs<<<grid_for(count, kBlock), kBlock, 0, st>>>(x, s, count);
+  return cudaGetLastError();
+}
+
+__global__ void k_repitch(const float* in, int32_t ipitch, float* out, int32_t opitch, int32_t n,
+                          int32_t cols) {
+  const size_t total = (size_t)n * opitch, step = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
+    const size_t row = i / opitch;
+    const int r = (int)(i - row * opitch);
+    out[i] = r < cols ? in[row * ipitch + r] : 0.f;
+  }
+}
+
+cudaError_t launch_repitch(const float* in, int32_t ipitch, float* out, int32_t opitch, int32_t n,
+                           int32_t cols, cudaStream_t s) {
+  const size_t total = (size_t)n * opitch;
+  if (!total) return cudaSuccess;
+  k_repitch<<<grid_for(total, kBlock), kBlock, 0, s>>>(in, ipitch, out, opitch, n, cols);
   return cudaGetLastError();
 }
 

@@ -23,6 +23,12 @@ Tiling make_tiling(int R);
 Tiling make_tiling_rt(int R, int RT);
 // dSB with int8 signs, 16 replicas per lane: valid when R / 16 is a power of two <= 32.
 bool dsb16_ok(int R);
+// Above this many spins dSB takes that kernel, below it k_step with sign bytes
+// (4 replicas per lane: four times the lanes, a quarter of the bytes per load).
+// us per step, 16 per lane / 4 per lane: 39,165 rows R = 32 (1.25 M spins) 23.5 /
+// 18.8, R = 64 (2.5 M) 24.5 / 29.1; 67,445 rows R = 32 (2.2 M) 14.0 / 13.9, R = 64
+// (4.3 M) 20.8 / 22.5; 10,878 rows R = 64 (0.7 M) 13.0 / 7.9, R = 512 (5.6 M) 25 / 30.
+constexpr int64_t kDsb16Spins = 2400000;
 // rows per CTA of k_step_dsb16 for a step's rows-per-CTA setting rpc
 int dsb16_rows_per_cta(int rpc);
 Tiling make_tiling_dsb16(int R);
@@ -96,6 +102,10 @@ cudaError_t launch_init(float* x, float* y, const int32_t* row_event, const int3
                         int32_t n, int32_t R, uint64_t seed, cudaStream_t s);
 // s[i] = sign byte of x[i]: 0x3C, 0xBC, 0x00 for x > 0, x < 0, x = 0 (signs.cuh)
 cudaError_t launch_signs(const float* x, uint8_t* s, size_t count, cudaStream_t st);
+// out rows (opitch floats apart) = in rows (ipitch apart), cols values each; the
+// rest of a longer out row is zeroed
+cudaError_t launch_repitch(const float* in, int32_t ipitch, float* out, int32_t opitch, int32_t n,
+                           int32_t cols, cudaStream_t s);
 // blocks of the untiled step kernel resident per SM for this tiling and unroll
 int step_blocks_per_sm(int variant, int jbf16, const Tiling& t, int unroll);
 
@@ -122,7 +132,8 @@ struct EnergyArgs {
   const double* qval;
   const double* qlin;
   const float* x;          // state positions (T = x > 0), or NULL when spins given
-  const int8_t* spins;     // +1 selects; used when x == NULL
+  const int8_t* spins;     // +1 selects; used when x == NULL; [n x R]
+  int32_t xstride = 0;     // floats between rows of x (0: R)
   const int32_t* blk_row;  // row range of each partial block [nblk + 1]
   int32_t nblk;
   int32_t n, R, G;
