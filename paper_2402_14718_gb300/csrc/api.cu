@@ -218,7 +218,13 @@ struct sb_ctx {
   int32_t* d_f_gmem = nullptr;
   int32_t* d_f_gout = nullptr;
   int4* d_f_item = nullptr;     // group-sum work items (block, member range, scratch slot)
-  int4* d_f_item1 = nullptr;    // the same with one item per block (the dSB form)
+  // dSB: blocks (block, member words, 0), member words, and the blocks of each
+  // CTA for the lane groups of the current replica count (ensure_fac_ctas)
+  int4* d_f_item1 = nullptr;
+  uint4* d_f_gword = nullptr;
+  int2* d_f_cta = nullptr;
+  int32_t f_cta_per = 0, f_nctas = 0;
+  std::vector<int32_t> h_f_cnt, h_f_ev;  // members and event of each block
   int32_t* d_f_gnc = nullptr;   // chunks per block
   int32_t* d_f_gscr0 = nullptr; // first scratch slot per block (-1: one chunk)
   int32_t fac_nitems = 0, fac_nslots = 0;
@@ -429,6 +435,13 @@ void free_factor(sb_ctx* c) {
   c->d_f_item = nullptr;
   if (c->d_f_item1) cudaFree(c->d_f_item1);
   c->d_f_item1 = nullptr;
+  if (c->d_f_gword) cudaFree(c->d_f_gword);
+  c->d_f_gword = nullptr;
+  if (c->d_f_cta) cudaFree(c->d_f_cta);
+  c->d_f_cta = nullptr;
+  c->f_cta_per = c->f_nctas = 0;
+  std::vector<int32_t>().swap(c->h_f_cnt);
+  std::vector<int32_t>().swap(c->h_f_ev);
   dfree(c->d_f_gnc);
   dfree(c->d_f_gscr0);
   dfree(c->d_f_cnt);
@@ -1532,14 +1545,26 @@ sb_status set_factor(sb_ctx* c, int32_t n_ids, int32_t K, const int32_t* member,
   // work items of the group sums. aSB / bSB (one block per warp): blocks of
   // more than kChunk members are cut into near-equal chunks (a warp walks its
   // members one after another, so the largest block would otherwise set the
-  // kernel's time). dSB (eight blocks per warp, advancing together): whole
-  // blocks (measured faster there: the chunk sums' fences cost more than the
-  // split saves).
+  // kernel's time). dSB: whole blocks, their members in words of four (row and
+  // slot), the large ones spread over a CTA (ensure_fac_ctas).
   constexpr int64_t kChunk = 16;
   std::vector<int4> items, items1;
+  std::vector<uint32_t> gword;
+  std::vector<int32_t> bcnt((size_t)ng), bev((size_t)ng, 0);
   items1.reserve((size_t)ng);
-  for (int32_t ga = 0; ga < ng; ++ga)
-    items1.push_back(make_int4(ga, gseg[(size_t)ga * K], gseg[(size_t)ga * K + K], -1));
+  gword.reserve(gmem.size() + (size_t)ng * 2);
+  for (int32_t ga = 0; ga < ng; ++ga) {
+    const int32_t w0 = (int32_t)(gword.size() / 4);
+    for (int s = 0; s < K; ++s)
+      for (int32_t t = gseg[(size_t)ga * K + s]; t < gseg[(size_t)ga * K + s + 1]; ++t)
+        gword.push_back((uint32_t)gmem[t] | (uint32_t)s << 28);
+    while (gword.size() % 4) gword.push_back(sbd::kFacPad);
+    items1.push_back(make_int4(ga, w0, (int32_t)(gword.size() / 4), 0));
+    bcnt[ga] = gseg[(size_t)ga * K + K] - gseg[(size_t)ga * K];
+    if (c->E > 1 && bcnt[ga] > 0)
+      bev[ga] = (int32_t)(std::upper_bound(c->ev_row0.begin(), c->ev_row0.end(),
+                                           gmem[gseg[(size_t)ga * K]]) - c->ev_row0.begin()) - 1;
+  }
   std::vector<int32_t> gnc(ng), gscr0(ng, -1);
   int32_t nslots = 0;
   for (int32_t ga = 0; ga < ng; ++ga) {
@@ -1603,6 +1628,7 @@ sb_status set_factor(sb_ctx* c, int32_t n_ids, int32_t K, const int32_t* member,
   if ((st = raw_alloc(&c->d_f_rJ, std::max<int64_t>(rnnz, 1) * esz)) ||
       (st = raw_alloc(reinterpret_cast<void**>(&c->d_f_item), std::max<size_t>(items.size(), 1) * sizeof(int4))) ||
       (st = raw_alloc(reinterpret_cast<void**>(&c->d_f_item1), std::max<size_t>(items1.size(), 1) * sizeof(int4))) ||
+      (st = raw_alloc(reinterpret_cast<void**>(&c->d_f_gword), std::max<size_t>(gword.size(), 4) * 4)) ||
       (st = raw_alloc(reinterpret_cast<void**>(&c->d_f_head),
                       std::max<size_t>((size_t)n * sbd::fac_head_words((int)esz) * 4, 16))))
     return st;
@@ -1615,6 +1641,10 @@ sb_status set_factor(sb_ctx* c, int32_t n_ids, int32_t K, const int32_t* member,
     SB_CUDA(cudaMemcpy(c->d_f_item, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
   if (!items1.empty())
     SB_CUDA(cudaMemcpy(c->d_f_item1, items1.data(), items1.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  if (!gword.empty())
+    SB_CUDA(cudaMemcpy(c->d_f_gword, gword.data(), gword.size() * 4, cudaMemcpyHostToDevice));
+  c->h_f_cnt.swap(bcnt);
+  c->h_f_ev.swap(bev);
   if (ng) {
     SB_CUDA(cudaMemcpy(c->d_f_gnc, gnc.data(), gnc.size() * 4, cudaMemcpyHostToDevice));
     SB_CUDA(cudaMemcpy(c->d_f_gscr0, gscr0.data(), gscr0.size() * 4, cudaMemcpyHostToDevice));
@@ -1761,6 +1791,44 @@ sb_status ensure_frw(sb_ctx* c, int RW) {
   return SB_OK;
 }
 
+// dSB group sums: which blocks each CTA takes when a CTA has `per` lane groups.
+// Blocks come by event, largest first; those of more than kFacBig members take a
+// CTA each, the others `per` to a CTA (never across events, whose sign bytes
+// would not share L2).
+sb_status ensure_fac_ctas(sb_ctx* c, int per) {
+  if (c->f_cta_per == per && c->d_f_cta) return SB_OK;
+  std::vector<int2> t;
+  const int32_t ng = c->fac_ng;
+  for (int32_t b = 0; b < ng;) {
+    if (c->h_f_cnt[b] > sbd::kFacBig && per > 1) {
+      t.push_back(make_int2(b, 0));
+      ++b;
+      continue;
+    }
+    int32_t e = b + 1;
+    while (e < ng && e - b < per && c->h_f_ev[e] == c->h_f_ev[b] &&
+           !(c->h_f_cnt[e] > sbd::kFacBig && per > 1))
+      ++e;
+    t.push_back(make_int2(b, e - b));
+    b = e;
+  }
+  if (c->d_f_cta) cudaFree(c->d_f_cta);
+  c->d_f_cta = nullptr;
+  c->f_cta_per = 0;
+  c->graph.reset();
+  cudaError_t e = cudaMalloc(&c->d_f_cta, std::max<size_t>(t.size(), 1) * sizeof(int2));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    c->d_f_cta = nullptr;
+    set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    return SB_ERR_OOM;
+  }
+  if (!t.empty()) SB_CUDA(cudaMemcpy(c->d_f_cta, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  c->f_cta_per = per;
+  c->f_nctas = (int32_t)t.size();
+  return SB_OK;
+}
+
 // Grow both x buffers to `rows` rows of the current replica count, keeping
 // the n state rows.
 sb_status ensure_x_rows(sb_ctx* c, int64_t rows) {
@@ -1885,8 +1953,15 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
       c->f_scr_count = scr_need;
       c->graph.reset();
     }
+    if (variant == SB_DSB) {
+      sb_status st0 = ensure_fac_ctas(c, sbd::kFacThreads / fG);
+      if (st0) return st0;
+    }
     fs.item = variant == SB_DSB ? c->d_f_item1 : c->d_f_item;
     fs.nitems = variant == SB_DSB ? c->fac_ng : c->fac_nitems;
+    fs.gword = c->d_f_gword;
+    fs.cta = c->d_f_cta;
+    fs.nctas = c->f_nctas;
     fs.gnc = c->d_f_gnc;
     fs.gscr0 = c->d_f_gscr0;
     fs.cnt = c->d_f_cnt;

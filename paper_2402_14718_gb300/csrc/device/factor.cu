@@ -41,7 +41,7 @@
 namespace sbd {
 namespace {
 
-constexpr int kFacBlock = 128;
+constexpr int kFacBlock = kFacThreads;
 // dSB: replicas per lane (measured on the 512-event batch against 16 per lane,
 // and against requesting the U rows and own x, y before the residual walk:
 // both cost occupancy and were slower)
@@ -105,19 +105,6 @@ struct Chunk<0, NCH> {
     }
   }
 };
-template <int NCH>
-struct Chunk<1, NCH> {
-  static constexpr int P = kSgnPer;
-  Words<P / 4> t;
-  __device__ __forceinline__ void load(const FacSumArgs& a, size_t off, int, int row) {
-    t.ldg(a.sgn_in + (size_t)row * a.R + off);
-  }
-  __device__ __forceinline__ void add_to(float (&u)[P]) const {
-#pragma unroll
-    for (int k = 0; k < P; ++k) u[k] += scaled_sign_of_byte(t.w[k >> 2], k & 3);
-  }
-};
-
 // Adds a member in slot s2 to every U_s it couples to (s2 is the same for the
 // whole lane group, so the branches do not diverge inside it).
 template <int K, typename CH>
@@ -172,23 +159,117 @@ __device__ __forceinline__ size_t scr_index(const FacSumArgs& a, int c, int s, s
   return MODE == 0 ? base + 4 * G * (v >> 2) + (v & 3) : base + v;
 }
 
-// residency bounds (CTAs of 128 threads per SM). dSB, measured on the
-// 512-event batch: 12 for the row step (40 registers) and 10 for the group
-// sums (48) beat the compiler's unbounded 48 / 64 registers (1.92 against
-// 2.03 ms per step). The FP32 forms: the bounds that give the compiler's own
-// unbounded register counts (about 48 / 56 registers with one 16-byte chunk per
+// residency bounds (CTAs of 128 threads per SM) of the FP32 forms: the bounds
+// that give the compiler's own unbounded register counts (about 48 / 56 registers with one 16-byte chunk per
 // lane, 64 / 72 with two).
 template <int MODE, int NCH>
 struct FacMinBlocks {
   static constexpr int sum = NCH == 2 ? 7 : 9, step = NCH == 2 ? 8 : 9;
 };
-#ifndef SB_FAC_DSB_STEP_MINB
-#define SB_FAC_DSB_STEP_MINB 12
-#endif
-template <int NCH>
-struct FacMinBlocks<1, NCH> {
-  static constexpr int sum = 10, step = SB_FAC_DSB_STEP_MINB;
-};
+
+// ---------------------------------------------------------------- dSB group sums
+// Lane l of a G-lane group holds the replicas tile0 + 8 l .. + 7 (one 8-byte
+// load per member). Members come four to a 16-byte word, so a lane reads its
+// words itself and has eight members' signs in flight with the next words on
+// their way, whatever G is; padding reads row 0 and couples to nothing, so no load has
+// a predicate. All sums are whole numbers of 2^-7 below 2^24, exact in FP32 in
+// any order: a block of more than kFacBig members is spread over a CTA's lane
+// groups and added up by shuffles and through shared memory, so that the
+// largest block (178 members on the 512-event batch) does not set the time.
+// Per-block chains of four members at two latencies each took 14.3 of the 21 us
+// of a step of 10,878 rows at R = 64; whole steps before / now with the row
+// step below: 10,878 rows R = 16 35 / 8.7, R = 64 21.4 / 9.4; 39,165 rows R = 16 53
+// / 11, R = 64 35 / 16.4, R = 256 63 / 46; 64 events (616,640 rows) R = 64 260 / 219
+// early and 240 / 197 late in the run; 472,812 rows R = 128 341 / 303 and 317 / 280.
+// Seven CTAs per SM (72 registers); eight spill.
+template <bool UF32, int K>
+__global__ void __launch_bounds__(kFacBlock, 7) k_fac_sum_sgn(const FacSumArgs a) {
+  constexpr int P = kSgnPer;
+  __shared__ float part[kFacBlock / 32][K * P][33];
+  const int G = a.G;
+  const int gq = threadIdx.x / G;
+  const int l = threadIdx.x - gq * G;
+  const int per = kFacBlock / G;
+  const int2 cta = __ldg(a.cta + blockIdx.x);
+  const bool big = cta.y == 0;
+  if (!big && gq >= cta.y) return;  // the whole lane group leaves together
+  const size_t off = (size_t)blockIdx.y * (kSgnPer * G) + kSgnPer * l;
+  const uint8_t* const sg = a.sgn_in + off;
+  const int R = a.R;
+  const int4 item = __ldg(a.item + cta.x + (big ? 0 : gq));
+  const int step = big ? per : 1;
+  float U[K][P];
+#pragma unroll
+  for (int s = 0; s < K; ++s)
+#pragma unroll
+    for (int v = 0; v < P; ++v) U[s][v] = 0.f;
+  const uint4 pad = make_uint4(kFacPad, kFacPad, kFacPad, kFacPad);
+  int w = item.y + (big ? gq : 0);
+  uint4 m0 = w < item.z ? __ldg(a.gword + w) : pad;
+  uint4 m1 = w + step < item.z ? __ldg(a.gword + w + step) : pad;
+  while (w < item.z) {
+    const uint32_t m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+    const bool two = w + step < item.z;
+    uint2 v[8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      v[u] = __ldg(reinterpret_cast<const uint2*>(
+          sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R));
+    if (two) {
+#pragma unroll
+      for (int u = 4; u < 8; ++u)
+        v[u] = __ldg(reinterpret_cast<const uint2*>(
+            sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R));
+    }
+    w += 2 * step;
+    m0 = w < item.z ? __ldg(a.gword + w) : pad;
+    m1 = w + step < item.z ? __ldg(a.gword + w + step) : pad;
+    auto add = [&](uint32_t mw, const uint2& sv) {
+      const uint32_t cs = a.couple >> (4 * (mw >> 28));  // W is symmetric: bit s of slot s2's nibble
+      const uint32_t ww[2] = {sv.x, sv.y};
+      float f[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) f[k] = scaled_sign_of_byte(ww[k >> 2], k & 3);
+#pragma unroll
+      for (int s = 0; s < K; ++s)
+        if ((cs >> s) & 1u) {
+#pragma unroll
+          for (int k = 0; k < P; ++k) U[s][k] += f[k];
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < 4; ++u) add(m[u], v[u]);
+    if (two) {
+#pragma unroll
+      for (int u = 4; u < 8; ++u) add(m[u], v[u]);
+    }
+  }
+  if (big) {
+    for (int o = G; o < 32; o <<= 1)
+#pragma unroll
+      for (int s = 0; s < K; ++s)
+#pragma unroll
+        for (int k = 0; k < P; ++k) U[s][k] += __shfl_xor_sync(0xffffffffu, U[s][k], o);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane < G)
+#pragma unroll
+      for (int s = 0; s < K; ++s)
+#pragma unroll
+        for (int k = 0; k < P; ++k) part[wid][s * P + k][lane] = U[s][k];
+    __syncthreads();
+    if (gq != 0) return;
+#pragma unroll
+    for (int s = 0; s < K; ++s)
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < kFacBlock / 32; ++q) t += part[q][s * P + k][l];
+        U[s][k] = t;
+      }
+  }
+  store_u<1, UF32 ? 2 : 1, K, P>(a, item.x, off, G, U);
+}
 
 template <int MODE, int NCH, int K>
 __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_fac_sum(const FacSumArgs a) {
@@ -562,6 +643,158 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   if (MODE == 1) sw.st(a.sgn_out + idx);
 }
 
+// ---------------------------------------------------------------- dSB row step
+// One row per G-lane group, 8 replicas per lane. The row head holds the first
+// eight residual entries and the U rows in one line: each lane reads it with
+// four 16-byte loads (no shuffles), then has all of the head's neighbours (zero
+// weights pad them, so no load has a predicate) and the U rows in flight at once;
+// longer residual rows follow four neighbours at a time, the U rows after the
+// head's neighbours (together with them the registers spill at this residency).
+// Bound by latency and issue. Ten CTAs per SM (48 registers); with eight (64,
+// U rows first) the 64-event batch takes 216 us a step late in the run, with
+// twelve (spills) 218, with ten 197; requesting the own x and y first took 216.
+template <bool UF32, int K, typename JT>
+__global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArgs a) {
+  constexpr int P = kSgnPer;
+  constexpr int NCH = UF32 ? 2 : 1;
+  const int G = a.G;
+  const int gq = threadIdx.x / G;
+  const int l = threadIdx.x - gq * G;
+  const int row = blockIdx.x * (kFacBlock / G) + gq;
+  if (row >= a.n) return;
+  const int R = a.R;
+  const size_t off = (size_t)blockIdx.y * (kSgnPer * G) + kSgnPer * l;
+  const size_t idx = (size_t)row * R + off;
+  constexpr int HW = fac_head_words(sizeof(JT));
+  const uint4* const hd = reinterpret_cast<const uint4*>(a.head + (size_t)row * HW);
+  const uint4 hc0 = __ldg(hd), hc1 = __ldg(hd + 1), hu = __ldg(hd + 2), hj0 = __ldg(hd + 3);
+  uint4 hj1 = make_uint4(0u, 0u, 0u, 0u);
+  if (sizeof(JT) == 4) hj1 = __ldg(hd + 4);
+  int p0 = __ldg(a.rrowptr + row), p1 = __ldg(a.rrowptr + row + 1);
+  const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
+  const float hi = __ldg(a.h + row);
+  chk_rows(p0, p1, a.rnnz);
+  prefetch_l2(a.xin + idx);
+  prefetch_l2(a.y + idx);
+  const uint8_t* const sg = a.sgn_in + off;
+  const int L = p1 - p0;
+  auto gather = [&](uint32_t c) {
+    return __ldg(reinterpret_cast<const uint2*>(sg + (size_t)chk_idx((int)c, a.n, kChkCol) * R));
+  };
+  uint2 s0[4], s1[4];
+  const uint32_t ca[4] = {hc0.x, hc0.y, hc0.z, hc0.w}, cb[4] = {hc1.x, hc1.y, hc1.z, hc1.w};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) s0[u] = gather(ca[u]);
+  if (L > 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s1[u] = gather(cb[u]);
+  }
+  const uint32_t uw[4] = {hu.x, hu.y, hu.z, hu.w};
+  const float c0 = __ldg(a.c0_ev + ev);
+  const float pa = a.a0 - __ldg(a.sched + a.k);
+
+  // residual row in column order: weights scaled by 2^7, sign bytes read as 2^-7 sgn
+  float acc[P];
+#pragma unroll
+  for (int v = 0; v < P; ++v) acc[v] = 0.f;
+  auto take = [&](float w, const uint2& sv) {
+    const uint32_t ww[2] = {sv.x, sv.y};
+#pragma unroll
+    for (int v = 0; v < P; ++v) acc[v] = fmaf(w, scaled_sign_of_byte(ww[v >> 2], v & 3), acc[v]);
+  };
+  auto weight = [&](const uint4& lo, const uint4& hi4, int t) {  // head weight t, times 2^7
+    if (sizeof(JT) == 4) {
+      const uint32_t q[8] = {lo.x, lo.y, lo.z, lo.w, hi4.x, hi4.y, hi4.z, hi4.w};
+      return __uint_as_float(q[t]) * kSignScale;
+    }
+    const uint32_t q[4] = {lo.x, lo.y, lo.z, lo.w};
+    const uint32_t wd = q[t >> 1];
+    return __uint_as_float(t & 1 ? wd & 0xffff0000u : wd << 16) * kSignScale;
+  };
+#pragma unroll
+  for (int u = 0; u < 4; ++u) take(weight(hj0, hj1, u), s0[u]);
+  if (L > 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) take(weight(hj0, hj1, 4 + u), s1[u]);
+  }
+  URow<1, NCH> ur[K];
+#pragma unroll
+  for (int s = 0; s < K; ++s)
+    if ((int)uw[s] >= 0)
+      ur[s].load(a.U, (size_t)chk_idx((int)uw[s], a.urows, kChkURow) * R + off, G);
+  if (L > kFacHead) {
+    const JT* J = static_cast<const JT*>(a.rJ);
+    int p = p0 + kFacHead;
+    for (; p + 4 <= p1; p += 4) {
+      uint2 sv[4];
+      float w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sv[u] = gather((uint32_t)__ldg(a.rcol + p + u));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] = jv(J, p + u) * kSignScale;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) take(w[u], sv[u]);
+    }
+    if (p < p1) {
+      uint2 sv[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (p + u < p1) sv[u] = gather((uint32_t)__ldg(a.rcol + p + u));
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (p + u < p1) take(jv(J, p + u) * kSignScale, sv[u]);
+    }
+  }
+  // the factored part: U holds sums of 2^-7 sgn, so the scale is 2^7 jf (exact)
+  bool any = false;
+  float fu[P];
+#pragma unroll
+  for (int v = 0; v < P; ++v) fu[v] = 0.f;
+#pragma unroll
+  for (int s = 0; s < K; ++s)
+    if ((int)uw[s] >= 0) {
+      any = true;
+      ur[s].add_to(fu);
+    }
+  if (any) {
+    const float jf = a.jf * kSignScale;
+#pragma unroll
+    for (int v = 0; v < P; ++v) acc[v] = fmaf(jf, fu[v], acc[v]);
+  }
+
+  // symplectic Euler: momentum with the old position, then position, then wall
+  Words<2> sw;  // the new sign bytes
+  sw.w[0] = sw.w[1] = 0u;
+  const bool inplace = a.xout == a.xin;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const size_t o = idx + 4 * j;
+    const float4 xq = *reinterpret_cast<const float4*>(a.xin + o);
+    const float4 yq = *reinterpret_cast<const float4*>(a.y + o);
+    float xs[4] = {xq.x, xq.y, xq.z, xq.w}, ys[4] = {yq.x, yq.y, yq.z, yq.w};
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      float x = xs[v], y = ys[v];
+      const float force = -pa * x + c0 * (acc[4 * j + v] + hi);
+      y = y + a.dt * force;
+      x = x + a.dta0 * y;
+      if (fabsf(x) > 1.f) {
+        x = copysignf(1.f, x);
+        y = 0.f;
+      }
+      xs[v] = x;
+      ys[v] = y;
+      sw.w[j] |= sign_byte(x) << (8 * v);
+    }
+    // a spin that stays on the wall keeps x = +-1, y = 0: nothing to write back
+    const float4 xn = make_float4(xs[0], xs[1], xs[2], xs[3]);
+    const float4 yn = make_float4(ys[0], ys[1], ys[2], ys[3]);
+    if (!inplace || bits_differ(xq, xn)) *reinterpret_cast<float4*>(a.xout + o) = xn;
+    if (bits_differ(yq, yn)) *reinterpret_cast<float4*>(a.y + o) = yn;
+  }
+  sw.st(a.sgn_out + idx);
+}
+
 template <int MODE, int NCH, int K>
 cudaError_t launch_sum_k(const FacSumArgs& a, cudaStream_t s) {
   if (a.nitems <= 0) return cudaSuccess;
@@ -601,9 +834,37 @@ cudaError_t launch_step_n(const FacStepArgs& a, cudaStream_t s) {
   }
 }
 
+template <bool UF32>
+cudaError_t launch_sum_sgn(const FacSumArgs& a, cudaStream_t s) {
+  if (a.nctas <= 0) return cudaSuccess;
+  dim3 grid(a.nctas, a.tiles);
+  switch (a.K) {
+    case 1: k_fac_sum_sgn<UF32, 1><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 2: k_fac_sum_sgn<UF32, 2><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 3: k_fac_sum_sgn<UF32, 3><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 4: k_fac_sum_sgn<UF32, 4><<<grid, kFacBlock, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+template <bool UF32, typename JT>
+cudaError_t launch_step_sgn(const FacStepArgs& a, cudaStream_t s) {
+  const int per = kFacBlock / a.G;
+  dim3 grid((a.n + per - 1) / per, a.tiles);
+  switch (a.K) {
+    case 1: k_step_fac_sgn<UF32, 1, JT><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 2: k_step_fac_sgn<UF32, 2, JT><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 3: k_step_fac_sgn<UF32, 3, JT><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 4: k_step_fac_sgn<UF32, 4, JT><<<grid, kFacBlock, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
 template <typename JT>
 cudaError_t launch_step_j(int variant, const FacStepArgs& a, cudaStream_t s) {
-  if (variant == 2) return a.NCH == 2 ? launch_step_n<2, 1, 2, JT>(a, s) : launch_step_n<2, 1, 1, JT>(a, s);
+  if (variant == 2) return a.NCH == 2 ? launch_step_sgn<true, JT>(a, s) : launch_step_sgn<false, JT>(a, s);
   if (a.NCH == 2)
     return variant == 0 ? launch_step_n<0, 0, 2, JT>(a, s) : launch_step_n<1, 0, 2, JT>(a, s);
   return variant == 0 ? launch_step_n<0, 0, 1, JT>(a, s) : launch_step_n<1, 0, 1, JT>(a, s);
@@ -661,7 +922,7 @@ cudaError_t launch_fac_head(const FacHeadArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_fac_sum(int variant, const FacSumArgs& a, cudaStream_t s) {
-  if (variant == 2) return a.NCH == 2 ? launch_sum_n<1, 2>(a, s) : launch_sum_n<1, 1>(a, s);
+  if (variant == 2) return a.NCH == 2 ? launch_sum_sgn<true>(a, s) : launch_sum_sgn<false>(a, s);
   return a.NCH == 2 ? launch_sum_n<0, 2>(a, s) : launch_sum_n<0, 1>(a, s);
 }
 

@@ -282,7 +282,19 @@ struct FacSumArgs {
   void* U;               // [U rows x R]: FP32 (aSB / bSB) or BF16 (dSB)
   int32_t R, G, NCH, tiles;
   int32_t n, urows;      // state rows and U rows (bounds-checked build)
+  // dSB (k_fac_sum_sgn): item = (block, first word, end word, 0) of every block,
+  // its members four to a word: row | slot << 28, padded with kFacPad; CTA b
+  // takes blocks cta[b].x .. + cta[b].y, one per lane group, or, where cta[b].y
+  // is 0, block cta[b].x with all its lane groups
+  const uint4* gword;
+  const int2* cta;
+  int32_t nctas;
 };
+constexpr uint32_t kFacPad = 0x70000000u;  // row 0, slot 7: couples to no slot
+constexpr int kFacThreads = 128;           // threads per CTA of the factored kernels
+// dSB: a block with more members than this takes a whole CTA (16, 32 and 64
+// measured the same on 39,165 rows and on the 64-event batch)
+constexpr int kFacBig = 32;
 
 // Row head of the factored step (fac_head_words() 32-bit words per row): the
 // first kFacHead residual columns (0 past the row's end), the U rows
