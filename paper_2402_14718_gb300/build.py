@@ -24,7 +24,7 @@ LIB_CHECKED = os.path.join(PKG, "libsbtrack_checked.so")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 CU = ["api.cu", "device/kernels.cu", "device/stream.cu", "device/rw.cu", "device/noalloc.cu", "device/build.cu",
-      "device/probe.cu", "device/factor.cu"]
+      "device/probe.cu", "device/factor.cu", "device/run1.cu"]
 # FP64 builder kernels: one IEEE operation per written operation, as on the host
 CU_FLAGS = {"device/build.cu": ["-fmad=false"]}
 CPP = ["host/events.cpp", "host/qubo.cpp", "host/tracks.cpp"]

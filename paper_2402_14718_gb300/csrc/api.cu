@@ -27,6 +27,8 @@ using sbh::set_error;
 namespace {
 
 const int kEnergyRowsMin = 64;
+// shortest one-replica run that is worth k_run_r1 and, the first time, its tables
+const int kRun1Steps = 16;
 
 // A run of steps is captured into a CUDA graph the second time the same run
 // shape is asked for in a row, and replayed from then on; the first time it is
@@ -252,6 +254,17 @@ struct sb_ctx {
   int32_t* d_frw_pos = nullptr;
   void* d_frw_ejv = nullptr;
   int64_t x_rows = 0;                          // rows of each x buffer (>= n)
+  // one-replica run in one launch (k_run_r1): tables for this context's rows
+  struct Run1 {
+    int built = 0;           // 0: not tried, 1: tables ready, -1: does not fit
+    int32_t nct = 0, nx = 0, max_ent = 0;
+    size_t smem = 0;
+    sbd::Run1Cta* d_cta = nullptr;
+    int32_t *d_perm = nullptr, *d_deg = nullptr, *d_slice = nullptr, *d_ucol = nullptr;
+    float* d_ej = nullptr;
+    uint16_t* d_ei = nullptr;
+    unsigned long long* d_word = nullptr;
+  } run1;
   // sb_backward's work memory, kept for the next call of the same shape
   struct AdjWork {
     int32_t n = 0, R = 0, S = 0, K = 0;
@@ -427,6 +440,20 @@ void free_adj(sb_ctx* c) {
   w.n = w.R = w.S = w.K = 0;
 }
 
+void free_run1(sb_ctx* c) {
+  sb_ctx::Run1& r = c->run1;
+  if (r.d_cta) cudaFree(r.d_cta);
+  r.d_cta = nullptr;
+  dfree(r.d_perm);
+  dfree(r.d_deg);
+  dfree(r.d_slice);
+  dfree(r.d_ucol);
+  dfree(r.d_ej);
+  dfree(r.d_ei);
+  dfree(r.d_word);
+  r.built = 0;
+}
+
 void free_factor(sb_ctx* c) {
   dfree(c->d_f_gseg);
   dfree(c->d_f_gmem);
@@ -504,6 +531,7 @@ void free_all(sb_ctx* c) {
   dfree(c->d_bestE);
   dfree(c->d_bestr);
   dfree(c->d_T);
+  free_run1(c);
   dfree(c->d_inexact);
   dfree(c->d_spins);
   dfree(c->d_blk_row0);
@@ -1880,9 +1908,199 @@ sbd::Tiling step_tiling(const sb_ctx* c) {
   return sbd::make_tiling(c->Rs);
 }
 
+// Tables of k_run_r1: rows in contiguous chunks of about equal cost (nonzeros
+// plus a share per row), one per CTA; inside a chunk by decreasing degree, in
+// slices of 32 whose entries are padded to the slice's longest row (a multiple
+// of 8). r.built = -1 where a chunk's couplings and union do not fit in shared
+// memory: the step kernels serve the run. CTAs: one per 1,024 nonzeros or 128
+// rows, at most one per SM (us per step with 16 / 48 / 152 CTAs: 1,721 rows 1.7 /
+// 1.8 / 1.7; 10,214 rows 1.7 / 1.5 / 1.5; 10,878 rows does not fit / 2.2 / 2.2).
+sb_status ensure_run1(sb_ctx* c) {
+  sb_ctx::Run1& r = c->run1;
+  if (r.built) return SB_OK;
+  r.built = -1;
+  const int32_t n = c->n;
+  const int64_t nnz = c->nnz;
+  if (!c->sms) SB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+  if (nnz > (int64_t)c->sms * (sbd::kRun1Smem / 6) || n > c->sms * sbd::kRun1Threads) return SB_OK;
+  if (sbd::run1_prepare() != cudaSuccess) {
+    cudaGetLastError();
+    return SB_OK;
+  }
+  const int32_t* rp = c->h_rowptr.data();
+  const int32_t* col = c->h_col.data();
+  const int32_t nct = (int32_t)std::min<int64_t>(c->sms, std::max<int64_t>({1, nnz / 1024, n / 128}));
+  // chunk boundaries by cumulative cost, at most kRun1Threads rows each
+  std::vector<int32_t> row0((size_t)nct + 1, n);
+  const double total = (double)nnz + 8.0 * n;
+  row0[0] = 0;
+  int32_t at = 0;
+  for (int32_t b = 1; b < nct; ++b) {
+    const double want = total * b / nct;
+    while (at < n && (double)rp[at] + 8.0 * at < want) ++at;
+    const int32_t lo = row0[b - 1];
+    // no more rows than threads, here and in the chunks that follow
+    row0[b] = std::max(std::max(lo, n - (nct - b) * sbd::kRun1Threads),
+                       std::min(at, lo + sbd::kRun1Threads));
+  }
+  if (n - row0[nct - 1] > sbd::kRun1Threads) return SB_OK;
+  const size_t esz = c->jbf16 ? 2 : 4;
+  std::vector<unsigned char> jraw((size_t)nnz * esz);
+  if (nnz) SB_CUDA(cudaMemcpy(jraw.data(), c->d_J, jraw.size(), cudaMemcpyDeviceToHost));
+  struct Part {
+    std::vector<int32_t> perm, deg, slice, ucol;
+    std::vector<float> ej;
+    std::vector<uint16_t> ei;
+    bool ok = true;
+  };
+  std::vector<Part> P((size_t)nct);
+  const int parts = std::min(nct, 32);
+  const bool built = parallel_parts(nct, parts, [&](int, int64_t b0, int64_t b1) {
+    std::vector<int32_t> local((size_t)n, -1);  // index in the union (-1 between CTAs)
+    for (int64_t b = b0; b < b1; ++b) {
+      Part& q = P[(size_t)b];
+      const int32_t r0 = row0[b], r1 = row0[b + 1];
+      for (int32_t i = r0; i < r1; ++i) q.perm.push_back(i);
+      std::stable_sort(q.perm.begin(), q.perm.end(), [&](int32_t i, int32_t j) {
+        return rp[i + 1] - rp[i] > rp[j + 1] - rp[j];
+      });
+      for (int32_t p = rp[r0]; p < rp[r1]; ++p)
+        if (local[col[p]] < 0) {
+          local[col[p]] = 0;
+          q.ucol.push_back(col[p]);
+        }
+      std::sort(q.ucol.begin(), q.ucol.end());
+      q.ok = q.ucol.size() <= 65535;
+      for (size_t u = 0; u < q.ucol.size(); ++u) local[q.ucol[u]] = (int32_t)u;
+      for (int32_t s = 0; s < r1 - r0; s += 32) {
+        const int32_t len = (rp[q.perm[s] + 1] - rp[q.perm[s]] + 7) / 8 * 8;
+        const size_t e0 = q.ej.size();
+        q.slice.push_back((int32_t)e0);
+        q.ej.resize(e0 + (size_t)len * 32, 0.f);
+        q.ei.resize(e0 + (size_t)len * 32, 0);
+        for (int32_t l = 0; l < 32 && s + l < r1 - r0; ++l) {
+          const int32_t row = q.perm[s + l], d = rp[row + 1] - rp[row];
+          q.deg.push_back(d);
+          for (int32_t k = 0; k < d; ++k) {
+            const size_t p = (size_t)rp[row] + k, e = e0 + (size_t)(k / 4) * 128 + 4 * l + k % 4;
+            uint32_t bits = 0;
+            memcpy(&bits, jraw.data() + p * esz, esz);
+            if (esz == 2) bits <<= 16;
+            memcpy(&q.ej[e], &bits, 4);
+            q.ei[e] = (uint16_t)local[col[p]];
+          }
+        }
+      }
+      for (int32_t u : q.ucol) local[u] = -1;
+    }
+  }, 1);
+  if (!built) {
+    set_error("sb_run: host allocation failed");
+    r.built = 0;
+    return SB_ERR_OOM;
+  }
+  std::vector<sbd::Run1Cta> cta((size_t)nct);
+  std::vector<int32_t> perm, deg, slice, ucol;
+  size_t ents = 0, max_ent = 0, max_u = 0;
+  bool ok = true;
+  for (int32_t b = 0; b < nct; ++b) {
+    const Part& q = P[(size_t)b];
+    ok = ok && q.ok;
+    cta[b] = {row0[b], row0[b + 1] - row0[b], (int32_t)ents, (int32_t)q.ej.size(),
+              (int32_t)slice.size(), (int32_t)ucol.size(), (int32_t)q.ucol.size(), 0};
+    ents += q.ej.size();
+    max_ent = std::max(max_ent, q.ej.size());
+    max_u = std::max(max_u, q.ucol.size());
+    perm.insert(perm.end(), q.perm.begin(), q.perm.end());
+    deg.insert(deg.end(), q.deg.begin(), q.deg.end());
+    slice.insert(slice.end(), q.slice.begin(), q.slice.end());
+    ucol.insert(ucol.end(), q.ucol.begin(), q.ucol.end());
+  }
+  const int32_t nx = (int32_t)((max_u + 3) / 4 * 4);
+  const size_t smem = (size_t)nx * 4 + max_ent * 6 + 16;
+  if (!ok || ents > (size_t)INT32_MAX || smem > (size_t)sbd::kRun1Smem ||
+      sbd::run1_blocks_per_sm(smem) < 1)
+    return SB_OK;
+  std::vector<float> ej(std::max<size_t>(ents, 4));
+  std::vector<uint16_t> ei(std::max<size_t>(ents, 4));
+  parallel_parts(nct, parts, [&](int, int64_t b0, int64_t b1) {
+    for (int64_t b = b0; b < b1; ++b) {
+      std::copy(P[b].ej.begin(), P[b].ej.end(), ej.begin() + cta[b].ent0);
+      std::copy(P[b].ei.begin(), P[b].ei.end(), ei.begin() + cta[b].ent0);
+    }
+  }, 1);
+  if (cudaMalloc(&r.d_cta, cta.size() * sizeof(sbd::Run1Cta)) != cudaSuccess) {
+    cudaGetLastError();
+    r.d_cta = nullptr;
+    return SB_OK;  // no memory for the tables: the step kernels serve the run
+  }
+  if (dalloc(&r.d_perm, perm.size()) || dalloc(&r.d_deg, deg.size()) ||
+      dalloc(&r.d_slice, std::max<size_t>(slice.size(), 1)) ||
+      dalloc(&r.d_ucol, std::max<size_t>(ucol.size(), 1)) || dalloc(&r.d_ej, ej.size()) ||
+      dalloc(&r.d_ei, ei.size()) || dalloc(&r.d_word, (size_t)2 * n)) {
+    free_run1(c);
+    r.built = -1;
+    return SB_OK;
+  }
+  SB_CUDA(cudaMemcpy(r.d_cta, cta.data(), cta.size() * sizeof(sbd::Run1Cta), cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_perm, perm.data(), perm.size() * 4, cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_deg, deg.data(), deg.size() * 4, cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_slice, slice.data(), slice.size() * 4, cudaMemcpyHostToDevice));
+  if (!ucol.empty())
+    SB_CUDA(cudaMemcpy(r.d_ucol, ucol.data(), ucol.size() * 4, cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_ej, ej.data(), ej.size() * 4, cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_ei, ei.data(), ei.size() * 2, cudaMemcpyHostToDevice));
+  r.nct = nct;
+  r.nx = nx;
+  r.max_ent = (int32_t)max_ent;
+  r.smem = smem;
+  r.built = 1;
+  return SB_OK;
+}
+
 sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
                         const float* sched, cudaStream_t stream) {
   if (steps <= 0) return SB_OK;
+  // one replica, a run of some length and no step option set: all steps in one
+  // launch (the bounds-checked build keeps the step kernels, whose indices it checks)
+  if (c->R == 1 && steps >= kRun1Steps && !SB_CHECKED && c->r1_lanes < 0 && c->step_rt == 0 &&
+      c->step_rpc == 0 && c->groups == 1 && !c->l2_persist) {
+    sb_status st0 = ensure_run1(c);
+    if (st0) return st0;
+    const sb_ctx::Run1& r = c->run1;
+    if (r.built > 0) {
+      sbd::Run1Args ua{};
+      ua.cta = r.d_cta;
+      ua.perm = r.d_perm;
+      ua.deg = r.d_deg;
+      ua.slice = r.d_slice;
+      ua.ej = r.d_ej;
+      ua.ei = r.d_ei;
+      ua.ucol = r.d_ucol;
+      ua.n = c->n;
+      ua.nct = r.nct;
+      ua.nx = r.nx;
+      ua.max_ent = r.max_ent;
+      ua.h = c->d_h32;
+      ua.row_event = c->d_row_event;
+      ua.c0_ev = c->d_c0ev;
+      ua.sched = sched;
+      ua.steps = steps;
+      ua.cur = c->cur;
+      ua.a0 = (float)a0;
+      ua.dt = (float)dt;
+      ua.dta0 = (float)(dt * a0);
+      ua.x[0] = c->d_x[0];
+      ua.x[1] = c->d_x[1];
+      ua.y = c->d_y;
+      ua.word = r.d_word;
+      ua.err = c->d_err;
+      ua.wait_ns = 2000000000ull;
+      SB_CUDA(sbd::launch_run_r1(variant, ua, r.smem, stream));
+      if (steps & 1) c->cur ^= 1;
+      return SB_OK;
+    }
+  }
   if (c->use_stream) {
     sb_status st0 = ensure_stream(c);
     if (st0) return st0;
@@ -2930,6 +3148,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     ctx->d_tz = nullptr;
     ctx->graph.reset();
     if (ctx->tiles_built && (st = setup_tiles(ctx, rp, col))) return st;
+    free_run1(ctx);  // its tables carry J
     // the row-group kernel's entries carry J too
     if ((st = refill_rw(ctx))) return st;
     // the factored form's weight and residual were formed for the old couplings

@@ -257,6 +257,42 @@ struct StreamArgs {
   int32_t skip_stage;
 };
 
+// ---------------------------------------------------------------- one-replica run
+// k_run_r1 (run1.cu): every step of a one-replica run in one launch.
+constexpr int kRun1Threads = 1024;         // one row per thread
+constexpr int kRun1Smem = 220 * 1024;      // dynamic shared memory limit
+struct Run1Cta {
+  int32_t row0, nrows;   // rows [row0, row0 + nrows), nrows <= kRun1Threads
+  int32_t ent0, nent;    // entries (a multiple of 256) in ej / ei
+  int32_t slice0;        // first entry of its slices in `slice`
+  int32_t u0, nu;        // union of its rows' columns, in ucol
+  int32_t pad;
+};
+struct Run1Args {
+  const Run1Cta* cta;
+  const int32_t* perm;   // [n] row of each slot (rows of a CTA by decreasing degree)
+  const int32_t* deg;    // [n] nonzeros of each slot's row
+  const int32_t* slice;  // first entry, inside the CTA's, of each slice of 32 slots
+  const float* ej;       // weights; entry q of lane l of a slice at first + 128 (q / 4) + 4 l + q % 4
+  const uint16_t* ei;    // index in the CTA's union
+  const int32_t* ucol;
+  int32_t n, nct, nx, max_ent;  // nx: positions of the largest union, padded to 4
+  const float* h;
+  const int32_t* row_event;
+  const float* c0_ev;
+  const float* sched;
+  int32_t steps, cur;
+  float a0, dt, dta0;
+  float* x[2];
+  float* y;
+  unsigned long long* word;  // [2 n] {position, step} (zeroed by the launch)
+  int* err;              // set when a wait gives up
+  unsigned long long wait_ns;
+};
+cudaError_t run1_prepare();  // raise the kernels' shared-memory limit (once per device)
+int run1_blocks_per_sm(size_t smem);  // resident CTAs per SM (0: it does not fit)
+cudaError_t launch_run_r1(int variant, const Run1Args& a, size_t smem, cudaStream_t s);
+
 // ---------------------------------------------------------------- factored step
 // Coupling product split as jf * (M^T W M) x + residual x (factor.cu): group
 // blocks g (e.g. one hit each) with K slots; U rows hold sum_{s'} W[s][s']
