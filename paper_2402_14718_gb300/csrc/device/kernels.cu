@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
     const int ch = ch0 + j * G;
     if (ch >= C) continue;
     const size_t idx = (size_t)row * R + (size_t)ch * V;
-    Vec<V> xv = xo[j], yv = yo[j];
-    uint32_t sw = 0;
+    Vec<V> xv = xo[j], yv = yo[j], yt, fr;
+    uint32_t sw = 0, mk = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float x = xv.v[v], y = yv.v[v];
@@ -256,12 +256,12 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
       if (VARIANT == 0) force -= x * x * x;
       y = y + a.dt * force;
       x = x + a.dta0 * y;
-      if (record) {
-        a.ytil[idx + v] = y;
-        a.frec[idx + v] = acc[j][v];
-      }
       const bool wall = VARIANT != 0 && fabsf(x) > 1.f;
-      if (record) a.mask[idx + v] = wall ? 1 : 0;
+      if (record) {
+        yt.v[v] = y;
+        fr.v[v] = acc[j][v];
+        mk |= (wall ? 1u : 0u) << (8 * v);
+      }
       if (wall) {
         x = copysignf(1.f, x);
         y = 0.f;
@@ -272,6 +272,14 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
     }
     xv.st(a.xout + idx);
     yv.st(a.y + idx);
+    if (record) {
+      yt.st(a.ytil + idx);
+      fr.st(a.frec + idx);
+      if (V == 4)
+        *reinterpret_cast<uint32_t*>(a.mask + idx) = mk;
+      else
+        a.mask[idx] = (uint8_t)mk;
+    }
     if (use_sgn) {
       if (V == 4) {
         *reinterpret_cast<uint32_t*>(a.sgn_out + idx) = sw;
@@ -771,85 +779,110 @@ __global__ void k_pack_tz_f32(const float* J, const uint16_t* lidx, int64_t nnz,
 
 
 // ---------------------------------------------------------------- bSB adjoint
-// FP64 block sum of up to 4 values into acc[0..n) (one atomic per block and value).
+// FP64 block sums of 4 values, each added into its target (one atomic per block
+// and value; NULL: none). FP64 adds issue at a sixteenth of a warp per clock and
+// SM, so the warp sums exchange halves: after two exchanges a lane holds one of the
+// values (six adds per warp instead of twenty), and four threads add the warps' sums.
 __device__ __forceinline__ void block_add(double v0, double v1, double v2, double v3,
                                           double* t0, double* t1, double* t2, double* t3) {
   __shared__ double sh[4][kBlock / 32];
-  double v[4] = {v0, v1, v2, v3};
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0)
+  const bool h16 = lane & 16, h8 = lane & 8;
+  const double a0 = (h16 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h16 ? v0 : v2, 16);
+  const double a1 = (h16 ? v3 : v1) + __shfl_xor_sync(0xffffffffu, h16 ? v1 : v3, 16);
+  double s = (h8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) sh[q][wid] = v[q];
+  for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((lane & 7) == 0) sh[lane >> 3][wid] = s;  // lanes 0, 8, 16, 24: v0 .. v3
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) s[q] += sh[q][w];
-    double* tg[4] = {t0, t1, t2, t3};
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (tg[q]) atomicAdd(tg[q], s[q]);
+  if (threadIdx.x < 4) {
+    double* const t = threadIdx.x == 0 ? t0 : (threadIdx.x == 1 ? t1 : (threadIdx.x == 2 ? t2 : t3));
+    s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[threadIdx.x][w];
+    if (t) atomicAdd(t, s);
   }
 }
 
-// Sparse products of one row for this thread's replica chunks:
-// sJ = sum_j J_ij u_j, and (when x given) fJ = sum_j J_ij x_j, fC = sum_{conflict j} x_j.
-template <int V, int NCH, typename JT, bool TWO>
-__device__ __forceinline__ void adj_row_products(const AdjArgs& a, int row, int ch0, int C,
-                                                 unsigned mask, const float* u, const float* xk,
-                                                 float (&sJ)[NCH][V], float (&fJ)[NCH][V],
-                                                 float (&fC)[NCH][V]) {
-  const int G = a.G, g = ch0 % G;
+// Sparse products of one row for this thread's replica chunks (chl: chunk to
+// load; a lane past the row's last chunk reads it again, unused): sJ = sum_j J_ij
+// u_j and sC = sum over conflict neighbours of u_j, in CSR order. As in k_step each
+// lane reads the (col, J, class) triples itself, U neighbours in flight without
+// predicates, the next U triples on their way.
+template <int V, int NCH, int U, typename JT>
+__device__ __forceinline__ void adj_row_products(const AdjArgs& a, int row, const int (&chl)[NCH],
+                                                 const float* src, float (&sJ)[NCH][V],
+                                                 float (&sC)[NCH][V]) {
   const JT* J = static_cast<const JT*>(a.J);
 #pragma unroll
   for (int j = 0; j < NCH; ++j)
 #pragma unroll
-    for (int v = 0; v < V; ++v) sJ[j][v] = fJ[j][v] = fC[j][v] = 0.f;
-  const int p0 = a.rowptr[row], p1 = a.rowptr[row + 1];
-  for (int pb = p0; pb < p1; pb += G) {
-    const int cnt = min(G, p1 - pb);
-    int mc = 0, mk = 0;
-    float mv = 0.f;
-    if (g < cnt) {
-      mc = a.col[pb + g];
-      mv = jval(J, pb + g);
-      mk = a.cls[pb + g];
+    for (int v = 0; v < V; ++v) sJ[j][v] = sC[j][v] = 0.f;
+  const int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
+  int c[U], kc[U];
+  float w[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    c[u] = kc[u] = 0;
+    w[u] = 0.f;
+    if (p0 + u < p1) {
+      c[u] = __ldg(a.col + p0 + u);
+      w[u] = jval(J, p0 + u);
+      kc[u] = __ldg(a.cls + p0 + u);
     }
-    for (int q = 0; q < cnt; ++q) {
-      const int c = __shfl_sync(mask, mc, q, G);
-      const float w = __shfl_sync(mask, mv, q, G);
-      const int kc = __shfl_sync(mask, mk, q, G);
+  }
+  int p = p0;
+  for (; p + U <= p1; p += U) {
+    Vec<V> uv[U][NCH];
+    float wc[U];
+    int kk[U];
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const int ch = ch0 + j * G;
-        if (ch >= C) continue;
-        const size_t off = (size_t)c * a.R + (size_t)ch * V;
-        Vec<V> uv;
-        uv.ldg(u + off);
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int v = 0; v < V; ++v) sJ[j][v] = fmaf(w, uv.v[v], sJ[j][v]);
-        if (TWO) {
-          Vec<V> xv;
-          xv.ldg(xk + off);
+      for (int j = 0; j < NCH; ++j) uv[u][j].ldg(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
 #pragma unroll
-          for (int v = 0; v < V; ++v) {
-            fJ[j][v] = fmaf(w, xv.v[v], fJ[j][v]);
-            if (kc) fC[j][v] += xv.v[v];
-          }
-        }
+    for (int u = 0; u < U; ++u) {
+      wc[u] = w[u];
+      kk[u] = kc[u];
+      if (p + U + u < p1) {
+        c[u] = __ldg(a.col + p + U + u);
+        w[u] = jval(J, p + U + u);
+        kc[u] = __ldg(a.cls + p + U + u);
       }
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < NCH; ++j)
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          sJ[j][v] = fmaf(wc[u], uv[u][j].v[v], sJ[j][v]);
+          if (kk[u]) sC[j][v] += uv[u][j].v[v];
+        }
+  }
+  if (p < p1) {
+    Vec<V> uv[U - 1][NCH];
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+#pragma unroll
+      for (int j = 0; j < NCH; ++j)
+        if (p + u < p1) uv[u][j].ldg(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (p + u < p1)
+#pragma unroll
+        for (int j = 0; j < NCH; ++j)
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            sJ[j][v] = fmaf(w[u], uv[u][j].v[v], sJ[j][v]);
+            if (kc[u]) sC[j][v] += uv[u][j].v[v];
+          }
   }
 }
 
 // lambda_x = (-J x_S - h) / R, lambda_y = 0; loss, dL/dh_i = -sum_r x_S / R and the
 // explicit w_c term sum x (C x) / (8 R).
-template <int V, int NCH, typename JT>
-__global__ void __launch_bounds__(kBlock) k_adj_init(const AdjArgs a) {
+template <int V, int NCH, int U, typename JT>
+__global__ void __launch_bounds__(kBlock, (V == 4 && NCH > 1 ? 1 : 2)) k_adj_init(const AdjArgs a) {
   const int G = a.G;
   const int gid = threadIdx.x / G, g = threadIdx.x - gid * G;
   const int row = blockIdx.x * (blockDim.x / G) + gid;
@@ -858,8 +891,11 @@ __global__ void __launch_bounds__(kBlock) k_adj_init(const AdjArgs a) {
   double loss = 0.0, wc = 0.0, ghr = 0.0;
   if (row < a.n) {
     const unsigned mask = group_mask(G);
-    float sJ[NCH][V], fJ[NCH][V], fC[NCH][V];
-    adj_row_products<V, NCH, JT, true>(a, row, ch0, C, mask, a.x, a.x, sJ, fJ, fC);
+    int chl[NCH];
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) chl[j] = min(ch0 + j * G, C - 1);
+    float fJ[NCH][V], fC[NCH][V];
+    adj_row_products<V, NCH, U, JT>(a, row, chl, a.x, fJ, fC);
     const float hi = a.h[row];
     const double invR = 1.0 / a.R;
 #pragma unroll
@@ -904,113 +940,79 @@ __global__ void k_adj_phase1(const AdjArgs a) {
 // in FP32 and summed in FP64 (FP64 arithmetic is scarce on this part). A
 // block walks several row groups (grid-stride), so only a few blocks per SM
 // add their sums into the shared FP64 totals.
-template <int V, int NCH, typename JT>
-__global__ void __launch_bounds__(kBlock) k_adj_phase2(const AdjArgs a) {
+// Neighbours as in k_step: each lane reads the (col, J, class) triples itself, U
+// in flight without predicates, the next U on their way, the row's own values
+// first. (Triples loaded G at a time and broadcast by shuffles, scalar own
+// values and twenty FP64 adds per warp sum: 19.8 us for 10,878 rows at R = 32 by
+// itself, 15.3 now.)
+template <int V, int NCH, int U, typename JT>
+__global__ void __launch_bounds__(kBlock, (V == 4 && NCH > 1 ? 1 : 2)) k_adj_phase2(const AdjArgs a) {
   const int G = a.G;
   const int gid = threadIdx.x / G, g = threadIdx.x - gid * G;
   const int C = a.R / V;
   const int ch0 = blockIdx.y * (G * NCH) + g;
   double gdt = 0.0, gc0 = 0.0, ga = 0.0, gwc = 0.0;
   const int rstep = gridDim.x * (blockDim.x / G);
+  const unsigned mask = group_mask(G);
+  int chl[NCH];
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) chl[j] = min(ch0 + j * G, C - 1);
+  const float pa = a.a0 - __ldg(a.sched + a.k);
+  const float dtc0 = a.dt * a.c0;
+  const float dta0 = a.dt * a.a0;
   for (int row = blockIdx.x * (blockDim.x / G) + gid; row < a.n; row += rstep) {
     double ghr = 0.0;
-    const unsigned mask = group_mask(G);
-    const JT* J = static_cast<const JT*>(a.J);
-    float sJ[NCH][V], sC[NCH][V];
-#pragma unroll
-    for (int j = 0; j < NCH; ++j)
-#pragma unroll
-      for (int v = 0; v < V; ++v) sJ[j][v] = sC[j][v] = 0.f;
-    const int p0 = a.rowptr[row], p1 = a.rowptr[row + 1];
-    for (int pb = p0; pb < p1; pb += G) {
-      const int cnt = min(G, p1 - pb);
-      int mc = 0, mk = 0;
-      float mv = 0.f;
-      if (g < cnt) {
-        mc = a.col[pb + g];
-        mv = jval(J, pb + g);
-        mk = a.cls[pb + g];
-      }
-      int q = 0;
-      for (; q + 4 <= cnt; q += 4) {  // four neighbours' loads in flight, then their FMAs in order
-        int c[4], kc[4];
-        float w[4];
-        Vec<V> uv[4][NCH];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          c[u] = __shfl_sync(mask, mc, q + u, G);
-          w[u] = __shfl_sync(mask, mv, q + u, G);
-          kc[u] = __shfl_sync(mask, mk, q + u, G);
-#pragma unroll
-          for (int j = 0; j < NCH; ++j) {
-            const int ch = ch0 + j * G;
-            if (ch < C) uv[u][j].ldg(a.lyt + (size_t)c[u] * a.R + (size_t)ch * V);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int j = 0; j < NCH; ++j) {
-            const int ch = ch0 + j * G;
-            if (ch >= C) continue;
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-              sJ[j][v] = fmaf(w[u], uv[u][j].v[v], sJ[j][v]);
-              if (kc[u]) sC[j][v] += uv[u][j].v[v];
-            }
-          }
-      }
-      for (; q < cnt; ++q) {
-        const int c = __shfl_sync(mask, mc, q, G);
-        const float w = __shfl_sync(mask, mv, q, G);
-        const int kc = __shfl_sync(mask, mk, q, G);
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {
-          const int ch = ch0 + j * G;
-          if (ch >= C) continue;
-          Vec<V> uv;
-          uv.ldg(a.lyt + (size_t)c * a.R + (size_t)ch * V);
-#pragma unroll
-          for (int v = 0; v < V; ++v) {
-            sJ[j][v] = fmaf(w, uv.v[v], sJ[j][v]);
-            if (kc) sC[j][v] += uv.v[v];
-          }
-        }
-      }
-    }
     const float hi = a.h[row];
-    const float pa = a.a0 - __ldg(a.sched + a.k);
-    const float dtc0 = a.dt * a.c0;
-    const float dta0 = a.dt * a.a0;
+    float sJ[NCH][V], sC[NCH][V];
+    adj_row_products<V, NCH, U, JT>(a, row, chl, a.lyt, sJ, sC);
     float tdt = 0.f, tc0 = 0.f, ta = 0.f, twc = 0.f, thr = 0.f;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       const int ch = ch0 + j * G;
       if (ch >= C) continue;
       const size_t idx = (size_t)row * a.R + (size_t)ch * V;
+      Vec<V> xv, lytv, lxv, fv, ytv, lxo, lyo;
+      xv.ldg(a.x + idx);
+      lytv.ldg(a.lyt + idx);
+      lxv.ld(a.lx + idx);
+      fv.ldg(a.frec + idx);
+      ytv.ldg(a.ytil + idx);
+      uint8_t mp[V];
+      if (a.mask_prev) {
+        if (V == 4) {
+          const uint32_t m4 = __ldg(reinterpret_cast<const uint32_t*>(a.mask_prev + idx));
+#pragma unroll
+          for (int v = 0; v < V; ++v) mp[v] = (uint8_t)(m4 >> (8 * v));
+        } else {
+#pragma unroll
+          for (int v = 0; v < V; ++v) mp[v] = __ldg(a.mask_prev + idx + v);
+        }
+      }
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        const float x = a.x[idx + v];
-        const float lyt = a.lyt[idx + v];
-        const float lxt = a.lx[idx + v];
-        const float fh = a.frec[idx + v] + hi;
+        const float x = xv.v[v];
+        const float lyt = lytv.v[v];
+        const float lxt = lxv.v[v];
+        const float fh = fv.v[v] + hi;
         const float F = -pa * x + a.c0 * fh;
-        tdt += lyt * F + lxt * a.a0 * a.ytil[idx + v];
+        tdt += lyt * F + lxt * a.a0 * ytv.v[v];
         tc0 += lyt * a.dt * fh;
         ta += lyt * a.dt * x;
         twc += dtc0 * x * (-0.25f * sC[j][v]);
         thr += dtc0 * lyt;
         const float lxk = lxt - a.dt * pa * lyt + a.dt * a.c0 * sJ[j][v];
         if (a.mask_prev) {  // phase 1 of step k - 1 on this element (as k_adj_phase1)
-          const bool keep = a.mask_prev[idx + v] == 0;
+          const bool keep = mp[v] == 0;
           const float lxp = keep ? lxk : 0.f;
-          a.lx[idx + v] = lxp;
-          a.lyt_out[idx + v] = (keep ? lyt : 0.f) + dta0 * lxp;
+          lxo.v[v] = lxp;
+          lyo.v[v] = (keep ? lyt : 0.f) + dta0 * lxp;
         } else {
-          a.lx[idx + v] = lxk;
-          a.ly[idx + v] = lyt;
+          lxo.v[v] = lxk;
+          lyo.v[v] = lyt;
         }
       }
+      lxo.st(a.lx + idx);
+      lyo.st((a.mask_prev ? a.lyt_out : a.ly) + idx);
     }
     gdt += tdt;
     gc0 += tc0;
@@ -1037,11 +1039,12 @@ cudaError_t launch_adj_vn(int which, int jbf16, const Tiling& t, const AdjArgs& 
                           cudaStream_t s) {
   const int groups = kBlock / t.G;
   dim3 grid((a.n + groups - 1) / groups, t.tiles);
+  constexpr int U = V == 1 ? 8 : (NCH == 1 ? 8 : (NCH == 2 ? 4 : 2));
   if (which == 0) {
     if (jbf16)
-      k_adj_init<V, NCH, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
+      k_adj_init<V, NCH, U, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
     else
-      k_adj_init<V, NCH, float><<<grid, kBlock, 0, s>>>(a);
+      k_adj_init<V, NCH, U, float><<<grid, kBlock, 0, s>>>(a);
   } else {
     // a few blocks per SM walk the rows, so few blocks add into the FP64 totals
     int dev = 0, sms = 0;
@@ -1049,9 +1052,9 @@ cudaError_t launch_adj_vn(int which, int jbf16, const Tiling& t, const AdjArgs& 
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
       grid.x = std::min<unsigned>(grid.x, (unsigned)std::max(1, 4 * sms / (int)grid.y));
     if (jbf16)
-      k_adj_phase2<V, NCH, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
+      k_adj_phase2<V, NCH, U, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
     else
-      k_adj_phase2<V, NCH, float><<<grid, kBlock, 0, s>>>(a);
+      k_adj_phase2<V, NCH, U, float><<<grid, kBlock, 0, s>>>(a);
   }
   return cudaGetLastError();
 }
@@ -1301,11 +1304,13 @@ __device__ __forceinline__ int whole_b(float j) {
 }
 
 // A team of L x S lanes owns a row: lane l of slice s holds the replicas 8 l ..
-// 8 l + 7 (one byte of bits per neighbour) of every S-th nonzero, four in
-// flight. Few replicas leave few bytes per row, so the slices then share a
+// 8 l + 7 (one byte of bits per neighbour) of every S-th nonzero, eight in flight
+// (39,165 rows R = 256, whole readout: 180 us with eight and three CTAs per SM, 198
+// with four and four CTAs). Few replicas leave few bytes per row, so the slices then share a
 // row's nonzeros (whole-number sums: any split gives the same value).
 template <typename JT>
-__global__ void __launch_bounds__(kBlock) k_energy_bits(const EnergyBitArgs a, int L, int S) {
+__global__ void __launch_bounds__(kBlock, 3) k_energy_bits(const EnergyBitArgs a, int L, int S) {
+  constexpr int U = 8;
   extern __shared__ double sm[];
   const int TS = L * S;
   const int team = threadIdx.x / TS, t = threadIdx.x - team * TS;
@@ -1333,22 +1338,50 @@ __global__ void __launch_bounds__(kBlock) k_energy_bits(const EnergyBitArgs a, i
     int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
     chk_rows(p0, p1, a.nnz);
     const unsigned own = bits[(size_t)row * a.bstride];
-    for (int p = p0 + sl; p < p1; p += 4 * S) {
-      int ib[4];
-      unsigned w[4];
+    // U neighbours in flight without predicates, the next U (col, J) on their way
+    auto take = [&](unsigned w, int ib) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = p + u * S;
-        const bool in_row = q < p1;
-        const int c = chk_idx(__ldg(a.col + (in_row ? q : p)), a.n, kChkCol);
-        ib[u] = in_row ? whole_b(jval(J, q)) : 0;
-        w[u] = __ldg(bits + (size_t)c * a.bstride);
+      for (int v = 0; v < 8; ++v)
+        if (w & (1u << v)) in[v] += ib;
+    };
+    int c[U];
+    float jq[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = p0 + sl + u * S;
+      c[u] = 0;
+      jq[u] = 0.f;
+      if (q < p1) {
+        c[u] = chk_idx(__ldg(a.col + q), a.n, kChkCol);
+        jq[u] = jval(J, q);
+      }
+    }
+    int p = p0 + sl;
+    for (; p + (U - 1) * S < p1; p += U * S) {
+      unsigned w[U];
+      int ib[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) w[u] = __ldg(bits + (size_t)c[u] * a.bstride);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        ib[u] = whole_b(jq[u]);
+        const int q = p + (U + u) * S;
+        if (q < p1) {
+          c[u] = chk_idx(__ldg(a.col + q), a.n, kChkCol);
+          jq[u] = jval(J, q);
+        }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < U; ++u) take(w[u], ib[u]);
+    }
+    if (p < p1) {
+      unsigned w[U - 1];
 #pragma unroll
-        for (int v = 0; v < 8; ++v)
-          if (w[u] & (1u << v)) in[v] += ib[u];
+      for (int u = 0; u < U - 1; ++u)
+        if (p + u * S < p1) w[u] = __ldg(bits + (size_t)c[u] * a.bstride);
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (p + u * S < p1) take(w[u], whole_b(jq[u]));
     }
     for (int off = L; off < TS; off <<= 1)
 #pragma unroll
