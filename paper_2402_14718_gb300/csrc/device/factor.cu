@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
+#include "pdl.cuh"
 #include "signs.cuh"
 
 namespace sbd {
@@ -53,8 +54,8 @@ struct Words;
 template <>
 struct Words<2> {
   uint32_t w[2];
-  __device__ __forceinline__ void ldg(const void* p) {
-    const uint2 t = __ldg(static_cast<const uint2*>(p));
+  __device__ __forceinline__ void ld(const void* p) {
+    const uint2 t = *static_cast<const uint2*>(p);
     w[0] = t.x;
     w[1] = t.y;
   }
@@ -65,8 +66,8 @@ struct Words<2> {
 template <>
 struct Words<4> {
   uint32_t w[4];
-  __device__ __forceinline__ void ldg(const void* p) {
-    const uint4 t = __ldg(static_cast<const uint4*>(p));
+  __device__ __forceinline__ void ld(const void* p) {
+    const uint4 t = *static_cast<const uint4*>(p);
     w[0] = t.x;
     w[1] = t.y;
     w[2] = t.z;
@@ -93,7 +94,7 @@ struct Chunk<0, NCH> {
   __device__ __forceinline__ void load(const FacSumArgs& a, size_t off, int G, int row) {
 #pragma unroll
     for (int j = 0; j < NCH; ++j)
-      t[j] = __ldg(reinterpret_cast<const float4*>(a.xin + (size_t)row * a.R + off) + G * j);
+      t[j] = reinterpret_cast<const float4*>(a.xin + (size_t)row * a.R + off)[G * j];
   }
   __device__ __forceinline__ void add_to(float (&u)[P]) const {
 #pragma unroll
@@ -207,19 +208,20 @@ __global__ void __launch_bounds__(kFacBlock, 7) k_fac_sum_sgn(const FacSumArgs a
   int w = item.y + (big ? gq : 0);
   uint4 m0 = w < item.z ? __ldg(a.gword + w) : pad;
   uint4 m1 = w + step < item.z ? __ldg(a.gword + w + step) : pad;
+  pdl_wait();  // from here on: what earlier launches write
   while (w < item.z) {
     const uint32_t m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
     const bool two = w + step < item.z;
     uint2 v[8];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      v[u] = __ldg(reinterpret_cast<const uint2*>(
-          sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R));
+      v[u] = *reinterpret_cast<const uint2*>(
+          sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R);
     if (two) {
 #pragma unroll
       for (int u = 4; u < 8; ++u)
-        v[u] = __ldg(reinterpret_cast<const uint2*>(
-            sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R));
+        v[u] = *reinterpret_cast<const uint2*>(
+            sg + (size_t)chk_idx((int)(m[u] & 0x0fffffffu), a.n, kChkMember) * R);
     }
     w += 2 * step;
     m0 = w < item.z ? __ldg(a.gword + w) : pad;
@@ -296,6 +298,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
     for (int v = 0; v < P; ++v) U[s][v] = 0.f;
   // this item's members in one pass, G entries per load, four rows in flight;
   // each lane's entry carries its row and slot, broadcast by shuffles
+  if (item.y >= item.z) pdl_wait();
   for (int mb = item.y; mb < item.z; mb += G) {
     const int cnt = min(G, item.z - mb);
     int mr = 0, ms = 0;
@@ -305,6 +308,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
 #pragma unroll
       for (int s = 1; s < K; ++s) ms += t >= bnd[s] ? 1 : 0;
     }
+    if (mb == item.y) pdl_wait();  // from here on: what earlier launches write
     int q = 0;
     for (; q + 4 <= cnt; q += 4) {
       int r[4], sl[4];
@@ -417,7 +421,7 @@ __device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, f
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int j = 0; j < NCH; ++j)
-          t[u][j] = __ldg(reinterpret_cast<const float4*>(xin + (size_t)c[u] * R + off) + G * j);
+          t[u][j] = reinterpret_cast<const float4*>(xin + (size_t)c[u] * R + off)[G * j];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -430,7 +434,7 @@ __device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, f
     } else {
       Words<kSgnPer / 4> t[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) t[u].ldg(sgn_in + (size_t)c[u] * R + off);
+      for (int u = 0; u < 4; ++u) t[u].ld(sgn_in + (size_t)c[u] * R + off);
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -444,7 +448,7 @@ __device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, f
     if (MODE == 0) {
 #pragma unroll
       for (int j = 0; j < NCH; ++j) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(xin + (size_t)c * R + off) + G * j);
+        const float4 t = reinterpret_cast<const float4*>(xin + (size_t)c * R + off)[G * j];
         acc[4 * j] = fmaf(w, t.x, acc[4 * j]);
         acc[4 * j + 1] = fmaf(w, t.y, acc[4 * j + 1]);
         acc[4 * j + 2] = fmaf(w, t.z, acc[4 * j + 2]);
@@ -452,7 +456,7 @@ __device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, f
       }
     } else {
       Words<kSgnPer / 4> t;
-      t.ldg(sgn_in + (size_t)c * R + off);
+      t.ld(sgn_in + (size_t)c * R + off);
 #pragma unroll
       for (int v = 0; v < kSgnPer && v < P; ++v)
         acc[v] = fmaf(w, scaled_sign_of_byte(t.w[v >> 2], v & 3), acc[v]);
@@ -469,7 +473,7 @@ struct URow<0, NCH> {
   __device__ __forceinline__ void load(const void* U, size_t base, int G) {
 #pragma unroll
     for (int j = 0; j < NCH; ++j)
-      t[j] = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(U) + base) + G * j);
+      t[j] = reinterpret_cast<const float4*>(static_cast<const float*>(U) + base)[G * j];
   }
   __device__ __forceinline__ void add_to(float (&fu)[4 * NCH]) const {
 #pragma unroll
@@ -487,7 +491,7 @@ struct URow<1, 2> {  // dSB with FP32 U rows
   __device__ __forceinline__ void load(const void* U, size_t base, int) {
 #pragma unroll
     for (int h = 0; h < kSgnPer / 4; ++h)
-      t[h] = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(U) + base) + h);
+      t[h] = reinterpret_cast<const float4*>(static_cast<const float*>(U) + base)[h];
   }
   __device__ __forceinline__ void add_to(float (&fu)[kSgnPer]) const {
 #pragma unroll
@@ -505,7 +509,7 @@ struct URow<1, NCH> {
   __device__ __forceinline__ void load(const void* U, size_t base, int) {
     const uint16_t* p = static_cast<const uint16_t*>(U) + base;
 #pragma unroll
-    for (int h = 0; h < kSgnPer / 8; ++h) t[h].ldg(p + 8 * h);
+    for (int h = 0; h < kSgnPer / 8; ++h) t[h].ld(p + 8 * h);
   }
   __device__ __forceinline__ void add_to(float (&fu)[kSgnPer]) const {
 #pragma unroll
@@ -534,6 +538,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
                                : (size_t)blockIdx.y * (kSgnPer * G) + kSgnPer * l;
   const size_t idx = (size_t)row * R + off;
   const JT* J = static_cast<const JT*>(a.rJ);
+  pdl_wait();
   // the row's own x and y and its U rows are read after the residual walk:
   // ask for them in L2 now, so that those loads do not wait on HBM
 #pragma unroll
@@ -606,7 +611,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   // symplectic Euler: momentum with the old position, then position, then wall
   const float pa = a.a0 - __ldg(a.sched + a.k);
   const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
-  const float c0 = __ldg(a.c0_ev + ev);
+  const float c0 = a.c0_ev[ev];
   const float hi = __ldg(a.h + row);
   Words<kSgnPer / 4> sw;  // dSB: the new sign bytes
 #pragma unroll
@@ -615,7 +620,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
     const size_t o = MODE == 0 ? idx + 4 * G * j : idx + 4 * j;
-    const float4 xo = __ldg(reinterpret_cast<const float4*>(a.xin + o));
+    const float4 xo = *reinterpret_cast<const float4*>(a.xin + o);
     const float4 yo = *reinterpret_cast<const float4*>(a.y + o);
     float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
 #pragma unroll
@@ -674,12 +679,13 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
   const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
   const float hi = __ldg(a.h + row);
   chk_rows(p0, p1, a.rnnz);
+  pdl_wait();  // from here on: what earlier launches write
   prefetch_l2(a.xin + idx);
   prefetch_l2(a.y + idx);
   const uint8_t* const sg = a.sgn_in + off;
   const int L = p1 - p0;
   auto gather = [&](uint32_t c) {
-    return __ldg(reinterpret_cast<const uint2*>(sg + (size_t)chk_idx((int)c, a.n, kChkCol) * R));
+    return *reinterpret_cast<const uint2*>(sg + (size_t)chk_idx((int)c, a.n, kChkCol) * R);
   };
   uint2 s0[4], s1[4];
   const uint32_t ca[4] = {hc0.x, hc0.y, hc0.z, hc0.w}, cb[4] = {hc1.x, hc1.y, hc1.z, hc1.w};
@@ -690,7 +696,7 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
     for (int u = 0; u < 4; ++u) s1[u] = gather(cb[u]);
   }
   const uint32_t uw[4] = {hu.x, hu.y, hu.z, hu.w};
-  const float c0 = __ldg(a.c0_ev + ev);
+  const float c0 = a.c0_ev[ev];
   const float pa = a.a0 - __ldg(a.sched + a.k);
 
   // residual row in column order: weights scaled by 2^7, sign bytes read as 2^-7 sgn
@@ -800,8 +806,7 @@ cudaError_t launch_sum_k(const FacSumArgs& a, cudaStream_t s) {
   if (a.nitems <= 0) return cudaSuccess;
   const int per = kFacBlock / a.G;
   dim3 grid((a.nitems + per - 1) / per, a.tiles);
-  k_fac_sum<MODE, NCH, K><<<grid, kFacBlock, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k_fac_sum<MODE, NCH, K>, grid, kFacBlock, a, s);
 }
 
 template <int MODE, int NCH>
@@ -819,8 +824,7 @@ template <int VARIANT, int MODE, int NCH, int K, typename JT>
 cudaError_t launch_step_k(const FacStepArgs& a, cudaStream_t s) {
   const int per = kFacBlock / a.G;
   dim3 grid((a.n + per - 1) / per, a.tiles);
-  k_step_fac<VARIANT, MODE, NCH, K, JT><<<grid, kFacBlock, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k_step_fac<VARIANT, MODE, NCH, K, JT>, grid, kFacBlock, a, s);
 }
 
 template <int VARIANT, int MODE, int NCH, typename JT>
@@ -839,13 +843,12 @@ cudaError_t launch_sum_sgn(const FacSumArgs& a, cudaStream_t s) {
   if (a.nctas <= 0) return cudaSuccess;
   dim3 grid(a.nctas, a.tiles);
   switch (a.K) {
-    case 1: k_fac_sum_sgn<UF32, 1><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 2: k_fac_sum_sgn<UF32, 2><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 3: k_fac_sum_sgn<UF32, 3><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 4: k_fac_sum_sgn<UF32, 4><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 1: return launch_pdl(k_fac_sum_sgn<UF32, 1>, grid, kFacBlock, a, s);
+    case 2: return launch_pdl(k_fac_sum_sgn<UF32, 2>, grid, kFacBlock, a, s);
+    case 3: return launch_pdl(k_fac_sum_sgn<UF32, 3>, grid, kFacBlock, a, s);
+    case 4: return launch_pdl(k_fac_sum_sgn<UF32, 4>, grid, kFacBlock, a, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <bool UF32, typename JT>
@@ -853,13 +856,12 @@ cudaError_t launch_step_sgn(const FacStepArgs& a, cudaStream_t s) {
   const int per = kFacBlock / a.G;
   dim3 grid((a.n + per - 1) / per, a.tiles);
   switch (a.K) {
-    case 1: k_step_fac_sgn<UF32, 1, JT><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 2: k_step_fac_sgn<UF32, 2, JT><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 3: k_step_fac_sgn<UF32, 3, JT><<<grid, kFacBlock, 0, s>>>(a); break;
-    case 4: k_step_fac_sgn<UF32, 4, JT><<<grid, kFacBlock, 0, s>>>(a); break;
+    case 1: return launch_pdl(k_step_fac_sgn<UF32, 1, JT>, grid, kFacBlock, a, s);
+    case 2: return launch_pdl(k_step_fac_sgn<UF32, 2, JT>, grid, kFacBlock, a, s);
+    case 3: return launch_pdl(k_step_fac_sgn<UF32, 3, JT>, grid, kFacBlock, a, s);
+    case 4: return launch_pdl(k_step_fac_sgn<UF32, 4, JT>, grid, kFacBlock, a, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename JT>

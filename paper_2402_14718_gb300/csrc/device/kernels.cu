@@ -19,6 +19,7 @@
 
 #include "../philox.h"
 #include "kernels.cuh"
+#include "pdl.cuh"
 #include "signs.cuh"
 
 namespace sbd {
@@ -102,15 +103,14 @@ struct Vec<1> {
 template <int V, bool SGN>
 struct Gathered {
   Vec<V> t;
-  __device__ __forceinline__ void ld(const StepArgs& a, size_t off) { t.ldg(a.xin + off); }
+  __device__ __forceinline__ void ld(const StepArgs& a, size_t off) { t.ld(a.xin + off); }
   __device__ __forceinline__ float get(int v) const { return t.v[v]; }
 };
 template <int V>
 struct Gathered<V, true> {
   uint32_t t;
   __device__ __forceinline__ void ld(const StepArgs& a, size_t off) {
-    t = V == 4 ? __ldg(reinterpret_cast<const uint32_t*>(a.sgn_in + off))
-               : (uint32_t)__ldg(a.sgn_in + off);
+    t = V == 4 ? *reinterpret_cast<const uint32_t*>(a.sgn_in + off) : (uint32_t)a.sgn_in[off];
   }
   __device__ __forceinline__ float get(int v) const { return scaled_sign_of_byte(t, v); }
 };
@@ -158,7 +158,6 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
   const int ch0 = (blockIdx.y + a.tile0) * (G * NCH) + g;
   const JT* J = static_cast<const JT*>(a.J);
   const int row_end = min(a.n, (blockIdx.x + 1) * a.rpc);
-  const float pa = a.a0 - __ldg(a.sched + a.k);
   int chl[NCH];  // chunk to load: a lane past the row's last chunk reads it again, unused
 #pragma unroll
   for (int j = 0; j < NCH; ++j) chl[j] = min(ch0 + j * G, C - 1);
@@ -173,16 +172,6 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
 
   int p0 = __ldg(a.rowptr + row), p1 = __ldg(a.rowptr + row + 1);
   chk_rows(p0, p1, a.nnz);
-  Vec<V> xo[NCH], yo[NCH];
-#pragma unroll
-  for (int j = 0; j < NCH; ++j) {
-    xo[j].ldg(a.xin + (size_t)row * R + (size_t)chl[j] * V);
-    if (ch0 + j * G < C) yo[j].ld(a.y + (size_t)row * R + (size_t)chl[j] * V);
-  }
-  const int e = a.row_event ? __ldg(a.row_event + row) : 0;
-  const float c0 = __ldg(a.c0_ev + e);
-  const float hi = __ldg(a.h + row);
-
   int c[U];
   float w[U];
 #pragma unroll
@@ -194,6 +183,18 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
       w[u] = jval(J, p0 + u);
     }
   }
+  const int e = a.row_event ? __ldg(a.row_event + row) : 0;
+  const float hi = __ldg(a.h + row);
+  pdl_wait();  // from here on: what earlier launches write
+  Vec<V> xo[NCH], yo[NCH];
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    xo[j].ld(a.xin + (size_t)row * R + (size_t)chl[j] * V);
+    if (ch0 + j * G < C) yo[j].ld(a.y + (size_t)row * R + (size_t)chl[j] * V);
+  }
+  const float c0 = a.c0_ev[e];
+  const float pa = a.a0 - __ldg(a.sched + a.k);
+
   int p = p0;
   for (; p + U <= p1; p += U) {
     Gathered<V, use_sgn> xv[U][NCH];
@@ -295,11 +296,8 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
 template <int V, int NCH, int U, int MODE>
 cudaError_t launch_step_u(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
   dim3 grid((a.n + a.rpc - 1) / a.rpc, t.tiles);
-  if (jbf16)
-    k_step<V, NCH, U, MODE, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
-  else
-    k_step<V, NCH, U, MODE, float><<<grid, kBlock, 0, s>>>(a);
-  return cudaGetLastError();
+  return jbf16 ? launch_pdl(k_step<V, NCH, U, MODE, __nv_bfloat16>, grid, kBlock, a, s)
+               : launch_pdl(k_step<V, NCH, U, MODE, float>, grid, kBlock, a, s);
 }
 
 // Neighbours in flight. More shorten the chain of a heavy row and cost
@@ -527,12 +525,13 @@ __global__ void __launch_bounds__(kDsbBlock, SB_DSB_MINB) k_step_dsb16(const Ste
         w[u] = jval(J, p0 + u);
       }
     }
+    pdl_wait();  // from here on: what earlier launches write
     int p = p0;
     for (; p + U <= p1; p += U) {
       uint4 sv[U];
       float wc[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) sv[u] = __ldg(reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R));
+      for (int u = 0; u < U; ++u) sv[u] = *reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         wc[u] = w[u] * kSignScale;  // 2^7 J: sign bytes read as 2^-7 sgn
@@ -553,7 +552,7 @@ __global__ void __launch_bounds__(kDsbBlock, SB_DSB_MINB) k_step_dsb16(const Ste
       uint4 sv[U - 1];
 #pragma unroll
       for (int u = 0; u < U - 1; ++u)
-        if (p + u < p1) sv[u] = __ldg(reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R));
+        if (p + u < p1) sv[u] = *reinterpret_cast<const uint4*>(sg + (size_t)c[u] * R);
 #pragma unroll
       for (int u = 0; u < U - 1; ++u)
         if (p + u < p1) {
@@ -566,14 +565,14 @@ __global__ void __launch_bounds__(kDsbBlock, SB_DSB_MINB) k_step_dsb16(const Ste
     }
     const float pa = a.a0 - __ldg(a.sched + a.k);
     const int e = a.row_event ? __ldg(a.row_event + row) : 0;
-    const float c0 = __ldg(a.c0_ev + e);
+    const float c0 = a.c0_ev[e];
     const float hi = __ldg(a.h + row);
     const size_t idx = (size_t)row * R + 16 * g;
     unsigned sw[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int h4 = 0; h4 < 4; ++h4) {
       Vec<4> xv, yv;
-      xv.ldg(a.xin + idx + 4 * h4);
+      xv.ld(a.xin + idx + 4 * h4);
       yv.ld(a.y + idx + 4 * h4);
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
@@ -830,6 +829,7 @@ __device__ __forceinline__ void adj_row_products(const AdjArgs& a, int row, cons
       kc[u] = __ldg(a.cls + p0 + u);
     }
   }
+  pdl_wait();  // from here on: what earlier launches write
   int p = p0;
   for (; p + U <= p1; p += U) {
     Vec<V> uv[U][NCH];
@@ -838,7 +838,7 @@ __device__ __forceinline__ void adj_row_products(const AdjArgs& a, int row, cons
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) uv[u][j].ldg(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
+      for (int j = 0; j < NCH; ++j) uv[u][j].ld(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       wc[u] = w[u];
@@ -865,7 +865,7 @@ __device__ __forceinline__ void adj_row_products(const AdjArgs& a, int row, cons
     for (int u = 0; u < U - 1; ++u)
 #pragma unroll
       for (int j = 0; j < NCH; ++j)
-        if (p + u < p1) uv[u][j].ldg(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
+        if (p + u < p1) uv[u][j].ld(src + (size_t)c[u] * a.R + (size_t)chl[j] * V);
 #pragma unroll
     for (int u = 0; u < U - 1; ++u)
       if (p + u < p1)
@@ -957,7 +957,6 @@ __global__ void __launch_bounds__(kBlock, (V == 4 && NCH > 1 ? 1 : 2)) k_adj_pha
   int chl[NCH];
 #pragma unroll
   for (int j = 0; j < NCH; ++j) chl[j] = min(ch0 + j * G, C - 1);
-  const float pa = a.a0 - __ldg(a.sched + a.k);
   const float dtc0 = a.dt * a.c0;
   const float dta0 = a.dt * a.a0;
   for (int row = blockIdx.x * (blockDim.x / G) + gid; row < a.n; row += rstep) {
@@ -965,6 +964,7 @@ __global__ void __launch_bounds__(kBlock, (V == 4 && NCH > 1 ? 1 : 2)) k_adj_pha
     const float hi = a.h[row];
     float sJ[NCH][V], sC[NCH][V];
     adj_row_products<V, NCH, U, JT>(a, row, chl, a.lyt, sJ, sC);
+    const float pa = a.a0 - __ldg(a.sched + a.k);
     float tdt = 0.f, tc0 = 0.f, ta = 0.f, twc = 0.f, thr = 0.f;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
@@ -972,20 +972,20 @@ __global__ void __launch_bounds__(kBlock, (V == 4 && NCH > 1 ? 1 : 2)) k_adj_pha
       if (ch >= C) continue;
       const size_t idx = (size_t)row * a.R + (size_t)ch * V;
       Vec<V> xv, lytv, lxv, fv, ytv, lxo, lyo;
-      xv.ldg(a.x + idx);
-      lytv.ldg(a.lyt + idx);
+      xv.ld(a.x + idx);
+      lytv.ld(a.lyt + idx);
       lxv.ld(a.lx + idx);
-      fv.ldg(a.frec + idx);
-      ytv.ldg(a.ytil + idx);
+      fv.ld(a.frec + idx);
+      ytv.ld(a.ytil + idx);
       uint8_t mp[V];
       if (a.mask_prev) {
         if (V == 4) {
-          const uint32_t m4 = __ldg(reinterpret_cast<const uint32_t*>(a.mask_prev + idx));
+          const uint32_t m4 = *reinterpret_cast<const uint32_t*>(a.mask_prev + idx);
 #pragma unroll
           for (int v = 0; v < V; ++v) mp[v] = (uint8_t)(m4 >> (8 * v));
         } else {
 #pragma unroll
-          for (int v = 0; v < V; ++v) mp[v] = __ldg(a.mask_prev + idx + v);
+          for (int v = 0; v < V; ++v) mp[v] = a.mask_prev[idx + v];
         }
       }
 #pragma unroll
@@ -1051,10 +1051,8 @@ cudaError_t launch_adj_vn(int which, int jbf16, const Tiling& t, const AdjArgs& 
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
       grid.x = std::min<unsigned>(grid.x, (unsigned)std::max(1, 4 * sms / (int)grid.y));
-    if (jbf16)
-      k_adj_phase2<V, NCH, U, __nv_bfloat16><<<grid, kBlock, 0, s>>>(a);
-    else
-      k_adj_phase2<V, NCH, U, float><<<grid, kBlock, 0, s>>>(a);
+    return jbf16 ? launch_pdl(k_adj_phase2<V, NCH, U, __nv_bfloat16>, grid, kBlock, a, s)
+                 : launch_pdl(k_adj_phase2<V, NCH, U, float>, grid, kBlock, a, s);
   }
   return cudaGetLastError();
 }
@@ -1573,11 +1571,8 @@ cudaError_t launch_step(int variant, int jbf16, const Tiling& t, const StepArgs&
     StepArgs b = a;
     b.rpc = rpc;
     dim3 grid((a.n + rpc - 1) / rpc, 1);
-    if (jbf16)
-      k_step_dsb16<__nv_bfloat16><<<grid, kDsbBlock, 0, s>>>(b);
-    else
-      k_step_dsb16<float><<<grid, kDsbBlock, 0, s>>>(b);
-    return cudaGetLastError();
+    return jbf16 ? launch_pdl(k_step_dsb16<__nv_bfloat16>, grid, kDsbBlock, b, s)
+                 : launch_pdl(k_step_dsb16<float>, grid, kDsbBlock, b, s);
   }
   if (t.V == 16) return cudaErrorInvalidValue;  // that tiling needs the dSB sign bytes
   if (t.V == 4) {

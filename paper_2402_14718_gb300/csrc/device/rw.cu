@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "kernels.cuh"
+#include "pdl.cuh"
 #include "signs.cuh"
 
 namespace sbd {
@@ -28,9 +29,6 @@ namespace {
 #endif
 #ifndef SB_RW_UB_NCH1
 #define SB_RW_UB_NCH1 4
-#endif
-#ifndef SB_RW_MINB
-#define SB_RW_MINB 1
 #endif
 
 // RW J values of one entry, read by one lane and broadcast by shuffles.
@@ -110,7 +108,7 @@ struct JPack<2, float> {
 // MODE: 0 aSB, 1 bSB, 2 dSB gathering x (sgn at use), 3 dSB gathering the
 // sign bytes written by the previous step (4 bytes per lane chunk)
 template <int RW, int NCH, int MODE, typename JT>
-__global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a) {
+__global__ void __launch_bounds__(kRwBlock, RW == 2 ? 9 : 1) k_step_rw(const RwArgs a) {
   constexpr int VARIANT = MODE == 3 ? 2 : MODE;
   constexpr bool use_sgn = MODE == 3;
   using P = JPack<RW, JT>;
@@ -125,7 +123,6 @@ __global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a
   const unsigned rb = (use_sgn ? 1u : 4u) * (unsigned)R;
   const int chunk = a.cta_order ? __ldg(a.cta_order + blockIdx.x) : (int)blockIdx.x;
   const int g_end = min(a.ngroups, (chunk + 1) * a.gpc);
-  const float pa = a.a0 - __ldg(a.sched + a.k);
   for (int grp = chunk * a.gpc + wid; grp < g_end; grp += kRwBlock / 32) {
     float acc[RW][NCH][4];
 #pragma unroll
@@ -144,6 +141,8 @@ __global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a
       pk = __ldg(a.ent + e0 + lane);
       jp.ld(a.ejv, e0 + lane);
     }
+    pdl_wait();  // from here on: what earlier launches write
+    const float pa = a.a0 - __ldg(a.sched + a.k);
     for (int eb = e0; eb < e1; eb += 32) {
       const int cnt = min(32, e1 - eb);
       int pkn = 0;
@@ -167,7 +166,7 @@ __global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a
             const uint32_t* ps = reinterpret_cast<const uint32_t*>(xl + (size_t)cu * rb);
 #pragma unroll
             for (int j = 0; j < NCH; ++j) {
-              const uint32_t t = __ldg(ps + 32 * j);
+              const uint32_t t = ps[32 * j];
 #pragma unroll
               for (int k = 0; k < 4; ++k) xv[u][j][k] = scaled_sign_of_byte(t, k);
             }
@@ -175,7 +174,7 @@ __global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a
             const float4* px = reinterpret_cast<const float4*>(xl + (size_t)cu * rb);
 #pragma unroll
             for (int j = 0; j < NCH; ++j) {
-              const float4 t = __ldg(px + 32 * j);
+              const float4 t = px[32 * j];
               xv[u][j][0] = t.x;
               xv[u][j][1] = t.y;
               xv[u][j][2] = t.z;
@@ -213,12 +212,12 @@ __global__ void __launch_bounds__(kRwBlock, SB_RW_MINB) k_step_rw(const RwArgs a
       const int row = __ldg(a.grows + (size_t)grp * RW + q);
       if (row < 0) continue;
       const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
-      const float c0 = __ldg(a.c0_ev + ev);
+      const float c0 = a.c0_ev[ev];
       const float hi = __ldg(a.h + row);
 #pragma unroll
       for (int j = 0; j < NCH; ++j) {
         const size_t idx = (size_t)row * R + rep0 + 128 * j;
-        const float4 xo = __ldg(reinterpret_cast<const float4*>(a.xin + idx));
+        const float4 xo = *reinterpret_cast<const float4*>(a.xin + idx);
         const float4 yo = *reinterpret_cast<const float4*>(a.y + idx);
         float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
         uint32_t sw = 0u;
@@ -249,16 +248,13 @@ template <int RW, int NCH, typename JT>
 cudaError_t launch_t(int variant, const RwArgs& a, cudaStream_t s) {
   dim3 grid((a.ngroups + a.gpc - 1) / a.gpc, a.R / (128 * NCH));
   switch (variant) {
-    case 0: k_step_rw<RW, NCH, 0, JT><<<grid, kRwBlock, 0, s>>>(a); break;
-    case 1: k_step_rw<RW, NCH, 1, JT><<<grid, kRwBlock, 0, s>>>(a); break;
+    case 0: return launch_pdl(k_step_rw<RW, NCH, 0, JT>, grid, kRwBlock, a, s);
+    case 1: return launch_pdl(k_step_rw<RW, NCH, 1, JT>, grid, kRwBlock, a, s);
     default:
       if (a.sgn_in)
-        k_step_rw<RW, NCH, 3, JT><<<grid, kRwBlock, 0, s>>>(a);
-      else
-        k_step_rw<RW, NCH, 2, JT><<<grid, kRwBlock, 0, s>>>(a);
-      break;
+        return launch_pdl(k_step_rw<RW, NCH, 3, JT>, grid, kRwBlock, a, s);
+      return launch_pdl(k_step_rw<RW, NCH, 2, JT>, grid, kRwBlock, a, s);
   }
-  return cudaGetLastError();
 }
 
 template <int RW, int NCH>
