@@ -1994,11 +1994,7 @@ sb_status ensure_run1(sb_ctx* c) {
       for (int32_t u : q.ucol) local[u] = -1;
     }
   }, 1);
-  if (!built) {
-    set_error("sb_run: host allocation failed");
-    r.built = 0;
-    return SB_ERR_OOM;
-  }
+  if (!built) return SB_OK;  // no host memory for the tables
   std::vector<sbd::Run1Cta> cta((size_t)nct);
   std::vector<int32_t> perm, deg, slice, ucol;
   size_t ents = 0, max_ent = 0, max_u = 0;
@@ -2058,15 +2054,25 @@ sb_status ensure_run1(sb_ctx* c) {
   return SB_OK;
 }
 
-sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
-                        const float* sched, cudaStream_t stream) {
+sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
+                                  const float* sched, cudaStream_t stream) {
   if (steps <= 0) return SB_OK;
   // one replica, a run of some length and no step option set: all steps in one
   // launch (the bounds-checked build keeps the step kernels, whose indices it checks)
   if (c->R == 1 && steps >= kRun1Steps && !SB_CHECKED && c->r1_lanes < 0 && c->step_rt == 0 &&
       c->step_rpc == 0 && c->groups == 1 && !c->l2_persist) {
-    sb_status st0 = ensure_run1(c);
-    if (st0) return st0;
+    // no tables are made on a stream that the caller captures: the step kernels,
+    // which need none, are recorded
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (!c->run1.built) SB_CUDA(cudaStreamIsCapturing(stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+      try {
+        if (sb_status st0 = ensure_run1(c)) return st0;
+      } catch (const std::bad_alloc&) {
+        free_run1(c);
+        c->run1.built = -1;
+      }
+    }
     const sb_ctx::Run1& r = c->run1;
     if (r.built > 0) {
       sbd::Run1Args ua{};
@@ -2114,7 +2120,7 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   int fG = 0, fNCH = 0, ftiles = 0;
   const int fac = (c->fac_set && c->fac_use != 0 && c->groups == 1 &&
                    sbd::fac_tiling(variant, c->Rs, &fG, &fNCH, &ftiles) &&
-                   (variant != SB_DSB || (c->dsb_signs && c->j_small)) &&
+                   (variant != SB_DSB || (c->dsb_signs && c->j_small && c->n <= sbd::kFacRows)) &&
                    (c->Rs == c->R || (variant == SB_DSB && c->b_whole)))
                       ? 1 : 0;
   // dSB: BF16 U rows hold sums of at most 256 members exactly; larger blocks
@@ -2534,6 +2540,32 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
   SB_CUDA(cudaGraphLaunch(gc.exec, stream));
   if ((steps & 1) && !x_inplace) c->cur ^= 1;
   return SB_OK;
+}
+
+// Rows R values apart again: the state of a replica count that was padded.
+sb_status unpad_state(sb_ctx* c, cudaStream_t stream) {
+  float *const x = c->d_x[c->cur], *const other = c->d_x[c->cur ^ 1];
+  const size_t bytes = (size_t)c->n * c->R * sizeof(float);
+  SB_CUDA(sbd::launch_repitch(x, c->Rs, other, c->R, c->n, c->R, stream));
+  SB_CUDA(sbd::launch_repitch(c->d_y, c->Rs, x, c->R, c->n, c->R, stream));
+  SB_CUDA(cudaMemcpyAsync(c->d_y, x, bytes, cudaMemcpyDeviceToDevice, stream));
+  c->cur ^= 1;
+  c->Rs = c->R;
+  c->graph.reset();
+  return SB_OK;
+}
+
+// The padded form takes kernels that want more memory than the unpadded one
+// (sign bytes, U rows, row-group tables). Where that is not there, the run takes
+// the unpadded form, which needs none of it; nothing has been launched by then.
+sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
+                        const float* sched, cudaStream_t stream) {
+  sb_status st = enqueue_steps_as_stored(c, variant, a0, dt, steps, sched, stream);
+  if (st != SB_ERR_OOM || c->Rs == c->R) return st;
+  dfree(c->d_sgn[0]);
+  dfree(c->d_sgn[1]);
+  if ((st = unpad_state(c, stream))) return st;
+  return enqueue_steps_as_stored(c, variant, a0, dt, steps, sched, stream);
 }
 
 // Energies of R replicas (from the current x, or from d_spins) into E_all (NULL:
@@ -3028,8 +3060,17 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
     }
     cudaStream_t s = (cudaStream_t)stream;
     // the kernels write the caller's buffers themselves where they are aligned
-    // for their type, else through the context's own and a copy
-    auto direct = [](void* p, size_t a) { return p && reinterpret_cast<uintptr_t>(p) % a == 0; };
+    // for their type and lie on the context's own device, else through the
+    // context's own and a copy (which refuses what is no device memory)
+    auto direct = [&](void* p, size_t a) {
+      cudaPointerAttributes at;
+      if (!p || reinterpret_cast<uintptr_t>(p) % a) return false;
+      if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+      return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+    };
     const bool dE = direct(d_E_all, 8), db = direct(d_best_E, 8), dr = direct(d_best_r, 4);
     sb_status st = readout(ctx, nullptr, ctx->R, s, dE ? d_E_all : nullptr,
                            db ? d_best_E : nullptr, dr ? d_best_r : nullptr);

@@ -327,6 +327,7 @@ struct FacSumArgs {
   int32_t nctas;
 };
 constexpr uint32_t kFacPad = 0x70000000u;  // row 0, slot 7: couples to no slot
+constexpr int32_t kFacRows = 1 << 28;      // rows that a member word can name
 constexpr int kFacThreads = 128;           // threads per CTA of the factored kernels
 // dSB: a block with more members than this takes a whole CTA (16, 32 and 64
 // measured the same on 39,165 rows and on the 64-event batch)
