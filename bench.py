@@ -210,8 +210,10 @@ def step_kernels(cfg, variant, R, info):
     if variant == "dsb" and cfg["tile"] == 0 and cfg["groups"] == 1 and R % 16 == 0 \
             and R // 16 <= 32 and (R // 16) & (R // 16 - 1) == 0:
         return ["k_step_dsb16"]
-    if R == 1:
-        return ["k_step_r1"]
+    if R == 1:  # all steps of a run in one launch unless a step option is set
+        one = cfg["tile"] == 0 and cfg["groups"] == 1 and not cfg["rows_per_cta"] \
+            and not cfg["l2_persist"]
+        return ["k_run_r1"] if one else ["k_step_r1"]
     return ["k_step"]
 
 
@@ -975,7 +977,8 @@ def run_ours(args):
                        "autotune": cfg, "autotune_us_per_step": tune_us,
                        "host_build_s": t_build},
             "roofline": roofline, "e2e": e2e,
-            "gpu_launches": (3 + (1 if variant == "dsb" else 0) + S * len(knames) + 4) * args.steps,
+            "gpu_launches": (3 + (1 if variant == "dsb" else 0) + (1 if knames == ["k_run_r1"] else S * len(knames)) + 4)
+            * args.steps,
             "clocks": clk, "wall_s_timed": t_wall}
     if ws > 1:
         # the job's best of every event over all ranks' replicas

@@ -107,8 +107,18 @@ struct JPack<2, float> {
 
 // MODE: 0 aSB, 1 bSB, 2 dSB gathering x (sgn at use), 3 dSB gathering the
 // sign bytes written by the previous step (4 bytes per lane chunk)
+// Residency (CTAs of 128 threads per SM): with two chunks per lane nine (BF16 J)
+// or eight (FP32), which fit without spills; with one chunk the compiler's own
+// choice (56 and 63 registers), whose order of loads is better than what a bound of
+// nine leaves it (10,878 rows, R = 128, FP32 12.6 us a step against 10.7). Per step
+// with / without the bound: 39,165 rows, R = 256, factored BF16 54.2 / 57.4 us, FP32
+// 68.1 / 72.0; R = 128, BF16 35.2 / 34.7.
+template <int RW, int NCH>
+constexpr int rw_blocks(int jbytes) {
+  return RW == 2 && NCH == 2 ? (jbytes == 2 ? 9 : 8) : 1;
+}
 template <int RW, int NCH, int MODE, typename JT>
-__global__ void __launch_bounds__(kRwBlock, RW == 2 ? 9 : 1) k_step_rw(const RwArgs a) {
+__global__ void __launch_bounds__(kRwBlock, (rw_blocks<RW, NCH>(sizeof(JT)))) k_step_rw(const RwArgs a) {
   constexpr int VARIANT = MODE == 3 ? 2 : MODE;
   constexpr bool use_sgn = MODE == 3;
   using P = JPack<RW, JT>;
@@ -206,25 +216,41 @@ __global__ void __launch_bounds__(kRwBlock, RW == 2 ? 9 : 1) k_step_rw(const RwA
       jp = jpn;
     }
 
-    // symplectic Euler: momentum with the old position, then position, then wall
+    // symplectic Euler: momentum with the old position, then position, then wall.
+    // The own values of all rows are asked for before the first store: x is a plain
+    // load (pdl.cuh) that the compiler must keep behind a store that may alias it,
+    // and row by row the second row's latency came on top of the first's (per step,
+    // row by row / now: 39,165 rows, R = 256, factored 55.6 / 54.2 us; 472,812 rows,
+    // R = 128, factored 452 / 439).
+    int row[RW];
+    float c0[RW], hi[RW];
 #pragma unroll
     for (int q = 0; q < RW; ++q) {
-      const int row = __ldg(a.grows + (size_t)grp * RW + q);
-      if (row < 0) continue;
-      const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
-      const float c0 = a.c0_ev[ev];
-      const float hi = __ldg(a.h + row);
+      row[q] = __ldg(a.grows + (size_t)grp * RW + q);
+      const int ev = a.row_event && row[q] >= 0 ? __ldg(a.row_event + row[q]) : 0;
+      c0[q] = a.c0_ev[ev];
+      hi[q] = row[q] >= 0 ? __ldg(a.h + row[q]) : 0.f;
+    }
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const size_t idx = (size_t)row * R + rep0 + 128 * j;
-        const float4 xo = *reinterpret_cast<const float4*>(a.xin + idx);
-        const float4 yo = *reinterpret_cast<const float4*>(a.y + idx);
-        float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
+    for (int j = 0; j < NCH; ++j) {
+      float4 xo[RW], yo[RW];
+#pragma unroll
+      for (int q = 0; q < RW; ++q) {
+        // a group's missing row reads its first one (no predicate: it spills)
+        const size_t idx = (size_t)(row[q] >= 0 ? row[q] : max(row[0], 0)) * R + rep0 + 128 * j;
+        xo[q] = *reinterpret_cast<const float4*>(a.xin + idx);
+        yo[q] = *reinterpret_cast<const float4*>(a.y + idx);
+      }
+#pragma unroll
+      for (int q = 0; q < RW; ++q) {
+        if (row[q] < 0) continue;
+        const size_t idx = (size_t)row[q] * R + rep0 + 128 * j;
+        float xs[4] = {xo[q].x, xo[q].y, xo[q].z, xo[q].w}, ys[4] = {yo[q].x, yo[q].y, yo[q].z, yo[q].w};
         uint32_t sw = 0u;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
           float x = xs[v], y = ys[v];
-          float force = -pa * x + c0 * (acc[q][j][v] + hi);
+          float force = -pa * x + c0[q] * (acc[q][j][v] + hi[q]);
           if (VARIANT == 0) force -= x * x * x;
           y = y + a.dt * force;
           x = x + a.dta0 * y;
