@@ -598,6 +598,17 @@ int32_t padded_replicas(int32_t R) {
   return (int64_t)3 * p <= (int64_t)4 * R ? p : (R + 3) / 4 * 4;
 }
 
+// memory of the context's device, aligned to a bytes: what a kernel may be given
+bool own_memory(const sb_ctx* c, const void* p, size_t a) {
+  cudaPointerAttributes at;
+  if (!p || reinterpret_cast<uintptr_t>(p) % a) return false;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
 sb_status ensure_state(sb_ctx* c, int32_t R) {
   if (c->R == R && c->d_y) return SB_OK;
   free_state(c);
@@ -2978,6 +2989,9 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
     if (ctx->Rs == replicas) {
       SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
       SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
+    } else if (on_device && own_memory(ctx, x, 4) && own_memory(ctx, y, 4)) {
+      SB_CUDA(sbd::launch_repitch(x, replicas, ctx->d_x[0], ctx->Rs, ctx->n, replicas, 0));
+      SB_CUDA(sbd::launch_repitch(y, replicas, ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
     } else {  // through the second x buffer, then into the padded rows
       for (int q = 0; q < 2; ++q) {
         SB_CUDA(cudaMemcpy(ctx->d_x[1], q ? y : x, bytes, k));
@@ -3009,6 +3023,10 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
     float* const out = q ? y : x;
     const float* src = q ? ctx->d_y : ctx->d_x[ctx->cur];
     if (!out) continue;
+    if (ctx->Rs != ctx->R && on_device && own_memory(ctx, out, 4)) {
+      SB_CUDA(sbd::launch_repitch(src, ctx->Rs, out, ctx->R, ctx->n, ctx->R, 0));
+      continue;
+    }
     if (ctx->Rs != ctx->R) {  // padded rows: gathered in the other x buffer first
       float* const tmp = ctx->d_x[ctx->cur ^ 1];
       SB_CUDA(sbd::launch_repitch(src, ctx->Rs, tmp, ctx->R, ctx->n, ctx->R, 0));
@@ -3062,15 +3080,7 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
     // the kernels write the caller's buffers themselves where they are aligned
     // for their type and lie on the context's own device, else through the
     // context's own and a copy (which refuses what is no device memory)
-    auto direct = [&](void* p, size_t a) {
-      cudaPointerAttributes at;
-      if (!p || reinterpret_cast<uintptr_t>(p) % a) return false;
-      if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-      }
-      return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
-    };
+    auto direct = [&](void* p, size_t a) { return own_memory(ctx, p, a); };
     const bool dE = direct(d_E_all, 8), db = direct(d_best_E, 8), dr = direct(d_best_r, 4);
     sb_status st = readout(ctx, nullptr, ctx->R, s, dE ? d_E_all : nullptr,
                            db ? d_best_E : nullptr, dr ? d_best_r : nullptr);
