@@ -261,6 +261,8 @@ struct sb_ctx {
     size_t smem = 0;
     sbd::Run1Cta* d_cta = nullptr;
     int32_t *d_perm = nullptr, *d_deg = nullptr, *d_slice = nullptr, *d_ucol = nullptr;
+    int64_t ents = 0;            // entries, padding included
+    int32_t* d_pos = nullptr;    // CSR position of each entry (-1: padding)
     float* d_ej = nullptr;
     uint16_t* d_ei = nullptr;
     unsigned long long* d_word = nullptr;
@@ -448,6 +450,7 @@ void free_run1(sb_ctx* c) {
   dfree(r.d_deg);
   dfree(r.d_slice);
   dfree(r.d_ucol);
+  dfree(r.d_pos);
   dfree(r.d_ej);
   dfree(r.d_ei);
   dfree(r.d_word);
@@ -1919,6 +1922,16 @@ sbd::Tiling step_tiling(const sb_ctx* c) {
   return sbd::make_tiling(c->Rs);
 }
 
+// The entries of k_run_r1's tables from the current J, in place: a run that a caller
+// has recorded keeps its addresses and takes the new couplings, as the step
+// kernels do, which read J itself.
+sb_status refill_run1(sb_ctx* c) {
+  if (c->run1.built <= 0) return SB_OK;
+  SB_CUDA(sbd::launch_fill_run1(c->d_J, c->jbf16, c->run1.d_pos, c->run1.ents, c->run1.d_ej, 0));
+  SB_CUDA(cudaStreamSynchronize(0));
+  return SB_OK;
+}
+
 // Tables of k_run_r1: rows in contiguous chunks of about equal cost (nonzeros
 // plus a share per row), one per CTA; inside a chunk by decreasing degree, in
 // slices of 32 whose entries are padded to the slice's longest row (a multiple
@@ -1955,12 +1968,8 @@ sb_status ensure_run1(sb_ctx* c) {
                        std::min(at, lo + sbd::kRun1Threads));
   }
   if (n - row0[nct - 1] > sbd::kRun1Threads) return SB_OK;
-  const size_t esz = c->jbf16 ? 2 : 4;
-  std::vector<unsigned char> jraw((size_t)nnz * esz);
-  if (nnz) SB_CUDA(cudaMemcpy(jraw.data(), c->d_J, jraw.size(), cudaMemcpyDeviceToHost));
   struct Part {
-    std::vector<int32_t> perm, deg, slice, ucol;
-    std::vector<float> ej;
+    std::vector<int32_t> perm, deg, slice, ucol, pos;
     std::vector<uint16_t> ei;
     bool ok = true;
   };
@@ -1985,19 +1994,17 @@ sb_status ensure_run1(sb_ctx* c) {
       for (size_t u = 0; u < q.ucol.size(); ++u) local[q.ucol[u]] = (int32_t)u;
       for (int32_t s = 0; s < r1 - r0; s += 32) {
         const int32_t len = (rp[q.perm[s] + 1] - rp[q.perm[s]] + 7) / 8 * 8;
-        const size_t e0 = q.ej.size();
+        const size_t e0 = q.pos.size();
         q.slice.push_back((int32_t)e0);
-        q.ej.resize(e0 + (size_t)len * 32, 0.f);
+        q.pos.resize(e0 + (size_t)len * 32, -1);
         q.ei.resize(e0 + (size_t)len * 32, 0);
         for (int32_t l = 0; l < 32 && s + l < r1 - r0; ++l) {
           const int32_t row = q.perm[s + l], d = rp[row + 1] - rp[row];
           q.deg.push_back(d);
           for (int32_t k = 0; k < d; ++k) {
-            const size_t p = (size_t)rp[row] + k, e = e0 + (size_t)(k / 4) * 128 + 4 * l + k % 4;
-            uint32_t bits = 0;
-            memcpy(&bits, jraw.data() + p * esz, esz);
-            if (esz == 2) bits <<= 16;
-            memcpy(&q.ej[e], &bits, 4);
+            const int32_t p = rp[row] + k;
+            const size_t e = e0 + (size_t)(k / 4) * 128 + 4 * l + k % 4;
+            q.pos[e] = p;
             q.ei[e] = (uint16_t)local[col[p]];
           }
         }
@@ -2013,10 +2020,10 @@ sb_status ensure_run1(sb_ctx* c) {
   for (int32_t b = 0; b < nct; ++b) {
     const Part& q = P[(size_t)b];
     ok = ok && q.ok;
-    cta[b] = {row0[b], row0[b + 1] - row0[b], (int32_t)ents, (int32_t)q.ej.size(),
+    cta[b] = {row0[b], row0[b + 1] - row0[b], (int32_t)ents, (int32_t)q.pos.size(),
               (int32_t)slice.size(), (int32_t)ucol.size(), (int32_t)q.ucol.size(), 0};
-    ents += q.ej.size();
-    max_ent = std::max(max_ent, q.ej.size());
+    ents += q.pos.size();
+    max_ent = std::max(max_ent, q.pos.size());
     max_u = std::max(max_u, q.ucol.size());
     perm.insert(perm.end(), q.perm.begin(), q.perm.end());
     deg.insert(deg.end(), q.deg.begin(), q.deg.end());
@@ -2028,11 +2035,11 @@ sb_status ensure_run1(sb_ctx* c) {
   if (!ok || ents > (size_t)INT32_MAX || smem > (size_t)sbd::kRun1Smem ||
       sbd::run1_blocks_per_sm(smem) < 1)
     return SB_OK;
-  std::vector<float> ej(std::max<size_t>(ents, 4));
+  std::vector<int32_t> pos(std::max<size_t>(ents, 4), -1);
   std::vector<uint16_t> ei(std::max<size_t>(ents, 4));
   parallel_parts(nct, parts, [&](int, int64_t b0, int64_t b1) {
     for (int64_t b = b0; b < b1; ++b) {
-      std::copy(P[b].ej.begin(), P[b].ej.end(), ej.begin() + cta[b].ent0);
+      std::copy(P[b].pos.begin(), P[b].pos.end(), pos.begin() + cta[b].ent0);
       std::copy(P[b].ei.begin(), P[b].ei.end(), ei.begin() + cta[b].ent0);
     }
   }, 1);
@@ -2043,8 +2050,8 @@ sb_status ensure_run1(sb_ctx* c) {
   }
   if (dalloc(&r.d_perm, perm.size()) || dalloc(&r.d_deg, deg.size()) ||
       dalloc(&r.d_slice, std::max<size_t>(slice.size(), 1)) ||
-      dalloc(&r.d_ucol, std::max<size_t>(ucol.size(), 1)) || dalloc(&r.d_ej, ej.size()) ||
-      dalloc(&r.d_ei, ei.size()) || dalloc(&r.d_word, (size_t)2 * n)) {
+      dalloc(&r.d_ucol, std::max<size_t>(ucol.size(), 1)) || dalloc(&r.d_ej, pos.size()) ||
+      dalloc(&r.d_pos, pos.size()) || dalloc(&r.d_ei, ei.size()) || dalloc(&r.d_word, (size_t)2 * n)) {
     free_run1(c);
     r.built = -1;
     return SB_OK;
@@ -2055,14 +2062,17 @@ sb_status ensure_run1(sb_ctx* c) {
   SB_CUDA(cudaMemcpy(r.d_slice, slice.data(), slice.size() * 4, cudaMemcpyHostToDevice));
   if (!ucol.empty())
     SB_CUDA(cudaMemcpy(r.d_ucol, ucol.data(), ucol.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_ej, ej.data(), ej.size() * 4, cudaMemcpyHostToDevice));
+  SB_CUDA(cudaMemcpy(r.d_pos, pos.data(), pos.size() * 4, cudaMemcpyHostToDevice));
   SB_CUDA(cudaMemcpy(r.d_ei, ei.data(), ei.size() * 2, cudaMemcpyHostToDevice));
   r.nct = nct;
   r.nx = nx;
   r.max_ent = (int32_t)max_ent;
   r.smem = smem;
+  r.ents = (int64_t)pos.size();
   r.built = 1;
-  return SB_OK;
+  const sb_status st = refill_run1(c);
+  if (st) r.built = -1;
+  return st;
 }
 
 sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
@@ -3199,7 +3209,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     ctx->d_tz = nullptr;
     ctx->graph.reset();
     if (ctx->tiles_built && (st = setup_tiles(ctx, rp, col))) return st;
-    free_run1(ctx);  // its tables carry J
+    if ((st = refill_run1(ctx))) return st;  // its tables carry J
     // the row-group kernel's entries carry J too
     if ((st = refill_rw(ctx))) return st;
     // the factored form's weight and residual were formed for the old couplings

@@ -291,6 +291,9 @@ struct Run1Args {
 };
 cudaError_t run1_prepare();  // raise the kernels' shared-memory limit (once per device)
 int run1_blocks_per_sm(size_t smem);  // resident CTAs per SM (0: it does not fit)
+// ej[e] = J[pos[e]] (0 where pos[e] < 0)
+cudaError_t launch_fill_run1(const void* J, int jbf16, const int32_t* pos, int64_t count, float* ej,
+                             cudaStream_t s);
 cudaError_t launch_run_r1(int variant, const Run1Args& a, size_t smem, cudaStream_t s);
 
 // ---------------------------------------------------------------- factored step

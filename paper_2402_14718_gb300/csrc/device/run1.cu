@@ -26,6 +26,8 @@
 // rows 6.5 / 2.4. A cluster of 16 CTAs that wrote its positions into each other's
 // shared memory took 1.45 us for 1,721 rows with the cluster's barrier, 2.9 us for
 // 10,214 rows, and 5 to 9 us when its threads polled shared memory instead.
+#include <cuda_bf16.h>
+
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -186,6 +188,15 @@ __global__ void __launch_bounds__(kRun1Threads, 1) k_run_r1(const Run1Args a) {
   }
 }
 
+template <typename JT>
+__global__ void k_fill_run1(const JT* J, const int32_t* pos, int64_t count, float* ej) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t p = pos[i];
+    ej[i] = p >= 0 ? (float)J[p] : 0.f;
+  }
+}
+
 template <int VARIANT>
 cudaError_t launch_t(const Run1Args& a, size_t smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
@@ -219,6 +230,17 @@ int run1_blocks_per_sm(size_t smem) {
     return 0;
   }
   return n;
+}
+
+cudaError_t launch_fill_run1(const void* J, int jbf16, const int32_t* pos, int64_t count, float* ej,
+                             cudaStream_t s) {
+  if (count <= 0) return cudaSuccess;
+  const int grid = (int)std::min<int64_t>((count + 255) / 256, 4096);
+  if (jbf16)
+    k_fill_run1<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(J), pos, count, ej);
+  else
+    k_fill_run1<<<grid, 256, 0, s>>>(static_cast<const float*>(J), pos, count, ej);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_run_r1(int variant, const Run1Args& a, size_t smem, cudaStream_t s) {
