@@ -3169,6 +3169,12 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
           (st = dalloc(&ctx->d_nconf, (size_t)n)))
         return st;
     }
+    double *row_off = nullptr, *row_sq = nullptr;
+    if ((st = dalloc(&row_off, (size_t)n)) || (st = dalloc(&row_sq, (size_t)n))) {
+      dfree(row_off);
+      dfree(row_sq);
+      return st;
+    }
     SB_CUDA(cudaDeviceSynchronize());
     if (ctx->nnz) {
       SB_CUDA(cudaMemcpy(ctx->d_cls, cls, (size_t)ctx->nnz, cudaMemcpyHostToDevice));
@@ -3178,12 +3184,6 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     SB_CUDA(cudaMemcpy(ctx->d_nconf, nconf.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
     SB_CUDA(cudaMemcpy(ctx->d_qlin, ql.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
     SB_CUDA(cudaMemset(ctx->d_inexact, 0, sizeof(int)));
-    double *row_off = nullptr, *row_sq = nullptr;
-    if ((st = dalloc(&row_off, (size_t)n)) || (st = dalloc(&row_sq, (size_t)n))) {
-      dfree(row_off);
-      dfree(row_sq);
-      return st;
-    }
     cudaError_t e1 = sbd::launch_convert(ctx->d_rowptr, ctx->d_col, ctx->d_qval, ctx->d_qlin, n,
                                          ctx->d_J, ctx->jbf16, ctx->d_h64, ctx->d_h32, row_off,
                                          row_sq, ctx->d_inexact, 0);
@@ -3195,6 +3195,14 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     SB_CUDA(e1);
     SB_CUDA(e2);
     SB_CUDA(e3);
+    // J is new: what holds copies of it comes before anything that can run out
+    // of memory, so that no table of old couplings outlives an error below
+    ctx->graph.reset();
+    ctx->have_classes = true;
+    // the factored form's weight and residual were formed for the old couplings
+    free_factor(ctx);
+    if ((st = refill_rw(ctx))) return st;
+    if ((st = refill_run1(ctx))) return st;
     SB_CUDA(cudaMemcpy(ctx->offset.data(), ctx->d_offset, 8, cudaMemcpyDeviceToHost));
     SB_CUDA(cudaMemcpy(ctx->sigma.data(), ctx->d_sigma, 8, cudaMemcpyDeviceToHost));
     SB_CUDA(cudaMemcpy(ctx->c0_auto.data(), ctx->d_c0auto, 8, cudaMemcpyDeviceToHost));
@@ -3207,14 +3215,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     dfree(ctx->d_own);
     if (ctx->d_tz) cudaFree(ctx->d_tz);
     ctx->d_tz = nullptr;
-    ctx->graph.reset();
     if (ctx->tiles_built && (st = setup_tiles(ctx, rp, col))) return st;
-    if ((st = refill_run1(ctx))) return st;  // its tables carry J
-    // the row-group kernel's entries carry J too
-    if ((st = refill_rw(ctx))) return st;
-    // the factored form's weight and residual were formed for the old couplings
-    free_factor(ctx);
-    ctx->have_classes = true;
     return SB_OK;
   });
 }
