@@ -234,6 +234,11 @@ int32_t sb_total_rows(const sb_ctx* ctx);
  * on-chip gather is union_entries x R x 4 bytes). Either pointer may be NULL. */
 sb_status sb_step_info(const sb_ctx* ctx, int32_t* rows_per_warp, int64_t* union_entries);
 
+/* Names of the kernels that the last sb_run, sb_advance or sb_autotune of the
+ * context launched (or recorded) for its steps, in launch order and joined by
+ * " + "; "" before the first step. A string literal of the library. */
+const char* sb_step_kernels(const sb_ctx* ctx);
+
 /*
  * sb_set_factor -- factored form of the coupling product of Eq. 2 / 6 / 10 for
  * QUBOs in which one weight w is shared by whole groups of rows (Eq. 13: every

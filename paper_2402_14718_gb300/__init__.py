@@ -25,7 +25,8 @@ __all__ = [
     "SB_ERR_BOUNDS", "SbError", "sb_checked_build", "sb_check_bounds", "decode_bounds",
     "event_params", "build_params", "sb_event_generate", "sb_qubo_build", "sb_tracks",
     "sb_qubo_build_device", "sb_qubo_factor", "sb_set_factor", "sb_factor_info",
-    "sb_create", "sb_create_batch", "sb_destroy", "sb_info", "sb_step_info", "sb_gather_probe",
+    "sb_create", "sb_create_batch", "sb_destroy", "sb_info", "sb_step_info", "sb_step_kernels",
+    "sb_gather_probe",
     "sb_run", "sb_advance",
     "sb_set_state", "sb_get_state", "sb_energy", "sb_best", "sb_readout_device", "sb_set_option",
     "sb_energy_noalloc", "sb_autotune", "sb_set_weights", "sb_backward", "SBRelaxedEnergy",
@@ -323,6 +324,11 @@ def sb_step_info(ctx):
     ent = ctypes.c_int64()
     check(lib.sb_step_info(ctx.handle, ctypes.byref(rw), ctypes.byref(ent)))
     return rw.value, ent.value
+
+
+def sb_step_kernels(ctx):
+    """Names of the kernels that the last steps of the context ran (see include/sb.h)."""
+    return lib.sb_step_kernels(ctx.handle).decode()
 
 
 def sb_gather_probe(array_bytes, row_bytes, repeats=5, seed=1, stream=None):

@@ -89,6 +89,7 @@ _SIGS = {
                                   c_void_p, c_int32, P(c_void_p)]),
     "sb_destroy": (None, [c_void_p]),
     "sb_step_info": (c_int32, [c_void_p, P(c_int32), P(c_int64)]),
+    "sb_step_kernels": (c_char_p, [c_void_p]),
     "sb_gather_probe": (c_int32, [c_int64, c_int32, c_int32, c_uint64, P(c_double), c_void_p]),
     "sb_info": (c_int32, [c_void_p, c_int32, P(c_int32), P(c_int64), P(c_double), P(c_double),
                           P(c_double)]),

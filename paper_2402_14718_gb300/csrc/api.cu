@@ -116,6 +116,7 @@ struct sb_ctx {
   float* d_x[2] = {nullptr, nullptr};
   float* d_y = nullptr;
   int cur = 0;
+  const char* step_kernels = "";  // kernels of the last steps (sb_step_kernels)
   bool have_state = false;
   float* d_sched = nullptr;  // default linear schedule
   int32_t sched_len = 0;
@@ -2124,6 +2125,7 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
       ua.err = c->d_err;
       ua.wait_ns = 2000000000ull;
       SB_CUDA(sbd::launch_run_r1(variant, ua, r.smem, stream));
+      c->step_kernels = "k_run_r1";
       if (steps & 1) c->cur ^= 1;
       return SB_OK;
     }
@@ -2522,6 +2524,16 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
     a.tile0 = 0;
     return err;
   };
+  c->step_kernels = fac        ? (variant == SB_DSB ? "k_fac_sum_sgn + k_step_fac_sgn"
+                                  : frw             ? "k_fac_sum + k_step_rw"
+                                                    : "k_fac_sum + k_step_fac")
+                    : streamed ? "k_step_stream"
+                    : rw       ? "k_step_rw"
+                    : tiled    ? "k_step_tiled"
+                    : dsb16    ? "k_step_dsb16"
+                    : c->R > 1 || a.rpc != 256 / t.G ? "k_step"
+                    : a.r1_lanes                     ? "k_step_r1g"
+                                                     : "k_step_r1";
   std::vector<int64_t> key;
   if (c->use_graph && steps >= 8) {
     int32_t a0b = 0, dtb = 0;
@@ -2825,6 +2837,8 @@ sb_status sb_step_info(const sb_ctx* ctx, int32_t* rows_per_warp, int64_t* union
   if (union_entries) *union_entries = ctx->rw_built ? ctx->rw_E : 0;
   return SB_OK;
 }
+
+const char* sb_step_kernels(const sb_ctx* ctx) { return ctx ? ctx->step_kernels : ""; }
 
 sb_status sb_set_factor(sb_ctx* ctx, int32_t n_ids, int32_t k, const int32_t* member,
                         const uint8_t* couple, double w) {
