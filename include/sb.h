@@ -507,19 +507,23 @@ sb_status sb_energy_noalloc(int32_t n, const int32_t* rowptr, const int32_t* col
  * does (same states). 0: one thread per row. -1 (default): the widest group
  * for which rows x lanes fit in the SMs' resident threads, else 0; and runs of 16
  * steps or more whose couplings fit in the SMs' shared memory take one launch
- * for all steps (same states; its waits are bounded by 2 s, after which the next
- * synchronising call returns SB_ERR_TIMEOUT). */
+ * for all steps (same states; its waits are bounded by SB_OPT_WAIT_NS, after
+ * which the next synchronising call returns SB_ERR_TIMEOUT, as for
+ * SB_OPT_STREAM). */
 #define SB_OPT_R1_LANES 11
 /* SB_OPT_WAIT_NS (12): limit, in nanoseconds of the GPU's global timer, of
  * every wait of the streamed step kernel (SB_OPT_STREAM) on its shared-memory
- * pipeline; 2e9 (2 s) by default, accepted in [1e3, 6e10]. */
+ * pipeline and of the one-launch run of one replica (SB_OPT_R1_LANES) on its
+ * neighbours' positions; 2e9 (2 s) by default, accepted in [1e3, 6e10]. */
 #define SB_OPT_WAIT_NS 12
 /* SB_OPT_TEST_SKIP_STAGE (13): test hook of the time-out path of the streamed
  * step kernel. A stage index s >= 0 makes the producer warp of CTA 0 leave
  * its s-th ring stage unissued (no barrier arrival, no copy started), so the
  * consumer warps' wait for that stage runs out after SB_OPT_WAIT_NS, they
  * record the time-out and return, and the producer drains its copies in
- * flight with a bound and returns. -1 (default) turns it off. Nothing
+ * flight with a bound and returns. In the one-launch run of one replica, step
+ * s leaves the position of CTA 0's first row unpublished, so that its
+ * neighbours' waits run out. -1 (default) turns it off. Nothing
  * faults or hangs either way: every wait is bounded. */
 #define SB_OPT_TEST_SKIP_STAGE 13
 /* SB_OPT_FACTOR (14): -1 (default) or 1 runs the factored coupling product

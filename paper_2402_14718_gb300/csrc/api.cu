@@ -182,7 +182,7 @@ struct sb_ctx {
   uint32_t* d_s_umask = nullptr;
   int* d_err = nullptr;  // set by a kernel whose bounded wait gave up
   unsigned long long wait_ns = 2000000000ull;  // limit of the streamed kernel's waits
-  int32_t skip_stage = -1;  // test hook of the streamed kernel (SB_OPT_TEST_SKIP_STAGE)
+  int32_t skip_stage = -1;  // test hook of the bounded waits (SB_OPT_TEST_SKIP_STAGE)
   // row-group step kernel (k_step_rw): groups of RW rows and their union entries
   int rw_rows = -1;      // -1: automatic (2 for aSB / bSB, off for dSB); 0: off; 2 or 4
   // dispatch the row-group CTAs heaviest chunk first: 1 on, 0 off, -1 when
@@ -1193,8 +1193,11 @@ sb_status check_wait_flag(const sb_ctx* c) {
   SB_CUDA(cudaMemcpy(&v, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (v) {
     SB_CUDA(cudaMemset(c->d_err, 0, sizeof(int)));
-    set_error("a step kernel gave up waiting for its shared-memory pipeline (code " +
-              std::to_string(v) + "); the state of that run is not valid");
+    set_error(v == sbd::kRun1Late
+                  ? "a one-replica run gave up waiting for a neighbour's position; the state of "
+                    "that run is not valid"
+                  : "a step kernel gave up waiting for its shared-memory pipeline (code " +
+                        std::to_string(v) + "); the state of that run is not valid");
     return SB_ERR_TIMEOUT;
   }
   return SB_OK;
@@ -2123,7 +2126,8 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
       ua.y = c->d_y;
       ua.word = r.d_word;
       ua.err = c->d_err;
-      ua.wait_ns = 2000000000ull;
+      ua.wait_ns = c->wait_ns;
+      ua.skip_step = c->skip_stage;
       SB_CUDA(sbd::launch_run_r1(variant, ua, r.smem, stream));
       c->step_kernels = "k_run_r1";
       if (steps & 1) c->cur ^= 1;

@@ -261,6 +261,7 @@ struct StreamArgs {
 // k_run_r1 (run1.cu): every step of a one-replica run in one launch.
 constexpr int kRun1Threads = 1024;         // one row per thread
 constexpr int kRun1Smem = 220 * 1024;      // dynamic shared memory limit
+constexpr int kRun1Late = 4;               // code of a wait that gave up (1 .. 3: streamed kernel)
 struct Run1Cta {
   int32_t row0, nrows;   // rows [row0, row0 + nrows), nrows <= kRun1Threads
   int32_t ent0, nent;    // entries (a multiple of 256) in ej / ei
@@ -286,8 +287,9 @@ struct Run1Args {
   float* x[2];
   float* y;
   unsigned long long* word;  // [2 n] {position, step} (zeroed by the launch)
-  int* err;              // set when a wait gives up
+  int* err;              // kRun1Late when a wait gives up
   unsigned long long wait_ns;
+  int32_t skip_step;     // test hook: this step's first word is not published (-1: none)
 };
 cudaError_t run1_prepare();  // raise the kernels' shared-memory limit (once per device)
 int run1_blocks_per_sm(size_t smem);  // resident CTAs per SM (0: it does not fit)

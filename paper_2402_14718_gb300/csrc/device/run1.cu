@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kRun1Threads, 1) k_run_r1(const Run1Args a) {
   if (own) r.load(a, c, t);
   const float4* const w4 = reinterpret_cast<const float4*>(wj) + r.base;
   const ushort4* const i4 = reinterpret_cast<const ushort4*>(wi) + r.base;
+  const int mute = blockIdx.x == 0 && t == 0 ? a.skip_step : -1;
   for (int k = 0; k < a.steps; ++k) {
     const float pa = a.a0 - __ldg(a.sched + k);
     bool late = false;
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kRun1Threads, 1) k_run_r1(const Run1Args a) {
       }
     }
     if (__syncthreads_or(late)) {
-      if (t == 0) *a.err = 2;
+      if (t == 0) *a.err = kRun1Late;
       return;
     }
     if (own) {
@@ -175,7 +176,8 @@ __global__ void __launch_bounds__(kRun1Threads, 1) k_run_r1(const Run1Args a) {
         }
       }
       update_row<VARIANT>(a, pa, r.c0, r.h, acc, r.x, r.y);
-      st_word(a.word + (size_t)((k + 1) & 1) * a.n + r.row, pack_word(r.x, (uint32_t)(k + 1)));
+      if (k != mute)
+        st_word(a.word + (size_t)((k + 1) & 1) * a.n + r.row, pack_word(r.x, (uint32_t)(k + 1)));
     }
     // every row of this CTA has read xs. (Two copies of xs without this barrier
     // let the threads without a row poll while the others still compute: 4.2
