@@ -351,6 +351,8 @@ sb_status sb_best(sb_ctx* ctx, uint8_t* out_T, double* out_E, int32_t* out_repli
 /*
  * sb_readout_device -- sb_best with device outputs, asynchronous on `stream`:
  * d_E_all[E x R] (may be NULL), d_best_E[E], d_best_r[E], d_T[N] (may be NULL).
+ * After a run whose bounded wait gave up (SB_OPT_WAIT_NS) every energy is NaN,
+ * until a synchronising call has returned SB_ERR_TIMEOUT.
  */
 sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int32_t* d_best_r,
                             uint8_t* d_T, void* stream);

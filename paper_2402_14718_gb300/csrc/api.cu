@@ -2614,6 +2614,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   if (!E_all) E_all = c->d_Eall;
   if (!best_E) best_E = c->d_bestE;
   if (!best_r) best_r = c->d_bestr;
+  const int* const err = d_spins ? nullptr : c->d_err;
   if (c->b_whole) {
     sbd::EnergyBitArgs b;
     b.rowptr = c->d_rowptr;
@@ -2633,7 +2634,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
                                     c->d_bits, s));
     SB_CUDA(sbd::launch_energy_bits(b, s));
     SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
-    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, s));
+    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
     return SB_OK;
   }
   const sbd::Tiling t = sbd::make_tiling(R);
@@ -2654,7 +2655,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   a.nnz = c->nnz;
   SB_CUDA(sbd::launch_energy_partial(t, a, s));
   SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
-  SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, s));
+  SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
   return SB_OK;
 }
 

@@ -1446,11 +1446,15 @@ __device__ __forceinline__ bool better(double v, int r, double bv, int br) {
   return v < bv || (v == bv && r < br);
 }
 
-// warp-shuffle arg-min over the replicas of one event
-__global__ void k_argmin(const double* E_all, int32_t R, double* best_E, int32_t* best_r) {
+// warp-shuffle arg-min over the replicas of one event. *err (may be NULL) is the
+// flag that a step kernel sets when one of its bounded waits gave up: the state is
+// not valid then, and every energy becomes NaN.
+__global__ void k_argmin(double* E_all, int32_t R, double* best_E, int32_t* best_r, const int* err) {
   __shared__ double sv[32];
   __shared__ int sr[32];
   const int e = blockIdx.x;
+  const bool bad = err && *err;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
   double bv = DBL_MAX;
   int br = INT_MAX;
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
@@ -1487,10 +1491,12 @@ __global__ void k_argmin(const double* E_all, int32_t R, double* best_E, int32_t
       }
     }
     if (lane == 0) {
-      best_E[e] = bv;
+      best_E[e] = bad ? nan : bv;
       best_r[e] = br == INT_MAX ? 0 : br;
     }
   }
+  if (bad)
+    for (int r = threadIdx.x; r < R; r += blockDim.x) E_all[(size_t)e * R + r] = nan;
 }
 
 __global__ void k_best_T(const float* x, const int32_t* row_event, const int32_t* best_r,
@@ -1763,10 +1769,10 @@ cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_argmin(const double* E_all, int32_t E, int32_t R, double* best_E,
-                          int32_t* best_r, cudaStream_t s) {
+cudaError_t launch_argmin(double* E_all, int32_t E, int32_t R, double* best_E, int32_t* best_r,
+                          const int* err, cudaStream_t s) {
   if (E <= 0) return cudaSuccess;
-  k_argmin<<<E, kBlock, 0, s>>>(E_all, R, best_E, best_r);
+  k_argmin<<<E, kBlock, 0, s>>>(E_all, R, best_E, best_r, err);
   return cudaGetLastError();
 }
 

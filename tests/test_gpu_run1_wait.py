@@ -32,3 +32,34 @@ def test_wait_runs_out(n, step):
     again = run1._run(ctx, "bsb", 40, -1)
     assert sb.sb_step_kernels(ctx) == "k_run_r1"
     assert np.array_equal(again[0], good[0]) and np.array_equal(again[1], good[1])
+
+
+@pytest.mark.parametrize("whole", [True, False])
+def test_asynchronous_readout_of_a_run_that_gave_up(whole):
+    """No host call has looked at the run when its energies are read: they are NaN."""
+    import torch
+    n = 700
+    rowptr, col, val, lin = run1._sparse(n, 12, 3)
+    ctx = sb.sb_create(n, rowptr, col, np.sign(val) if whole else val, lin, sb.SB_J_FP32)
+    for _ in range(50):
+        run1._run(ctx, "bsb", 40, -1)
+    E, b = (torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    r = torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    T = torch.zeros(n, dtype=torch.uint8, device="cuda")
+
+    def read(step):
+        sb.sb_set_option(ctx, sb.SB_OPT_TEST_SKIP_STAGE, step)
+        sb.sb_set_option(ctx, sb.SB_OPT_WAIT_NS, 1_000_000 if step >= 0 else 2_000_000_000)
+        sb.sb_run(ctx, "bsb", 1.0, 0.4, 0.3, 40, 1, seed=7)
+        assert sb.sb_step_kernels(ctx) == "k_run_r1"
+        sb.sb_readout_device(ctx, E, b, r, T)
+        torch.cuda.synchronize()
+        return E.item(), b.item(), r.item()
+
+    good = read(-1)
+    assert np.isfinite(good[0]) and good[:1] == good[1:2] and good[2] == 0
+    late = read(3)
+    assert np.isnan(late[0]) and np.isnan(late[1]) and late[2] == 0
+    with pytest.raises(sb.SbError, match="neighbour's position"):
+        sb.sb_best(ctx)
+    assert read(-1) == good
