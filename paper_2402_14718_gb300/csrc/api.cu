@@ -3027,8 +3027,10 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
         SB_CUDA(sbd::launch_repitch(ctx->d_x[1], replicas, q ? ctx->d_y : ctx->d_x[0], ctx->Rs,
                                     ctx->n, replicas, 0));
       }
-      SB_CUDA(cudaDeviceSynchronize());
     }
+    // neither a device copy nor a kernel has finished when its call returns, and a
+    // stream of the caller's need not wait for the default stream
+    SB_CUDA(cudaStreamSynchronize(0));
     ctx->have_state = true;
     return SB_OK;
   });
@@ -3063,6 +3065,7 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
     }
     SB_CUDA(cudaMemcpy(out, src, bytes, k));
   }
+  SB_CUDA(cudaStreamSynchronize(0));  // as in sb_set_state
   return SB_OK;
 }
 

@@ -1,0 +1,49 @@
+"""States passed in and out of device memory beside a stream that does not wait for
+the default stream: sb_set_state and sb_get_state have finished when they
+return, so the next call on any stream sees the whole state."""
+import numpy as np
+import pytest
+
+import paper_2402_14718_gb300 as sb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("R", [50, 64, 99])
+def test_set_advance_get_on_a_side_stream(R):
+    """A ring of 400,000 rows: copying the state takes longer than starting a step."""
+    import torch
+    n = 400000
+    i = np.arange(n)
+    col = np.sort((i[:, None] + np.array([-7, -1, 1, 7])) % n, axis=1).ravel().astype(np.int32)
+    ctx = sb.sb_create(n, (4 * np.arange(n + 1)).astype(np.int32), col, np.ones(4 * n),
+                       np.full(n, 0.3))
+    g = torch.Generator(device="cuda").manual_seed(R)
+    x = 2 * torch.rand((n, R), generator=g, device="cuda") - 1
+    y = 0.6 * torch.rand((n, R), generator=g, device="cuda") - 0.3
+    sched = torch.linspace(0.2, 0.6, 2, device="cuda")
+    side = torch.cuda.Stream()
+    out = [torch.empty_like(x) for _ in range(4)]
+
+    def get(a, b):
+        sb._lib.check(sb.lib.sb_get_state(ctx.handle, a.data_ptr(), b.data_ptr(), 1))
+
+    def two_runs(wait):
+        res = []
+        sb.sb_set_state(ctx, x, y)
+        for k in (0, 2):
+            wait()
+            sb.sb_advance(ctx, "bsb", 1.0, 0.3, 0.4, 2, sched, stream=side)
+            wait()
+            get(out[k], out[k + 1])
+            wait()
+            with torch.cuda.stream(side):  # reads the copy, then the next run overwrites the state
+                res += [out[k].clone(), out[k + 1].clone()]
+        torch.cuda.synchronize()
+        return res
+
+    want = two_runs(torch.cuda.synchronize)
+    assert not torch.equal(want[0], want[2])
+    for _ in range(5):
+        got = two_runs(lambda: None)
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
