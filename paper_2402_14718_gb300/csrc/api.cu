@@ -2583,8 +2583,8 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
 sb_status unpad_state(sb_ctx* c, cudaStream_t stream) {
   float *const x = c->d_x[c->cur], *const other = c->d_x[c->cur ^ 1];
   const size_t bytes = (size_t)c->n * c->R * sizeof(float);
-  SB_CUDA(sbd::launch_repitch(x, c->Rs, other, c->R, c->n, c->R, stream));
-  SB_CUDA(sbd::launch_repitch(c->d_y, c->Rs, x, c->R, c->n, c->R, stream));
+  SB_CUDA(sbd::launch_repitch(x, nullptr, c->Rs, other, nullptr, c->R, c->n, c->R, stream));
+  SB_CUDA(sbd::launch_repitch(c->d_y, nullptr, c->Rs, x, nullptr, c->R, c->n, c->R, stream));
   SB_CUDA(cudaMemcpyAsync(c->d_y, x, bytes, cudaMemcpyDeviceToDevice, stream));
   c->cur ^= 1;
   c->Rs = c->R;
@@ -3019,14 +3019,14 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
       SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
       SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
     } else if (on_device && own_memory(ctx, x, 4) && own_memory(ctx, y, 4)) {
-      SB_CUDA(sbd::launch_repitch(x, replicas, ctx->d_x[0], ctx->Rs, ctx->n, replicas, 0));
-      SB_CUDA(sbd::launch_repitch(y, replicas, ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
-    } else {  // through the second x buffer, then into the padded rows
-      for (int q = 0; q < 2; ++q) {
-        SB_CUDA(cudaMemcpy(ctx->d_x[1], q ? y : x, bytes, k));
-        SB_CUDA(sbd::launch_repitch(ctx->d_x[1], replicas, q ? ctx->d_y : ctx->d_x[0], ctx->Rs,
-                                    ctx->n, replicas, 0));
-      }
+      SB_CUDA(sbd::launch_repitch(x, y, replicas, ctx->d_x[0], ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
+    } else {  // both through the x buffers, then into the padded rows
+      SB_CUDA(cudaMemcpy(ctx->d_x[0], y, bytes, k));
+      SB_CUDA(cudaMemcpy(ctx->d_x[1], x, bytes, k));
+      SB_CUDA(sbd::launch_repitch(ctx->d_x[0], nullptr, replicas, ctx->d_y, nullptr, ctx->Rs, ctx->n,
+                                  replicas, 0));
+      SB_CUDA(sbd::launch_repitch(ctx->d_x[1], nullptr, replicas, ctx->d_x[0], nullptr, ctx->Rs, ctx->n,
+                                  replicas, 0));
     }
     // neither a device copy nor a kernel has finished when its call returns, and a
     // stream of the caller's need not wait for the default stream
@@ -3048,25 +3048,27 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
   const size_t bytes = (size_t)ctx->n * ctx->R * 4;
   const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   SB_CUDA(cudaDeviceSynchronize());
-  sb_status st = check_wait_flag(ctx);
-  if (st) return st;
-  for (int q = 0; q < 2; ++q) {
-    float* const out = q ? y : x;
-    const float* src = q ? ctx->d_y : ctx->d_x[ctx->cur];
-    if (!out) continue;
-    if (ctx->Rs != ctx->R && on_device && own_memory(ctx, out, 4)) {
-      SB_CUDA(sbd::launch_repitch(src, ctx->Rs, out, ctx->R, ctx->n, ctx->R, 0));
-      continue;
+  const float *const sx = ctx->d_x[ctx->cur], *const sy = ctx->d_y;
+  const bool padded = ctx->Rs != ctx->R;
+  if (padded && on_device && (!x || own_memory(ctx, x, 4)) && (!y || own_memory(ctx, y, 4))) {
+    SB_CUDA(sbd::launch_repitch(x ? sx : sy, x && y ? sy : nullptr, ctx->Rs, x ? x : y, y, ctx->R,
+                                ctx->n, ctx->R, 0));
+  } else {
+    for (int q = 0; q < 2; ++q) {
+      float* const out = q ? y : x;
+      const float* src = q ? sy : sx;
+      if (!out) continue;
+      if (padded) {  // gathered in the other x buffer first
+        float* const tmp = ctx->d_x[ctx->cur ^ 1];
+        SB_CUDA(sbd::launch_repitch(src, nullptr, ctx->Rs, tmp, nullptr, ctx->R, ctx->n, ctx->R, 0));
+        src = tmp;
+      }
+      SB_CUDA(cudaMemcpy(out, src, bytes, k));
     }
-    if (ctx->Rs != ctx->R) {  // padded rows: gathered in the other x buffer first
-      float* const tmp = ctx->d_x[ctx->cur ^ 1];
-      SB_CUDA(sbd::launch_repitch(src, ctx->Rs, tmp, ctx->R, ctx->n, ctx->R, 0));
-      src = tmp;
-    }
-    SB_CUDA(cudaMemcpy(out, src, bytes, k));
   }
-  SB_CUDA(cudaStreamSynchronize(0));  // as in sb_set_state
-  return SB_OK;
+  // the flag comes to the host behind the copies on the default stream: when it is
+  // here, they have finished, as in sb_set_state
+  return check_wait_flag(ctx);
 }
 
 sb_status sb_energy(sb_ctx* ctx, const int8_t* spins, int32_t replicas, double* out_E) {

@@ -102,10 +102,10 @@ cudaError_t launch_init(float* x, float* y, const int32_t* row_event, const int3
                         int32_t n, int32_t R, uint64_t seed, cudaStream_t s);
 // s[i] = sign byte of x[i]: 0x3C, 0xBC, 0x00 for x > 0, x < 0, x = 0 (signs.cuh)
 cudaError_t launch_signs(const float* x, uint8_t* s, size_t count, cudaStream_t st);
-// out rows (opitch floats apart) = in rows (ipitch apart), cols values each; the
-// rest of a longer out row is zeroed
-cudaError_t launch_repitch(const float* in, int32_t ipitch, float* out, int32_t opitch, int32_t n,
-                           int32_t cols, cudaStream_t s);
+// xo, yo: rows of opitch floats = x, y: rows of ipitch, cols values each; the
+// rest of a longer row is zeroed. y NULL: x alone.
+cudaError_t launch_repitch(const float* x, const float* y, int32_t ipitch, float* xo, float* yo,
+                           int32_t opitch, int32_t n, int32_t cols, cudaStream_t s);
 // blocks of the untiled step kernel resident per SM for this tiling and unroll
 int step_blocks_per_sm(int variant, int jbf16, const Tiling& t, int unroll);
 

@@ -47,3 +47,22 @@ def test_set_advance_get_on_a_side_stream(R):
     for _ in range(5):
         got = two_runs(lambda: None)
         assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("n", [1, 7, 300, 40000])
+@pytest.mark.parametrize("R", [2, 3, 31, 33, 50, 64, 130])
+def test_both_arrays_or_one(n, R):
+    """Rows shorter and longer than a warp, x and y together and each alone."""
+    import torch
+    ctx = sb.sb_create(n, np.zeros(n + 1, np.int32), np.zeros(0, np.int32), np.zeros(0), np.zeros(n))
+    g = torch.Generator(device="cuda").manual_seed(n + R)
+    x, y = (torch.rand((n, R), generator=g, device="cuda") for _ in range(2))
+    sb.sb_set_state(ctx, x, y)
+    hx, hy = sb.sb_get_state(ctx)
+    assert np.array_equal(hx, x.cpu().numpy()) and np.array_equal(hy, y.cpu().numpy())
+    for want_x, want_y in ((1, 1), (1, 0), (0, 1)):
+        a, b = torch.full_like(x, 7.0), torch.full_like(y, 7.0)
+        sb._lib.check(sb.lib.sb_get_state(ctx.handle, a.data_ptr() if want_x else None,
+                                          b.data_ptr() if want_y else None, 1))
+        assert torch.equal(a, x) if want_x else bool((a == 7.0).all())
+        assert torch.equal(b, y) if want_y else bool((b == 7.0).all())
