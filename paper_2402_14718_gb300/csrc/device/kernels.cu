@@ -489,10 +489,15 @@ __global__ void __launch_bounds__(kBlock) k_step_r1g(const StepArgs a) {
 #ifndef SB_DSB_BLOCK
 #define SB_DSB_BLOCK 128
 #endif
-// eight CTAs of 128 threads per SM: 64 registers, no spills (nine spill and take
-// twice the time, ten 42 registers 1.1 to 1.9 times)
+// seven CTAs of 128 threads per SM: with the sign bytes, x and y in plain loads
+// (pdl.cuh) eight leave the compiler too few registers to keep the loads together.
+// us per step with eight / seven, and with the shuffled walk and nine CTAs that came
+// before: 10,878 rows R = 256 17.9 / 14.9, 17.4; 39,165 rows R = 64 47.7 / 31.5, 47.3,
+// R = 512 124.5 / 119, 121; 91,504 rows R = 256 200 / 188, 199; 472,812 rows R = 128
+// 458 / 424, 486. Six: R = 512 122, 91,504 rows 194; asking for all own values before
+// the first store, with seven: R = 512 123.5, 91,504 rows 198.
 #ifndef SB_DSB_MINB
-#define SB_DSB_MINB 8
+#define SB_DSB_MINB 7
 #endif
 constexpr int kDsbBlock = SB_DSB_BLOCK;  // threads per CTA of k_step_dsb16
 
