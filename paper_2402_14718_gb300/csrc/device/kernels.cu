@@ -144,8 +144,8 @@ __device__ __forceinline__ unsigned group_mask(int G) {
 constexpr int step_blocks(int V, int NCH, int U) {
   return V == 1 ? (NCH == 1 ? 4 : 3) : (NCH * U <= 4 ? 3 : 2);
 }
-template <int V, int NCH, int U, int MODE, typename JT>
-__global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const StepArgs a) {
+template <int V, int NCH, int U, int B, int MODE, typename JT>
+__global__ void __launch_bounds__(kBlock, B) k_step(const StepArgs a) {
   constexpr int VARIANT = MODE == 3 ? 2 : (MODE == 4 ? 1 : MODE);
   constexpr bool use_sgn = MODE == 3;
   constexpr bool record = MODE == 4;
@@ -293,11 +293,11 @@ __global__ void __launch_bounds__(kBlock, (step_blocks(V, NCH, U))) k_step(const
   }
 }
 
-template <int V, int NCH, int U, int MODE>
+template <int V, int NCH, int U, int MODE, int B = step_blocks(V, NCH, U)>
 cudaError_t launch_step_u(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
   dim3 grid((a.n + a.rpc - 1) / a.rpc, t.tiles);
-  return jbf16 ? launch_pdl(k_step<V, NCH, U, MODE, __nv_bfloat16>, grid, kBlock, a, s)
-               : launch_pdl(k_step<V, NCH, U, MODE, float>, grid, kBlock, a, s);
+  return jbf16 ? launch_pdl(k_step<V, NCH, U, B, MODE, __nv_bfloat16>, grid, kBlock, a, s)
+               : launch_pdl(k_step<V, NCH, U, B, MODE, float>, grid, kBlock, a, s);
 }
 
 // Neighbours in flight. More shorten the chain of a heavy row and cost
@@ -308,7 +308,11 @@ cudaError_t launch_step_u(int jbf16, const Tiling& t, const StepArgs& a, cudaStr
 //  GPU's threads;
 //  two chunks per lane, 2 / 4 in flight: 10,878 rows R = 100 12.9 / 11.4, R = 192
 //  16.2 / 17.1; 109,775 rows R = 100 88 / 105. So 2 from 1.5 M spins on (4 with
-//  sign bytes, which hold a quarter of the registers: 89 / 84).
+//  sign bytes, which hold a quarter of the registers: 89 / 84);
+//  sign bytes, two chunks, two / three CTAs per SM: 67,445 rows R = 192 110 / 82 (107
+//  with the shuffled walk that came before), R = 20 14.9 / 13.2; 39,165 rows R = 160
+//  111 / 91, R = 12 27.9 / 31.4; 10,878 rows R = 160 18.2 / 16.2, R = 96 FP32 11.7 / 12.2,
+//  R = 33 8.2 / 9.5. So three from 1.5 M spins on as well.
 template <int V, int NCH, int MODE>
 cudaError_t launch_step_t(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
   const int64_t spins = (int64_t)a.n * a.R;
@@ -320,19 +324,22 @@ cudaError_t launch_step_t(int jbf16, const Tiling& t, const StepArgs& a, cudaStr
   } else if constexpr (NCH == 2 && MODE != 3) {
     return spins >= 1500000 ? launch_step_u<V, NCH, 2, MODE>(jbf16, t, a, s)
                             : launch_step_u<V, NCH, 4, MODE>(jbf16, t, a, s);
+  } else if constexpr (NCH == 2) {
+    return spins >= 1500000 ? launch_step_u<V, NCH, 4, MODE, 3>(jbf16, t, a, s)
+                            : launch_step_u<V, NCH, 4, MODE>(jbf16, t, a, s);
   } else {
-    return launch_step_u<V, NCH, NCH == 2 ? 4 : 2, MODE>(jbf16, t, a, s);
+    return launch_step_u<V, NCH, 2, MODE>(jbf16, t, a, s);
   }
 }
 
 template <int V, int NCH, int MODE>
 int blocks_per_sm_t(int jbf16) {
-  constexpr int U = V == 1 ? (NCH == 4 ? 4 : 8) : (NCH == 4 ? 2 : 4);
+  constexpr int U = V == 1 ? (NCH == 4 ? 4 : 8) : (NCH == 4 ? 2 : 4), B = step_blocks(V, NCH, U);
   int b = 0;
   const cudaError_t e =
       jbf16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                  &b, k_step<V, NCH, U, MODE, __nv_bfloat16>, kBlock, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step<V, NCH, U, MODE, float>,
+                  &b, k_step<V, NCH, U, B, MODE, __nv_bfloat16>, kBlock, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step<V, NCH, U, B, MODE, float>,
                                                             kBlock, 0);
   return e == cudaSuccess && b > 0 ? b : 1;
 }
