@@ -11,12 +11,12 @@
 // and the diagonal -- is an exact sparse residual formed on the host.
 //
 // One step is two launches:
-//   k_fac_sum:  for each group block g (one hit), T_s = sum of x (or, for
-//               dSB, of sgn x) over the block's members in slot s, then
+//   k_fac_sum (dSB: k_fac_sum_sgn): for each group block g (one hit), T_s = sum
+//               of x (dSB: of sgn x) over the block's members in slot s, then
 //               U_s = sum_{s'} W[s][s'] T_{s'} for every slot whose U row a
 //               factored row reads;
-//   k_step_fac: for each row, f = jf * sum of its U rows + residual row . x,
-//               then the fused symplectic-Euler update and wall.
+//   k_step_fac (dSB: k_step_fac_sgn): for each row, f = jf * sum of its U rows
+//               + residual row . x, then the fused symplectic-Euler update and wall.
 // A row that the host found cheaper in its plain CSR form has no U rows and
 // its whole CSR row as residual, so one kernel serves both kinds of rows.
 //
@@ -83,12 +83,9 @@ __device__ __forceinline__ unsigned lane_group_mask(int G) {
   return G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
 }
 
-// One member's values at this lane's replicas, as loaded: FP32 chunks
-// (MODE 0) or 16 sign bytes (MODE 1, unpacked to 2^-7 sgn only when added).
-template <int MODE, int NCH>
-struct Chunk;
+// One member's values at this lane's replicas
 template <int NCH>
-struct Chunk<0, NCH> {
+struct Chunk {
   static constexpr int P = 4 * NCH;
   float4 t[NCH];
   __device__ __forceinline__ void load(const FacSumArgs& a, size_t off, int G, int row) {
@@ -153,17 +150,15 @@ __device__ __forceinline__ void store_u(const FacSumArgs& a, int g, size_t off, 
 }
 
 // Lane l's P values of slot s of scratch slot c (the lane's own replicas).
-template <int MODE, int NCH, int P>
 __device__ __forceinline__ size_t scr_index(const FacSumArgs& a, int c, int s, size_t off, int G,
                                             int v) {
-  const size_t base = ((size_t)c * a.K + s) * a.R + off;
-  return MODE == 0 ? base + 4 * G * (v >> 2) + (v & 3) : base + v;
+  return ((size_t)c * a.K + s) * a.R + off + 4 * G * (v >> 2) + (v & 3);
 }
 
 // residency bounds (CTAs of 128 threads per SM) of the FP32 forms: the bounds
 // that give the compiler's own unbounded register counts (about 48 / 56 registers with one 16-byte chunk per
 // lane, 64 / 72 with two).
-template <int MODE, int NCH>
+template <int NCH>
 struct FacMinBlocks {
   static constexpr int sum = NCH == 2 ? 7 : 9, step = NCH == 2 ? 8 : 9;
 };
@@ -273,9 +268,9 @@ __global__ void __launch_bounds__(kFacBlock, 7) k_fac_sum_sgn(const FacSumArgs a
   store_u<1, UF32 ? 2 : 1, K, P>(a, item.x, off, G, U);
 }
 
-template <int MODE, int NCH, int K>
-__global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_fac_sum(const FacSumArgs a) {
-  using C = Chunk<MODE, NCH>;
+template <int NCH, int K>
+__global__ void __launch_bounds__(kFacBlock, FacMinBlocks<NCH>::sum) k_fac_sum(const FacSumArgs a) {
+  using C = Chunk<NCH>;
   constexpr int P = C::P;
   const int G = a.G;
   const int gq = threadIdx.x / G;
@@ -283,8 +278,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
   const int it = blockIdx.x * (kFacBlock / G) + gq;
   if (it >= a.nitems) return;  // the whole lane group leaves together
   const unsigned mask = lane_group_mask(G);
-  const size_t off = MODE == 0 ? (size_t)blockIdx.y * (4 * G * NCH) + 4 * l
-                               : (size_t)blockIdx.y * (kSgnPer * G) + kSgnPer * l;
+  const size_t off = (size_t)blockIdx.y * (4 * G * NCH) + 4 * l;
   const int4 item = __ldg(a.item + it);
   const int g = item.x;
   // slot boundaries of the block's members (members grouped by slot)
@@ -331,7 +325,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
     }
   }
   if (item.w < 0) {  // the whole block in one item
-    store_u<MODE, NCH, K, P>(a, g, off, G, U);
+    store_u<0, NCH, K, P>(a, g, off, G, U);
     return;
   }
   // one chunk of a split block: its sums to the scratch slot; the chunk that
@@ -340,7 +334,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
 #pragma unroll
   for (int s = 0; s < K; ++s)
 #pragma unroll
-    for (int v = 0; v < P; ++v) a.scratch[scr_index<MODE, NCH, P>(a, item.w, s, off, G, v)] = U[s][v];
+    for (int v = 0; v < P; ++v) a.scratch[scr_index(a, item.w, s, off, G, v)] = U[s][v];
   __threadfence();
   __syncwarp(mask);
   int last = 0;
@@ -359,8 +353,8 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::sum)) k_f
 #pragma unroll
     for (int s = 0; s < K; ++s)
 #pragma unroll
-      for (int v = 0; v < P; ++v) U[s][v] += __ldcg(a.scratch + scr_index<MODE, NCH, P>(a, c0 + c, s, off, G, v));
-  store_u<MODE, NCH, K, P>(a, g, off, G, U);
+      for (int v = 0; v < P; ++v) U[s][v] += __ldcg(a.scratch + scr_index(a, c0 + c, s, off, G, v));
+  store_u<0, NCH, K, P>(a, g, off, G, U);
   if (l == 0) *cnt = 0;  // ready for the next launch
 }
 
@@ -402,10 +396,10 @@ __global__ void k_fac_head(const FacHeadArgs a) {
 
 // Adds cnt residual entries (lane q of the lane group holds column mc and
 // weight mw of entry q) to this lane's replicas, four neighbour rows in flight.
-template <int MODE, int NCH, int P>
-__device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, float mw,
-                                             unsigned mask, int G, const float* xin,
-                                             const uint8_t* sgn_in, size_t off, int R) {
+template <int NCH>
+__device__ __forceinline__ void walk_entries(float (&acc)[4 * NCH], int cnt, int mc, float mw,
+                                             unsigned mask, int G, const float* xin, size_t off,
+                                             int R) {
   int q = 0;
   for (; q + 4 <= cnt; q += 4) {
     int c[4];
@@ -415,51 +409,32 @@ __device__ __forceinline__ void walk_entries(float (&acc)[P], int cnt, int mc, f
       c[u] = __shfl_sync(mask, mc, q + u, G);
       w[u] = __shfl_sync(mask, mw, q + u, G);
     }
-    if (MODE == 0) {
-      float4 t[4][NCH];
+    float4 t[4][NCH];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int j = 0; j < NCH; ++j)
-          t[u][j] = reinterpret_cast<const float4*>(xin + (size_t)c[u] * R + off)[G * j];
+      for (int j = 0; j < NCH; ++j)
+        t[u][j] = reinterpret_cast<const float4*>(xin + (size_t)c[u] * R + off)[G * j];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int j = 0; j < NCH; ++j) {
-          acc[4 * j] = fmaf(w[u], t[u][j].x, acc[4 * j]);
-          acc[4 * j + 1] = fmaf(w[u], t[u][j].y, acc[4 * j + 1]);
-          acc[4 * j + 2] = fmaf(w[u], t[u][j].z, acc[4 * j + 2]);
-          acc[4 * j + 3] = fmaf(w[u], t[u][j].w, acc[4 * j + 3]);
-        }
-    } else {
-      Words<kSgnPer / 4> t[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) t[u].ld(sgn_in + (size_t)c[u] * R + off);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < kSgnPer && v < P; ++v)
-          acc[v] = fmaf(w[u], scaled_sign_of_byte(t[u].w[v >> 2], v & 3), acc[v]);
-    }
+      for (int j = 0; j < NCH; ++j) {
+        acc[4 * j] = fmaf(w[u], t[u][j].x, acc[4 * j]);
+        acc[4 * j + 1] = fmaf(w[u], t[u][j].y, acc[4 * j + 1]);
+        acc[4 * j + 2] = fmaf(w[u], t[u][j].z, acc[4 * j + 2]);
+        acc[4 * j + 3] = fmaf(w[u], t[u][j].w, acc[4 * j + 3]);
+      }
   }
   for (; q < cnt; ++q) {
     const int c = __shfl_sync(mask, mc, q, G);
     const float w = __shfl_sync(mask, mw, q, G);
-    if (MODE == 0) {
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const float4 t = reinterpret_cast<const float4*>(xin + (size_t)c * R + off)[G * j];
-        acc[4 * j] = fmaf(w, t.x, acc[4 * j]);
-        acc[4 * j + 1] = fmaf(w, t.y, acc[4 * j + 1]);
-        acc[4 * j + 2] = fmaf(w, t.z, acc[4 * j + 2]);
-        acc[4 * j + 3] = fmaf(w, t.w, acc[4 * j + 3]);
-      }
-    } else {
-      Words<kSgnPer / 4> t;
-      t.ld(sgn_in + (size_t)c * R + off);
-#pragma unroll
-      for (int v = 0; v < kSgnPer && v < P; ++v)
-        acc[v] = fmaf(w, scaled_sign_of_byte(t.w[v >> 2], v & 3), acc[v]);
+    for (int j = 0; j < NCH; ++j) {
+      const float4 t = reinterpret_cast<const float4*>(xin + (size_t)c * R + off)[G * j];
+      acc[4 * j] = fmaf(w, t.x, acc[4 * j]);
+      acc[4 * j + 1] = fmaf(w, t.y, acc[4 * j + 1]);
+      acc[4 * j + 2] = fmaf(w, t.z, acc[4 * j + 2]);
+      acc[4 * j + 3] = fmaf(w, t.w, acc[4 * j + 3]);
     }
   }
 }
@@ -522,11 +497,10 @@ struct URow<1, NCH> {
   }
 };
 
-// VARIANT 0 aSB, 1 bSB (MODE 0: FP32 x), 2 dSB (MODE 1: sign bytes)
-template <int VARIANT, int MODE, int NCH, int K, typename JT>
-__global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_step_fac(const FacStepArgs a) {
-  constexpr int P = MODE == 0 ? 4 * NCH : kSgnPer;
-  constexpr int NV = P / 4;  // float4 of own x (and y) per lane
+// VARIANT 0 aSB, 1 bSB
+template <int VARIANT, int NCH, int K, typename JT>
+__global__ void __launch_bounds__(kFacBlock, FacMinBlocks<NCH>::step) k_step_fac(const FacStepArgs a) {
+  constexpr int P = 4 * NCH;
   const int G = a.G;
   const int gq = threadIdx.x / G;
   const int l = threadIdx.x - gq * G;
@@ -534,18 +508,16 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   if (row >= a.n) return;
   const unsigned mask = lane_group_mask(G);
   const int R = a.R;
-  const size_t off = MODE == 0 ? (size_t)blockIdx.y * (4 * G * NCH) + 4 * l
-                               : (size_t)blockIdx.y * (kSgnPer * G) + kSgnPer * l;
+  const size_t off = (size_t)blockIdx.y * (4 * G * NCH) + 4 * l;
   const size_t idx = (size_t)row * R + off;
   const JT* J = static_cast<const JT*>(a.rJ);
   pdl_wait();
   // the row's own x and y and its U rows are read after the residual walk:
   // ask for them in L2 now, so that those loads do not wait on HBM
 #pragma unroll
-  for (int j = 0; j < P / 4; ++j) {
-    const size_t o = MODE == 0 ? idx + 4 * G * j : idx + 4 * j;
-    prefetch_l2(a.xin + o);
-    prefetch_l2(a.y + o);
+  for (int j = 0; j < NCH; ++j) {
+    prefetch_l2(a.xin + idx + 4 * G * j);
+    prefetch_l2(a.y + idx + 4 * G * j);
   }
   constexpr int HW = fac_head_words(sizeof(JT));
   const uint32_t* hd = a.head + (size_t)row * HW;
@@ -554,8 +526,7 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   for (int s = 0; s < K; ++s) {
     us[s] = (int)__ldg(hd + kFacHead + s);
     if (us[s] >= 0) us[s] = chk_idx(us[s], a.urows, kChkURow);
-    if (us[s] >= 0)
-      prefetch_l2(static_cast<const char*>(a.U) + ((size_t)us[s] * R + off) * (MODE == 0 || NCH == 2 ? 4 : 2));
+    if (us[s] >= 0) prefetch_l2(static_cast<const char*>(a.U) + ((size_t)us[s] * R + off) * 4);
   }
   int p0 = __ldg(a.rrowptr + row), p1 = __ldg(a.rrowptr + row + 1);
   chk_rows(p0, p1, a.rnnz);
@@ -573,9 +544,8 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
     if (l < cnt) {
       mc = chk_idx((int)__ldg(hd + hb + l), a.n, kChkCol);
       mw = head_j<JT>(hd, hb + l);
-      if (MODE == 1) mw *= kSignScale;  // 2^7 J: sign bytes read as 2^-7 sgn
     }
-    walk_entries<MODE, NCH, P>(acc, cnt, mc, mw, mask, G, a.xin, a.sgn_in, off, R);
+    walk_entries<NCH>(acc, cnt, mc, mw, mask, G, a.xin, off, R);
   }
   for (int pb = p0 + kFacHead; pb < p1; pb += G) {
     const int cnt = min(G, p1 - pb);
@@ -584,9 +554,8 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
     if (l < cnt) {
       mc = chk_idx(__ldg(a.rcol + pb + l), a.n, kChkCol);
       mw = jv(J, pb + l);
-      if (MODE == 1) mw *= kSignScale;
     }
-    walk_entries<MODE, NCH, P>(acc, cnt, mc, mw, mask, G, a.xin, a.sgn_in, off, R);
+    walk_entries<NCH>(acc, cnt, mc, mw, mask, G, a.xin, off, R);
   }
   // the factored part: sum of this row's U rows (none for a plain row)
   bool any = false;
@@ -597,15 +566,13 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   for (int s = 0; s < K; ++s) {
     if (us[s] < 0) continue;
     any = true;
-    URow<MODE, NCH> ur;
+    URow<0, NCH> ur;
     ur.load(a.U, (size_t)us[s] * R + off, G);
     ur.add_to(fu);
   }
-  // dSB: U holds sums of 2^-7 sgn, so the scale is 2^7 jf (exact)
-  const float jf = MODE == 1 ? a.jf * kSignScale : a.jf;
   if (any) {
 #pragma unroll
-    for (int v = 0; v < P; ++v) acc[v] = fmaf(jf, fu[v], acc[v]);
+    for (int v = 0; v < P; ++v) acc[v] = fmaf(a.jf, fu[v], acc[v]);
   }
 
   // symplectic Euler: momentum with the old position, then position, then wall
@@ -613,13 +580,9 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
   const int ev = a.row_event ? __ldg(a.row_event + row) : 0;
   const float c0 = a.c0_ev[ev];
   const float hi = __ldg(a.h + row);
-  Words<kSgnPer / 4> sw;  // dSB: the new sign bytes
 #pragma unroll
-  for (int k = 0; k < kSgnPer / 4; ++k) sw.w[k] = 0u;
-  const bool inplace = a.xout == a.xin;
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    const size_t o = MODE == 0 ? idx + 4 * G * j : idx + 4 * j;
+  for (int j = 0; j < NCH; ++j) {
+    const size_t o = idx + 4 * G * j;
     const float4 xo = *reinterpret_cast<const float4*>(a.xin + o);
     const float4 yo = *reinterpret_cast<const float4*>(a.y + o);
     float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
@@ -636,16 +599,13 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<MODE, NCH>::step)) k_
       }
       xs[v] = x;
       ys[v] = y;
-      if (MODE == 1 && j < kSgnPer / 4) sw.w[j] |= sign_byte(x) << (8 * v);
     }
-    // a spin that stays on the wall keeps x = +-1, y = 0: nothing to write back
-    // where the value is updated in place (y always; x on the dSB path)
+    // a spin that stays on the wall keeps y = 0: nothing to write back there
     const float4 xn = make_float4(xs[0], xs[1], xs[2], xs[3]);
     const float4 yn = make_float4(ys[0], ys[1], ys[2], ys[3]);
-    if (!inplace || bits_differ(xo, xn)) *reinterpret_cast<float4*>(a.xout + o) = xn;
+    *reinterpret_cast<float4*>(a.xout + o) = xn;
     if (bits_differ(yo, yn)) *reinterpret_cast<float4*>(a.y + o) = yn;
   }
-  if (MODE == 1) sw.st(a.sgn_out + idx);
 }
 
 // ---------------------------------------------------------------- dSB row step
@@ -801,39 +761,39 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
   sw.st(a.sgn_out + idx);
 }
 
-template <int MODE, int NCH, int K>
+template <int NCH, int K>
 cudaError_t launch_sum_k(const FacSumArgs& a, cudaStream_t s) {
   if (a.nitems <= 0) return cudaSuccess;
   const int per = kFacBlock / a.G;
   dim3 grid((a.nitems + per - 1) / per, a.tiles);
-  return launch_pdl(k_fac_sum<MODE, NCH, K>, grid, kFacBlock, a, s);
+  return launch_pdl(k_fac_sum<NCH, K>, grid, kFacBlock, a, s);
 }
 
-template <int MODE, int NCH>
+template <int NCH>
 cudaError_t launch_sum_n(const FacSumArgs& a, cudaStream_t s) {
   switch (a.K) {
-    case 1: return launch_sum_k<MODE, NCH, 1>(a, s);
-    case 2: return launch_sum_k<MODE, NCH, 2>(a, s);
-    case 3: return launch_sum_k<MODE, NCH, 3>(a, s);
-    case 4: return launch_sum_k<MODE, NCH, 4>(a, s);
+    case 1: return launch_sum_k<NCH, 1>(a, s);
+    case 2: return launch_sum_k<NCH, 2>(a, s);
+    case 3: return launch_sum_k<NCH, 3>(a, s);
+    case 4: return launch_sum_k<NCH, 4>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <int VARIANT, int MODE, int NCH, int K, typename JT>
+template <int VARIANT, int NCH, int K, typename JT>
 cudaError_t launch_step_k(const FacStepArgs& a, cudaStream_t s) {
   const int per = kFacBlock / a.G;
   dim3 grid((a.n + per - 1) / per, a.tiles);
-  return launch_pdl(k_step_fac<VARIANT, MODE, NCH, K, JT>, grid, kFacBlock, a, s);
+  return launch_pdl(k_step_fac<VARIANT, NCH, K, JT>, grid, kFacBlock, a, s);
 }
 
-template <int VARIANT, int MODE, int NCH, typename JT>
+template <int VARIANT, int NCH, typename JT>
 cudaError_t launch_step_n(const FacStepArgs& a, cudaStream_t s) {
   switch (a.K) {
-    case 1: return launch_step_k<VARIANT, MODE, NCH, 1, JT>(a, s);
-    case 2: return launch_step_k<VARIANT, MODE, NCH, 2, JT>(a, s);
-    case 3: return launch_step_k<VARIANT, MODE, NCH, 3, JT>(a, s);
-    case 4: return launch_step_k<VARIANT, MODE, NCH, 4, JT>(a, s);
+    case 1: return launch_step_k<VARIANT, NCH, 1, JT>(a, s);
+    case 2: return launch_step_k<VARIANT, NCH, 2, JT>(a, s);
+    case 3: return launch_step_k<VARIANT, NCH, 3, JT>(a, s);
+    case 4: return launch_step_k<VARIANT, NCH, 4, JT>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -868,8 +828,8 @@ template <typename JT>
 cudaError_t launch_step_j(int variant, const FacStepArgs& a, cudaStream_t s) {
   if (variant == 2) return a.NCH == 2 ? launch_step_sgn<true, JT>(a, s) : launch_step_sgn<false, JT>(a, s);
   if (a.NCH == 2)
-    return variant == 0 ? launch_step_n<0, 0, 2, JT>(a, s) : launch_step_n<1, 0, 2, JT>(a, s);
-  return variant == 0 ? launch_step_n<0, 0, 1, JT>(a, s) : launch_step_n<1, 0, 1, JT>(a, s);
+    return variant == 0 ? launch_step_n<0, 2, JT>(a, s) : launch_step_n<1, 2, JT>(a, s);
+  return variant == 0 ? launch_step_n<0, 1, JT>(a, s) : launch_step_n<1, 1, JT>(a, s);
 }
 
 }  // namespace
@@ -925,7 +885,7 @@ cudaError_t launch_fac_head(const FacHeadArgs& a, cudaStream_t s) {
 
 cudaError_t launch_fac_sum(int variant, const FacSumArgs& a, cudaStream_t s) {
   if (variant == 2) return a.NCH == 2 ? launch_sum_sgn<true>(a, s) : launch_sum_sgn<false>(a, s);
-  return a.NCH == 2 ? launch_sum_n<0, 2>(a, s) : launch_sum_n<0, 1>(a, s);
+  return a.NCH == 2 ? launch_sum_n<2>(a, s) : launch_sum_n<1>(a, s);
 }
 
 cudaError_t launch_step_fac(int variant, int jbf16, const FacStepArgs& a, cudaStream_t s) {
