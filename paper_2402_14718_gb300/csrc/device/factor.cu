@@ -155,13 +155,28 @@ __device__ __forceinline__ size_t scr_index(const FacSumArgs& a, int c, int s, s
   return ((size_t)c * a.K + s) * a.R + off + 4 * G * (v >> 2) + (v & 3);
 }
 
-// residency bounds (CTAs of 128 threads per SM) of the FP32 forms: the bounds
-// that give the compiler's own unbounded register counts (about 48 / 56 registers with one 16-byte chunk per
-// lane, 64 / 72 with two).
-template <int NCH>
+// Residency bounds of the FP32 forms (CTAs of 128 threads per SM). Two chunks per
+// lane: seven and eight. One chunk: eight or nine, by fac_blocks().
+template <int NCH, int B>
 struct FacMinBlocks {
-  static constexpr int sum = NCH == 2 ? 7 : 9, step = NCH == 2 ? 8 : 9;
+  static constexpr int sum = NCH == 2 ? 7 : B, step = NCH == 2 ? 8 : B;
 };
+// Nine CTAs leave 56 registers and spill up to 52 bytes since x and U come by plain
+// loads (pdl.cuh); eight fit. Nine stay the better choice where there are lanes
+// enough to use the warps. bSB, us per step with nine / eight, and with __ldg and
+// nine, launch by launch, that came before:
+//   R = 16: 39,445 rows (158 k lanes) 21.2 / 17.4, 18.3; 98,134 rows (393 k) 28.6 /
+//   27.2, 28.1; 156,688 rows (627 k) 31.1 / 31.3, 31.0; 242,044 rows (968 k) 48.3 / 50.4,
+//   48.7. R = 32: 39,445 rows 21.2 / 19.6, 21.3; 98,134 rows (785 k) 36.1 / 35.6, 35.8;
+//   114,665 rows (917 k) 42.2 / 43.0, 41.7. R = 64: 39,445 rows 25.4 / 24.6, 25.4;
+//   108,750 rows (1.7 M) 58.2 / 61.0, 59.4.
+//   R = 8 (two lanes a row): 39,445 rows (79 k) 26.4 / 25.5, 26.4; 67,374 rows (135 k)
+//   19.2 / 20.8, 19.6; 98,134 rows (196 k) 31.9 / 31.1, 31.0; 242,044 rows 40.8 / 41.4, 40.9.
+//   R = 4: 39,165 rows 33.0 / 32.2, 32.7; 472,812 rows 77.4 / 73.0, 71.8.
+inline int fac_blocks(int64_t n, int R, int G) {
+  const int64_t lanes = n * R / 4;
+  return G >= 2 && lanes >= (G == 2 ? 100000 : 800000) ? 9 : 8;
+}
 
 // ---------------------------------------------------------------- dSB group sums
 // Lane l of a G-lane group holds the replicas tile0 + 8 l .. + 7 (one 8-byte
@@ -268,8 +283,8 @@ __global__ void __launch_bounds__(kFacBlock, 7) k_fac_sum_sgn(const FacSumArgs a
   store_u<1, UF32 ? 2 : 1, K, P>(a, item.x, off, G, U);
 }
 
-template <int NCH, int K>
-__global__ void __launch_bounds__(kFacBlock, FacMinBlocks<NCH>::sum) k_fac_sum(const FacSumArgs a) {
+template <int NCH, int K, int B>
+__global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<NCH, B>::sum)) k_fac_sum(const FacSumArgs a) {
   using C = Chunk<NCH>;
   constexpr int P = C::P;
   const int G = a.G;
@@ -498,8 +513,8 @@ struct URow<1, NCH> {
 };
 
 // VARIANT 0 aSB, 1 bSB
-template <int VARIANT, int NCH, int K, typename JT>
-__global__ void __launch_bounds__(kFacBlock, FacMinBlocks<NCH>::step) k_step_fac(const FacStepArgs a) {
+template <int VARIANT, int NCH, int K, int B, typename JT>
+__global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<NCH, B>::step)) k_step_fac(const FacStepArgs a) {
   constexpr int P = 4 * NCH;
   const int G = a.G;
   const int gq = threadIdx.x / G;
@@ -766,7 +781,9 @@ cudaError_t launch_sum_k(const FacSumArgs& a, cudaStream_t s) {
   if (a.nitems <= 0) return cudaSuccess;
   const int per = kFacBlock / a.G;
   dim3 grid((a.nitems + per - 1) / per, a.tiles);
-  return launch_pdl(k_fac_sum<NCH, K>, grid, kFacBlock, a, s);
+  if (NCH == 1 && fac_blocks(a.n, a.R, a.G) == 9)
+    return launch_pdl(k_fac_sum<NCH, K, NCH == 1 ? 9 : 8>, grid, kFacBlock, a, s);
+  return launch_pdl(k_fac_sum<NCH, K, 8>, grid, kFacBlock, a, s);
 }
 
 template <int NCH>
@@ -784,7 +801,9 @@ template <int VARIANT, int NCH, int K, typename JT>
 cudaError_t launch_step_k(const FacStepArgs& a, cudaStream_t s) {
   const int per = kFacBlock / a.G;
   dim3 grid((a.n + per - 1) / per, a.tiles);
-  return launch_pdl(k_step_fac<VARIANT, NCH, K, JT>, grid, kFacBlock, a, s);
+  if (NCH == 1 && fac_blocks(a.n, a.R, a.G) == 9)
+    return launch_pdl(k_step_fac<VARIANT, NCH, K, NCH == 1 ? 9 : 8, JT>, grid, kFacBlock, a, s);
+  return launch_pdl(k_step_fac<VARIANT, NCH, K, 8, JT>, grid, kFacBlock, a, s);
 }
 
 template <int VARIANT, int NCH, typename JT>
