@@ -123,15 +123,20 @@ struct sb_ctx {
   double sched_a0 = 0.0;
   // readout (sized for eR replicas, independent of the state's R)
   int32_t eR = 0;
-  int32_t energy_rows = 0, nblk = 0;
-  int32_t* d_blk_row = nullptr;
-  int32_t* d_ev_blk0 = nullptr;
-  double* d_partial = nullptr;
+  // blocks of rows whose energies are summed first, and their sums for eR
+  // replicas: in FP64 ([0], always there) and from selection bits ([1])
+  struct EnergyBlocks {
+    int32_t rows = 0, nblk = 0;
+    int32_t* d_row = nullptr;
+    int32_t* d_ev0 = nullptr;
+    double* d_partial = nullptr;
+  } eb[2];
   double* d_Eall = nullptr;
   double* d_bestE = nullptr;
   int32_t* d_bestr = nullptr;
   uint8_t* d_T = nullptr;
   uint8_t* d_bits = nullptr;    // selections of eR replicas as bits (whole-number couplings)
+  bool bits_oom = false;        // no memory for the bits at eR replicas: FP64 instead
   bool b_whole = false;         // couplings are whole numbers of 2^-8 (k_energy_bits)
   int32_t* d_inexact = nullptr;  // k_convert's verdict on that
   int8_t* d_spins = nullptr;
@@ -407,8 +412,10 @@ sb_status validate_csr(int32_t n, int64_t nnz, const int32_t* rowptr, const int3
 
 void free_readout(sb_ctx* c) {
   dfree(c->d_bits);
-  dfree(c->d_partial);
+  dfree(c->eb[0].d_partial);
+  dfree(c->eb[1].d_partial);
   dfree(c->d_Eall);
+  c->bits_oom = false;
   c->eR = 0;
 }
 
@@ -530,8 +537,10 @@ void free_all(sb_ctx* c) {
   dfree(c->d_c0auto);
   dfree(c->d_c0ev);
   dfree(c->d_sched);
-  dfree(c->d_blk_row);
-  dfree(c->d_ev_blk0);
+  for (sb_ctx::EnergyBlocks& b : c->eb) {
+    dfree(b.d_row);
+    dfree(b.d_ev0);
+  }
   dfree(c->d_bestE);
   dfree(c->d_bestr);
   dfree(c->d_T);
@@ -566,26 +575,26 @@ void free_all(sb_ctx* c) {
 }
 
 // (Re)build the energy block table: blocks of `rows` rows that never straddle an event.
-sb_status ensure_energy_blocks(sb_ctx* c, int32_t rows) {
-  if (c->energy_rows == rows && c->d_blk_row) return SB_OK;
-  std::vector<int32_t> blk_row, ev_blk0;
-  for (int32_t e = 0; e < c->E; ++e) {
+sb_status ensure_energy_blocks(sb_ctx* c, sb_ctx::EnergyBlocks& b, int32_t rows, int32_t R) {
+  sb_status st;
+  if (b.rows != rows) {
+    std::vector<int32_t> blk_row, ev_blk0;
+    for (int32_t e = 0; e < c->E; ++e) {
+      ev_blk0.push_back((int32_t)blk_row.size());
+      for (int32_t r = c->ev_row0[e]; r < c->ev_row0[e + 1]; r += rows) blk_row.push_back(r);
+    }
     ev_blk0.push_back((int32_t)blk_row.size());
-    for (int32_t r = c->ev_row0[e]; r < c->ev_row0[e + 1]; r += rows) blk_row.push_back(r);
+    blk_row.push_back(c->n);
+    b.rows = 0;
+    dfree(b.d_row);
+    dfree(b.d_ev0);
+    if ((st = dalloc(&b.d_row, blk_row.size())) || (st = dalloc(&b.d_ev0, ev_blk0.size()))) return st;
+    SB_CUDA(cudaMemcpy(b.d_row, blk_row.data(), blk_row.size() * 4, cudaMemcpyHostToDevice));
+    SB_CUDA(cudaMemcpy(b.d_ev0, ev_blk0.data(), ev_blk0.size() * 4, cudaMemcpyHostToDevice));
+    b.nblk = (int32_t)blk_row.size() - 1;
+    b.rows = rows;
   }
-  ev_blk0.push_back((int32_t)blk_row.size());
-  blk_row.push_back(c->n);
-  dfree(c->d_blk_row);
-  dfree(c->d_ev_blk0);
-  sb_status st = dalloc(&c->d_blk_row, blk_row.size());
-  if (st) return st;
-  st = dalloc(&c->d_ev_blk0, ev_blk0.size());
-  if (st) return st;
-  SB_CUDA(cudaMemcpy(c->d_blk_row, blk_row.data(), blk_row.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(c->d_ev_blk0, ev_blk0.data(), ev_blk0.size() * 4, cudaMemcpyHostToDevice));
-  c->nblk = (int32_t)blk_row.size() - 1;
-  c->energy_rows = rows;
-  return SB_OK;
+  return dalloc(&b.d_partial, (size_t)b.nblk * R);
 }
 
 // Replicas as stored. Counts that are no multiple of 4 (the paper's 50 shots)
@@ -635,23 +644,27 @@ sb_status ensure_state(sb_ctx* c, int32_t R) {
   return SB_OK;
 }
 
+// Nothing here is freed while the replica count stays, whatever the weights become:
+// a readout that a caller has recorded keeps its buffers.
 sb_status ensure_readout(sb_ctx* c, int32_t R) {
-  const sbd::Tiling t = sbd::make_tiling(R);
-  int32_t rows = std::max(kEnergyRowsMin, 256 / t.G);
+  sb_status st;
+  if (c->eR != R || !c->eb[0].d_partial || !c->d_Eall) {
+    free_readout(c);
+    if ((st = ensure_energy_blocks(c, c->eb[0], std::max(kEnergyRowsMin, 256 / sbd::make_tiling(R).G), R)) ||
+        (st = dalloc(&c->d_Eall, (size_t)c->E * R)))
+      return st;
+    c->eR = R;
+  }
+  if (!c->b_whole || c->d_bits || c->bits_oom) return SB_OK;
   // whole-number couplings: larger blocks where that still leaves eight CTAs
   // per SM (fewer partial sums to add; the 472,812-row event: 2 ms of block sums)
-  if (c->b_whole) rows = std::min(sbd::kEnergyBitRows, std::max(kEnergyRowsMin, c->n / (152 * 8) / 64 * 64));
-  if (c->eR == R && c->energy_rows == rows && c->d_partial && c->d_Eall &&
-      (!c->b_whole || c->d_bits))
-    return SB_OK;
-  free_readout(c);
-  sb_status st = ensure_energy_blocks(c, rows);
-  if (st) return st;
-  if (c->b_whole && (st = dalloc(&c->d_bits, (size_t)c->n * sbd::energy_bit_stride(R)))) return st;
-  if ((st = dalloc(&c->d_partial, (size_t)c->nblk * R)) ||
-      (st = dalloc(&c->d_Eall, (size_t)c->E * R)))
-    return st;
-  c->eR = R;
+  if (!c->sms) SB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+  const int32_t rows = std::min(sbd::kEnergyBitRows, std::max(kEnergyRowsMin, c->n / (c->sms * 8) / 64 * 64));
+  st = ensure_energy_blocks(c, c->eb[1], rows, R);
+  if (!st) st = dalloc(&c->d_bits, (size_t)c->n * sbd::energy_bit_stride(R));
+  if (st != SB_ERR_OOM) return st;
+  dfree(c->eb[1].d_partial);  // the FP64 sums need none of it
+  c->bits_oom = true;
   return SB_OK;
 }
 
@@ -2615,7 +2628,14 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   if (!best_E) best_E = c->d_bestE;
   if (!best_r) best_r = c->d_bestr;
   const int* const err = d_spins ? nullptr : c->d_err;
-  if (c->b_whole) {
+  // A readout that the caller records is replayed after sb_set_weights as well,
+  // whose weights need not be whole numbers: both sums are recorded then, and
+  // k_convert's verdict on the weights of the day picks one on the device.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool bits = c->b_whole && c->d_bits;
+  if (bits) SB_CUDA(cudaStreamIsCapturing(s, &cap));
+  const int32_t* const gate = cap == cudaStreamCaptureStatusNone ? nullptr : c->d_inexact;
+  if (bits) {
     sbd::EnergyBitArgs b;
     b.rowptr = c->d_rowptr;
     b.col = c->d_col;
@@ -2624,16 +2644,19 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
     b.qlin = c->d_qlin;
     b.bits = c->d_bits;
     b.bstride = sbd::energy_bit_stride(R);
-    b.blk_row = c->d_blk_row;
-    b.nblk = c->nblk;
+    b.blk_row = c->eb[1].d_row;
+    b.nblk = c->eb[1].nblk;
     b.n = c->n;
     b.R = R;
-    b.partial = c->d_partial;
+    b.partial = c->eb[1].d_partial;
+    b.gate = gate;
     b.nnz = c->nnz;
     SB_CUDA(sbd::launch_select_bits(d_spins ? nullptr : c->d_x[c->cur], c->Rs, d_spins, c->n, R,
                                     c->d_bits, s));
     SB_CUDA(sbd::launch_energy_bits(b, s));
-    SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
+    SB_CUDA(sbd::launch_energy_reduce(b.partial, c->eb[1].d_ev0, c->E, R, E_all, gate, 0, s));
+  }
+  if (bits && !gate) {
     SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
     return SB_OK;
   }
@@ -2646,15 +2669,16 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   a.x = d_spins ? nullptr : c->d_x[c->cur];
   a.xstride = c->Rs;
   a.spins = d_spins;
-  a.blk_row = c->d_blk_row;
-  a.nblk = c->nblk;
+  a.blk_row = c->eb[0].d_row;
+  a.nblk = c->eb[0].nblk;
   a.n = c->n;
   a.R = R;
   a.G = t.G;
-  a.partial = c->d_partial;
+  a.partial = c->eb[0].d_partial;
+  a.gate = gate;
   a.nnz = c->nnz;
   SB_CUDA(sbd::launch_energy_partial(t, a, s));
-  SB_CUDA(sbd::launch_energy_reduce(c->d_partial, c->d_ev_blk0, c->E, R, E_all, s));
+  SB_CUDA(sbd::launch_energy_reduce(a.partial, c->eb[0].d_ev0, c->E, R, E_all, gate, 1, s));
   SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
   return SB_OK;
 }

@@ -1199,6 +1199,7 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
   const int C = R / V;
   const int tile_base = blockIdx.y * (G * NCH);
   const int ch0 = tile_base + g;
+  if (a.gate && *a.gate == 0) return;
   const int b = blockIdx.x;
   const int r0 = a.blk_row[b], r1 = a.blk_row[b + 1];
   double acc[NCH][V];
@@ -1332,6 +1333,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_energy_bits(const EnergyBitArgs a
   const JT* J = static_cast<const JT*>(a.J);
   const int lane = threadIdx.x & 31;
   const unsigned mask = TS == 32 ? 0xffffffffu : (((1u << TS) - 1u) << (lane & ~(TS - 1)));
+  if (a.gate && *a.gate != 0) return;
   const int b = blockIdx.x;
   const int r0 = a.blk_row[b], r1 = a.blk_row[b + 1];
   int pair[8];     // sum over the rows of T_i sum_j 256 b_ij T_j
@@ -1426,8 +1428,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_energy_bits(const EnergyBitArgs a
 constexpr int kReduceWarps = 32;
 __global__ void __launch_bounds__(32 * kReduceWarps) k_energy_reduce(const double* partial,
                                                                      const int32_t* ev_blk0,
-                                                                     int32_t R, double* out) {
+                                                                     int32_t R, double* out,
+                                                                     const int32_t* gate, int want) {
   __shared__ double sm[kReduceWarps][32];
+  if (gate && (*gate != 0) != (want != 0)) return;
   const int e = blockIdx.y;
   const int b0 = ev_blk0[e], b1 = ev_blk0[e + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1773,10 +1777,11 @@ cudaError_t launch_energy_partial(const Tiling& t, const EnergyArgs& a, cudaStre
 }
 
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
-                                 int32_t R, double* E_out, cudaStream_t s) {
+                                 int32_t R, double* E_out, const int32_t* gate, int want,
+                                 cudaStream_t s) {
   if (E <= 0 || R <= 0) return cudaSuccess;
   dim3 grid((R + 31) / 32, E);
-  k_energy_reduce<<<grid, 32 * kReduceWarps, 0, s>>>(partial, ev_blk0, R, E_out);
+  k_energy_reduce<<<grid, 32 * kReduceWarps, 0, s>>>(partial, ev_blk0, R, E_out, gate, want);
   return cudaGetLastError();
 }
 

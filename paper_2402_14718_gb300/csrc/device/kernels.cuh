@@ -139,6 +139,7 @@ struct EnergyArgs {
   int32_t n, R, G;
   double* partial;         // [nblk x R] scratch
   int64_t nnz = INT64_MAX; // CSR entries, where known (bounds-checked build)
+  const int32_t* gate = nullptr;  // device, may be NULL: does nothing where it holds 0
 };
 cudaError_t launch_energy_partial(const Tiling& t, const EnergyArgs& a, cudaStream_t s);
 
@@ -157,6 +158,7 @@ struct EnergyBitArgs {
   int32_t nblk, n, R;
   double* partial;         // [nblk x R]
   int64_t nnz;
+  const int32_t* gate;     // device, may be NULL: does nothing unless it holds 0
 };
 // bytes per row of the selection bits for R replicas
 inline int32_t energy_bit_stride(int R) { return (R + 31) / 32 * 4; }
@@ -164,9 +166,11 @@ inline int32_t energy_bit_stride(int R) { return (R + 31) / 32 * 4; }
 cudaError_t launch_select_bits(const float* x, int32_t xstride, const int8_t* spins, int32_t n,
                                int32_t R, uint8_t* bits, cudaStream_t s);
 cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s);
-// E[e*R + r] = sum of the event's block partials, in block order.
+// E[e*R + r] = sum of the event's block partials, in a fixed order. gate (device, may
+// be NULL): does nothing unless (*gate != 0) == want.
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
-                                 int32_t R, double* E_out, cudaStream_t s);
+                                 int32_t R, double* E_out, const int32_t* gate, int want,
+                                 cudaStream_t s);
 // arg-min over replicas per event (ties -> lowest index).
 // err (device, may be NULL): where it is set, every energy becomes NaN
 cudaError_t launch_argmin(double* E_all, int32_t E, int32_t R, double* best_E, int32_t* best_r,

@@ -61,3 +61,46 @@ def test_one_replica_run(n, variant, prec):
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
         seen.append(got[0])
     assert not np.array_equal(seen[0], seen[1])
+
+
+def _ring(n):
+    """Rows joined to their neighbours at distance 1 (conflict) and 7 (consistent)."""
+    i = np.arange(n)
+    col = np.sort((i[:, None] + np.array([-7, -1, 1, 7])) % n, axis=1)
+    gap = np.abs(col - i[:, None])
+    cls = (np.minimum(gap, n - gap) == 1).astype(np.int8).ravel()
+    return inputs.QuboArrays(n, (4 * np.arange(n + 1)).astype(np.int32), col.ravel().astype(np.int32),
+                             np.where(cls, 1.0, -1.0), np.full(n, 0.3))
+
+
+@pytest.mark.parametrize("n,R", [(700, 8), (700, 50), (40000, 64), (200000, 4)])
+@pytest.mark.parametrize("first", [1.0, 0.6])
+def test_readout(n, R, first):
+    """Energies from selection bits need whole-number weights, which sb_set_weights
+    takes and gives; a fresh readout of another context is the reference."""
+    import torch
+    q = _ring(n)
+    ctx, other = (sb.sb_create(q.n, q.rowptr, q.col, q.val, q.lin) for _ in range(2))
+    rng = np.random.default_rng(n + R)
+    x = rng.uniform(-1, 1, size=(n, R)).astype(np.float32)
+    E, want = (torch.zeros((1, R), dtype=torch.float64, device="cuda") for _ in range(2))
+    b, r = torch.zeros(1, dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    _weights(ctx, q, first)
+    sb.sb_set_state(ctx, x, x)
+    sb.sb_readout_device(ctx, E, b, r, stream=stream)
+    g = _record(stream, lambda: sb.sb_readout_device(ctx, E, b, r, stream=stream))
+    for w_c in (first, 0.6, 1.0, 0.37, 2.0, first):
+        _weights(ctx, q, w_c)
+        _weights(other, q, w_c)
+        sb.sb_set_state(other, x, x)
+        sb.sb_readout_device(other, want)
+        sb.sb_readout_device(ctx, E, b, r)           # a fresh one, between two replays
+        torch.cuda.synchronize()
+        assert torch.allclose(E, want, rtol=1e-12, atol=0)
+        E.zero_()
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.allclose(E, want, rtol=1e-12, atol=0)
+        assert b.item() == E.min().item() and r.item() == E.argmin().item()
