@@ -645,8 +645,9 @@ sb_status ensure_state(sb_ctx* c, int32_t R) {
 }
 
 // Nothing here is freed while the replica count stays, whatever the weights become:
-// a readout that a caller has recorded keeps its buffers.
-sb_status ensure_readout(sb_ctx* c, int32_t R) {
+// a readout that a caller has recorded keeps its buffers. And nothing new is made for
+// the bits while one is being recorded: it takes the FP64 sums.
+sb_status ensure_readout(sb_ctx* c, int32_t R, bool recording) {
   sb_status st;
   if (c->eR != R || !c->eb[0].d_partial || !c->d_Eall) {
     free_readout(c);
@@ -655,7 +656,7 @@ sb_status ensure_readout(sb_ctx* c, int32_t R) {
       return st;
     c->eR = R;
   }
-  if (!c->b_whole || c->d_bits || c->bits_oom) return SB_OK;
+  if (!c->b_whole || c->d_bits || c->bits_oom || recording) return SB_OK;
   // whole-number couplings: larger blocks where that still leaves eight CTAs
   // per SM (fewer partial sums to add; the 472,812-row event: 2 ms of block sums)
   if (!c->sms) SB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
@@ -2622,7 +2623,10 @@ sb_status enqueue_steps(sb_ctx* c, int variant, double a0, double dt, int32_t st
 // d_Eall), arg-min into best_E / best_r (NULL: d_bestE / d_bestr).
 sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
                   double* E_all = nullptr, double* best_E = nullptr, int32_t* best_r = nullptr) {
-  sb_status st = ensure_readout(c, R);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  SB_CUDA(cudaStreamIsCapturing(s, &cap));
+  const bool recording = cap != cudaStreamCaptureStatusNone;
+  sb_status st = ensure_readout(c, R, recording);
   if (st) return st;
   if (!E_all) E_all = c->d_Eall;
   if (!best_E) best_E = c->d_bestE;
@@ -2631,10 +2635,8 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   // A readout that the caller records is replayed after sb_set_weights as well,
   // whose weights need not be whole numbers: both sums are recorded then, and
   // k_convert's verdict on the weights of the day picks one on the device.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool bits = c->b_whole && c->d_bits;
-  if (bits) SB_CUDA(cudaStreamIsCapturing(s, &cap));
-  const int32_t* const gate = cap == cudaStreamCaptureStatusNone ? nullptr : c->d_inexact;
+  const int32_t* const gate = bits && recording ? c->d_inexact : nullptr;
   if (bits) {
     sbd::EnergyBitArgs b;
     b.rowptr = c->d_rowptr;

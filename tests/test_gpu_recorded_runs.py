@@ -104,3 +104,25 @@ def test_readout(n, R, first):
         torch.cuda.synchronize()
         assert torch.allclose(E, want, rtol=1e-12, atol=0)
         assert b.item() == E.min().item() and r.item() == E.argmin().item()
+
+
+def test_readout_recorded_right_after_the_weights_became_whole():
+    """Buffers made for other weights serve the recording: it makes none of its own."""
+    import torch
+    n, R = 3000, 8
+    q = _ring(n)
+    ctx = sb.sb_create(q.n, q.rowptr, q.col, q.val, q.lin)
+    x = np.random.default_rng(1).uniform(-1, 1, size=(n, R)).astype(np.float32)
+    E = torch.zeros((1, R), dtype=torch.float64, device="cuda")
+    stream = torch.cuda.Stream()
+    _weights(ctx, q, 0.6)
+    sb.sb_set_state(ctx, x, x)
+    sb.sb_readout_device(ctx, E, stream=stream)
+    _weights(ctx, q, 1.0)
+    g = _record(stream, lambda: sb.sb_readout_device(ctx, E, stream=stream))
+    for w_c in (1.0, 0.6):
+        _weights(ctx, q, w_c)
+        g.replay()
+        torch.cuda.synchronize()
+        got = E.cpu().numpy()
+        assert np.allclose(got, sb.sb_energy(ctx, None, R), rtol=1e-12, atol=0)
