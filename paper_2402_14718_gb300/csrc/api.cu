@@ -2148,20 +2148,29 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
       return SB_OK;
     }
   }
-  if (c->use_stream) {
+  // A run of padded rows that the caller records reads the CSR in place: the tables
+  // of the other kernels go or move with new weights, a new factor or new options, and
+  // no kernel that takes the replica count itself has any, so a recorded run of that
+  // count has always outlived them; nor does it allocate.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (c->Rs != c->R) SB_CUDA(cudaStreamIsCapturing(stream, &cap));
+  const bool csr_only = cap != cudaStreamCaptureStatusNone;
+  const bool use_tiled = c->use_tiled && !csr_only, use_stream = c->use_stream && !csr_only;
+  const bool dsb_signs = c->dsb_signs && c->j_small && (!csr_only || (c->d_sgn[0] && c->d_sgn[1]));
+  if (use_stream) {
     sb_status st0 = ensure_stream(c);
     if (st0) return st0;
   }
-  if (c->use_tiled && c->Rs % sbd::kTileRT == 0) {
+  if (use_tiled && c->Rs % sbd::kTileRT == 0) {
     sb_status st0 = ensure_tiles(c);
     if (st0) return st0;
   }
   // factored coupling product: set, not switched off, a supported replica count;
   // dSB needs the sign bytes and U sums that BF16 holds exactly
   int fG = 0, fNCH = 0, ftiles = 0;
-  const int fac = (c->fac_set && c->fac_use != 0 && c->groups == 1 &&
+  const int fac = (c->fac_set && c->fac_use != 0 && c->groups == 1 && !csr_only &&
                    sbd::fac_tiling(variant, c->Rs, &fG, &fNCH, &ftiles) &&
-                   (variant != SB_DSB || (c->dsb_signs && c->j_small && c->n <= sbd::kFacRows)) &&
+                   (variant != SB_DSB || (dsb_signs && c->n <= sbd::kFacRows)) &&
                    (c->Rs == c->R || (variant == SB_DSB && c->b_whole)))
                       ? 1 : 0;
   // dSB: BF16 U rows hold sums of at most 256 members exactly; larger blocks
@@ -2270,7 +2279,7 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   // streamed kernel: chosen, tables valid, a supported replica count, and a ring that fits
   sbd::StreamArgs sa{};
   size_t s_smem = 0;
-  if (!fac && c->use_stream && c->stream_ok && c->groups == 1) {
+  if (!fac && use_stream && c->stream_ok && c->groups == 1) {
     sa.W = sbd::stream_tile_width(c->Rs);
     if (sa.W) s_smem = sbd::stream_smem(sa.W, c->stream_jbuf, &sa.nst);
   }
@@ -2281,8 +2290,8 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   // automatic choice: row groups of 2 for aSB / bSB, which gather FP32 x;
   // dSB keeps its sign-byte kernel (fewer instructions per neighbour)
   const int rw_want = c->rw_rows < 0 ? (variant == SB_DSB ? 0 : 2) : c->rw_rows;
-  const bool rw_auto_ok = c->rw_rows >= 0 || (!c->use_tiled && c->step_rt == 0);
-  if (!fac && !streamed && rw_want && rw_auto_ok && c->groups == 1 && c->Rs % 128 == 0) {
+  const bool rw_auto_ok = c->rw_rows >= 0 || (!use_tiled && c->step_rt == 0);
+  if (!fac && !streamed && !csr_only && rw_want && rw_auto_ok && c->groups == 1 && c->Rs % 128 == 0) {
     sb_status st0 = ensure_rw(c, rw_want);
     if (st0) return st0;
     if (c->rw_built == rw_want) {
@@ -2305,7 +2314,7 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
       ra.ngroups = c->rw_ngroups;
       ra.gpc = std::max(sbd::kRwBlock / 32, c->step_rpc > 0 ? c->step_rpc / rw : 0);
       ra.cta_order = nullptr;
-      const bool sgn_rw = variant == SB_DSB && c->dsb_signs && c->j_small;
+      const bool sgn_rw = variant == SB_DSB && dsb_signs;
       const int64_t ctas = ((int64_t)c->rw_ngroups + ra.gpc - 1) / ra.gpc;
       if (heavy_first(c, (size_t)c->n * c->Rs * (sgn_rw ? 1 : 4), ctas)) {
         st0 = ensure_rw_order(c, ra.gpc);
@@ -2365,10 +2374,10 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   }
   // the 16-replica dSB kernel exists only with sign bytes: its tiling and the
   // byte condition below must agree
-  const bool dsb16 = !fac && !streamed && !rw && variant == SB_DSB && c->dsb_signs && c->j_small &&
+  const bool dsb16 = !fac && !streamed && !rw && variant == SB_DSB && dsb_signs &&
                      c->step_rt == 0 &&
                      c->groups == 1 && sbd::dsb16_ok(c->Rs) && (int64_t)c->n * c->Rs > sbd::kDsb16Spins &&
-                     !(c->tiled_ok && c->use_tiled && c->Rs % sbd::kTileRT == 0);
+                     !(c->tiled_ok && use_tiled && c->Rs % sbd::kTileRT == 0);
   const sbd::Tiling t = dsb16 ? sbd::make_tiling_dsb16(c->Rs) : step_tiling(c);
   sbd::StepArgs a;
   a.rowptr = c->d_rowptr;
@@ -2405,14 +2414,14 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   a.r1_lanes = r1_lanes_for(c);
   if (dsb16) {
     const int rpc16 = sbd::dsb16_rows_per_cta(a.rpc);
-    if (heavy_first(c, (size_t)c->n * c->Rs, ((int64_t)c->n + rpc16 - 1) / rpc16)) {
+    if (!csr_only && heavy_first(c, (size_t)c->n * c->Rs, ((int64_t)c->n + rpc16 - 1) / rpc16)) {
       sb_status st2 = ensure_row_order(c, rpc16);
       if (st2) return st2;
       a.cta_order = c->d_row_order;
     }
   }
   const int tiled =
-      (!fac && !streamed && !rw && c->tiled_ok && c->use_tiled && c->Rs % sbd::kTileRT == 0) ? 1 : 0;
+      (!fac && !streamed && !rw && c->tiled_ok && use_tiled && c->Rs % sbd::kTileRT == 0) ? 1 : 0;
   sbd::TiledArgs ta;
   ta.blk_row0 = c->d_blk_row0;
   ta.blk_u0 = c->d_blk_u0;
@@ -2431,7 +2440,7 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   ta.n = c->n;
   ta.R = c->Rs;
   ta.nb = c->nb;
-  const int sgn = (variant == SB_DSB && c->dsb_signs && c->j_small && !tiled && !streamed &&
+  const int sgn = (variant == SB_DSB && dsb_signs && !tiled && !streamed &&
                    c->Rs % 4 == 0) ? 1 : 0;
   if (sgn && !(c->d_sgn[0] && c->d_sgn[1])) {
     dfree(c->d_sgn[0]);  // a failed earlier attempt may have left one of the pair

@@ -6,6 +6,7 @@ import pytest
 
 import paper_2402_14718_gb300 as sb
 from tests import inputs
+from tests import test_gpu_factor_blocks as blocks
 
 pytestmark = pytest.mark.gpu
 
@@ -126,3 +127,51 @@ def test_readout_recorded_right_after_the_weights_became_whole():
         torch.cuda.synchronize()
         got = E.cpu().numpy()
         assert np.allclose(got, sb.sb_energy(ctx, None, R), rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("variant", ["dsb", "bsb", "asb"])
+@pytest.mark.parametrize("R", [6, 50, 127])
+@pytest.mark.parametrize("warm", [False, True])
+def test_padded_run(variant, R, warm):
+    """Replica counts that are stored padded, with a factor set, recorded before any other
+    run of the context or after one: the recorded run takes what the kernels for the
+    count itself took, the CSR, and outlives the factor and the weights."""
+    import torch
+    q, member, couple = blocks._grouped((3, 8, 40, 130), 3, 1)
+    n = len(q[3])
+    rng = np.random.default_rng(R)
+    x = rng.uniform(-1, 1, size=(n, R)).astype(np.float32)
+    y = rng.uniform(-0.3, 0.3, size=(n, R)).astype(np.float32)
+    sched = torch.linspace(0.2, 0.6, 4, device="cuda")
+    dt = 0.1 if variant == "asb" else 0.4
+    stream = torch.cuda.Stream()
+
+    def make():
+        ctx = sb.sb_create(n, *q, sb.SB_J_BF16)
+        sb.sb_set_factor(ctx, 4, member, couple, 1.0)
+        return ctx
+
+    def advance(ctx):
+        sb.sb_advance(ctx, variant, 1.0, 0.05, dt, 4, sched, stream=stream)
+
+    ctx, other = make(), make()
+    sb.sb_set_option(other, sb.SB_OPT_FACTOR, 0)
+    sb.sb_set_state(ctx, x, y)
+    if warm:
+        advance(ctx)
+        sb.sb_set_state(ctx, x, y)
+    g = _record(stream, lambda: advance(ctx))
+    assert sb.sb_step_kernels(ctx) in ("k_step", "k_step_dsb16")
+    qa = inputs.QuboArrays(n, *q)
+    for w_c in (None, 1.0, 0.25):
+        if w_c:
+            for c in (ctx, other):
+                _weights(c, qa, w_c)
+        sb.sb_set_state(other, x, y)
+        advance(other)
+        want = sb.sb_get_state(other)
+        for _ in range(2):
+            sb.sb_set_state(ctx, x, y)
+            g.replay()
+            got = sb.sb_get_state(ctx)
+            assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
