@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
@@ -117,6 +118,7 @@ struct sb_ctx {
   float* d_y = nullptr;
   int cur = 0;
   const char* step_kernels = "";  // kernels of the last steps (sb_step_kernels)
+  mutable std::mutex get_mutex;    // padded states come out through the other x buffer
   bool have_state = false;
   float* d_sched = nullptr;  // default linear schedule
   int32_t sched_len = 0;
@@ -3085,10 +3087,12 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
   SB_CUDA(cudaDeviceSynchronize());
   const float *const sx = ctx->d_x[ctx->cur], *const sy = ctx->d_y;
   const bool padded = ctx->Rs != ctx->R;
+  std::unique_lock<std::mutex> one_at_a_time(ctx->get_mutex, std::defer_lock);
   if (padded && on_device && (!x || own_memory(ctx, x, 4)) && (!y || own_memory(ctx, y, 4))) {
     SB_CUDA(sbd::launch_repitch(x ? sx : sy, x && y ? sy : nullptr, ctx->Rs, x ? x : y, y, ctx->R,
                                 ctx->n, ctx->R, 0));
   } else {
+    if (padded) one_at_a_time.lock();
     for (int q = 0; q < 2; ++q) {
       float* const out = q ? y : x;
       const float* src = q ? sy : sx;

@@ -66,3 +66,23 @@ def test_both_arrays_or_one(n, R):
                                           b.data_ptr() if want_y else None, 1))
         assert torch.equal(a, x) if want_x else bool((a == 7.0).all())
         assert torch.equal(b, y) if want_y else bool((b == 7.0).all())
+
+
+@pytest.mark.parametrize("R", [50, 64])
+def test_get_state_from_several_threads(R):
+    """sb_get_state reads a context that it does not change: threads may call it at once."""
+    from concurrent.futures import ThreadPoolExecutor
+    n = 30000
+    ctx = sb.sb_create(n, np.zeros(n + 1, np.int32), np.zeros(0, np.int32), np.zeros(0), np.zeros(n))
+    rng = np.random.default_rng(R)
+    x, y = (rng.random((n, R), dtype=np.float32) for _ in range(2))
+    sb.sb_set_state(ctx, x, y)
+
+    def get(k):
+        out = np.zeros((n, R), np.float32)
+        p = out.ctypes.data
+        sb._lib.check(sb.lib.sb_get_state(ctx.handle, p if k % 2 else None, None if k % 2 else p, 0))
+        return np.array_equal(out, x if k % 2 else y)
+
+    with ThreadPoolExecutor(8) as ex:
+        assert all(ex.map(get, range(160)))
