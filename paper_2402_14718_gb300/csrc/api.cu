@@ -1,5 +1,6 @@
 // C ABI of the SB solver: context life cycle, QUBO -> Ising set-up, SB runs
 // (one launch per step, replayed from a captured CUDA graph), FP64 readout.
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <stdio.h>
 #include <string.h>
@@ -613,15 +614,39 @@ int32_t padded_replicas(int32_t R) {
   return (int64_t)3 * p <= (int64_t)4 * R ? p : (R + 3) / 4 * 4;
 }
 
-// memory of the context's device, aligned to a bytes: what a kernel may be given
-bool own_memory(const sb_ctx* c, const void* p, size_t a) {
-  cudaPointerAttributes at;
-  if (!p || reinterpret_cast<uintptr_t>(p) % a) return false;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// `bytes` of memory of the context's device at p, aligned to a bytes and allocated (or
+// mapped piece by piece without a gap) to the last one, which a copy checks and a
+// kernel does not: what a kernel may be given.
+bool own_memory(const sb_ctx* c, const void* p, size_t bytes, size_t a) {
+  static const PFN_cuPointerGetAttributes_v7000 attributes = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &q) !=
+            cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(f);
+  }();
+  if (!attributes || !p || reinterpret_cast<uintptr_t>(p) % a) return false;
+  CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                 CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  const CUdeviceptr end = at + bytes;
+  while (at < end) {
+    unsigned type = 0, managed = 0;
+    int device = -1;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    void* out[5] = {&type, &device, &managed, &base, &size};
+    if (attributes(5, what, out, at) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed ||
+        device != c->device || base + size <= at)
+      return false;
+    at = base + size;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == c->device;
+  return true;
 }
 
 sb_status ensure_state(sb_ctx* c, int32_t R) {
@@ -3055,7 +3080,7 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
     if (ctx->Rs == replicas) {
       SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
       SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
-    } else if (on_device && own_memory(ctx, x, 4) && own_memory(ctx, y, 4)) {
+    } else if (on_device && own_memory(ctx, x, bytes, 4) && own_memory(ctx, y, bytes, 4)) {
       SB_CUDA(sbd::launch_repitch(x, y, replicas, ctx->d_x[0], ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
     } else {  // both through the x buffers, then into the padded rows
       SB_CUDA(cudaMemcpy(ctx->d_x[0], y, bytes, k));
@@ -3088,7 +3113,8 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
   const float *const sx = ctx->d_x[ctx->cur], *const sy = ctx->d_y;
   const bool padded = ctx->Rs != ctx->R;
   std::unique_lock<std::mutex> one_at_a_time(ctx->get_mutex, std::defer_lock);
-  if (padded && on_device && (!x || own_memory(ctx, x, 4)) && (!y || own_memory(ctx, y, 4))) {
+  if (padded && on_device && (!x || own_memory(ctx, x, bytes, 4)) &&
+      (!y || own_memory(ctx, y, bytes, 4))) {
     SB_CUDA(sbd::launch_repitch(x ? sx : sy, x && y ? sy : nullptr, ctx->Rs, x ? x : y, y, ctx->R,
                                 ctx->n, ctx->R, 0));
   } else {
@@ -3151,10 +3177,11 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
     }
     cudaStream_t s = (cudaStream_t)stream;
     // the kernels write the caller's buffers themselves where they are aligned
-    // for their type and lie on the context's own device, else through the
+    // for their type, long enough and on the context's own device, else through the
     // context's own and a copy (which refuses what is no device memory)
-    auto direct = [&](void* p, size_t a) { return own_memory(ctx, p, a); };
-    const bool dE = direct(d_E_all, 8), db = direct(d_best_E, 8), dr = direct(d_best_r, 4);
+    auto direct = [&](void* p, size_t count, size_t a) { return own_memory(ctx, p, count * a, a); };
+    const bool dE = direct(d_E_all, (size_t)ctx->E * ctx->R, 8), db = direct(d_best_E, ctx->E, 8),
+               dr = direct(d_best_r, ctx->E, 4);
     sb_status st = readout(ctx, nullptr, ctx->R, s, dE ? d_E_all : nullptr,
                            db ? d_best_E : nullptr, dr ? d_best_r : nullptr);
     if (st) return st;

@@ -86,3 +86,46 @@ def test_get_state_from_several_threads(R):
 
     with ThreadPoolExecutor(8) as ex:
         assert all(ex.map(get, range(160)))
+
+
+@pytest.mark.parametrize("pieces", [False, True])
+def test_buffers_that_end_with_their_memory(pieces):
+    """A kernel is given a buffer only when all of it is allocated: ones that fill their
+    allocation to the last byte, and ones that torch maps in several pieces, count."""
+    import torch
+    n, R = 65536, 50  # 12.5 MiB: exactly 6.25 pieces of 2 MiB
+    code = f"""if True:
+        import ctypes, torch
+        import paper_2402_14718_gb300 as sb
+        import numpy as np
+        rt = ctypes.CDLL("libcudart.so.13")
+        rt.cudaMemcpy.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
+        n, R, pieces = {n}, {R}, {pieces}
+        ctx = sb.sb_create(n, np.zeros(n + 1, np.int32), np.zeros(0, np.int32), np.zeros(0), np.zeros(n))
+        x = torch.rand((n, R), device="cuda")
+        y = x + 1
+        if pieces:
+            a, b = torch.zeros_like(x), torch.zeros_like(x)
+            pa, pb = a.data_ptr(), b.data_ptr()
+        else:
+            pa, pb = ctypes.c_void_p(), ctypes.c_void_p()
+            assert rt.cudaMalloc(ctypes.byref(pa), ctypes.c_size_t(n * R * 4)) == 0
+            assert rt.cudaMalloc(ctypes.byref(pb), ctypes.c_size_t(n * R * 4)) == 0
+            a, b = torch.zeros_like(x), torch.zeros_like(x)
+        sb.sb_set_state(ctx, x, y)
+        sb._lib.check(sb.lib.sb_get_state(ctx.handle, pa, pb, 1))
+        if not pieces:
+            rt.cudaMemcpy(a.data_ptr(), pa, n * R * 4, 3)
+            rt.cudaMemcpy(b.data_ptr(), pb, n * R * 4, 3)
+        assert torch.equal(a, x) and torch.equal(b, y)
+    """
+    import os
+    import subprocess
+    import sys
+    env = dict(os.environ)
+    if pieces:
+        env["PYTORCH_CUDA_ALLOC_CONF"] = "expandable_segments:True"
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
