@@ -2695,7 +2695,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
     SB_CUDA(sbd::launch_energy_reduce(b.partial, c->eb[1].d_ev0, c->E, R, E_all, gate, 0, s));
   }
   if (bits && !gate) {
-    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
+    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, c->d_bestr, err, s));
     return SB_OK;
   }
   const sbd::Tiling t = sbd::make_tiling(R);
@@ -2717,7 +2717,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   a.nnz = c->nnz;
   SB_CUDA(sbd::launch_energy_partial(t, a, s));
   SB_CUDA(sbd::launch_energy_reduce(a.partial, c->eb[0].d_ev0, c->E, R, E_all, gate, 1, s));
-  SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, err, s));
+  SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, c->d_bestr, err, s));
   return SB_OK;
 }
 
@@ -3186,8 +3186,8 @@ sb_status sb_readout_device(sb_ctx* ctx, double* d_E_all, double* d_best_E, int3
                            db ? d_best_E : nullptr, dr ? d_best_r : nullptr);
     if (st) return st;
     if (d_T)
-      SB_CUDA(sbd::launch_best_T(ctx->d_x[ctx->cur], ctx->d_row_event,
-                                 dr ? d_best_r : ctx->d_bestr, ctx->n, ctx->Rs, d_T, s));
+      SB_CUDA(sbd::launch_best_T(ctx->d_x[ctx->cur], ctx->d_row_event, ctx->d_bestr, ctx->n,
+                                 ctx->Rs, d_T, s));
     if (d_E_all && !dE)
       SB_CUDA(cudaMemcpyAsync(d_E_all, ctx->d_Eall, (size_t)ctx->E * ctx->R * 8,
                               cudaMemcpyDeviceToDevice, s));

@@ -1464,8 +1464,11 @@ __device__ __forceinline__ bool better(double v, int r, double bv, int br) {
 
 // warp-shuffle arg-min over the replicas of one event. *err (may be NULL) is the
 // flag that a step kernel sets when one of its bounded waits gave up: the state is
-// not valid then, and every energy becomes NaN.
-__global__ void k_argmin(double* E_all, int32_t R, double* best_E, int32_t* best_r, const int* err) {
+// not valid then, and every energy becomes NaN. own_r (may be NULL): best_r once more,
+// for k_best_T, which takes it as an index and must not find it in memory that the
+// caller may be writing.
+__global__ void k_argmin(double* E_all, int32_t R, double* best_E, int32_t* best_r, int32_t* own_r,
+                         const int* err) {
   __shared__ double sv[32];
   __shared__ int sr[32];
   const int e = blockIdx.x;
@@ -1508,7 +1511,9 @@ __global__ void k_argmin(double* E_all, int32_t R, double* best_E, int32_t* best
     }
     if (lane == 0) {
       best_E[e] = bad ? nan : bv;
-      best_r[e] = br == INT_MAX ? 0 : br;
+      br = br == INT_MAX ? 0 : br;
+      best_r[e] = br;
+      if (own_r) own_r[e] = br;
     }
   }
   if (bad)
@@ -1812,9 +1817,9 @@ cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_argmin(double* E_all, int32_t E, int32_t R, double* best_E, int32_t* best_r,
-                          const int* err, cudaStream_t s) {
+                          int32_t* own_r, const int* err, cudaStream_t s) {
   if (E <= 0) return cudaSuccess;
-  k_argmin<<<E, kBlock, 0, s>>>(E_all, R, best_E, best_r, err);
+  k_argmin<<<E, kBlock, 0, s>>>(E_all, R, best_E, best_r, own_r, err);
   return cudaGetLastError();
 }
 

@@ -172,9 +172,10 @@ cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, 
                                  int32_t R, double* E_out, const int32_t* gate, int want,
                                  cudaStream_t s);
 // arg-min over replicas per event (ties -> lowest index).
-// err (device, may be NULL): where it is set, every energy becomes NaN
+// own_r (device, may be NULL): best_r once more; err (device, may be NULL): where it
+// is set, every energy becomes NaN
 cudaError_t launch_argmin(double* E_all, int32_t E, int32_t R, double* best_E, int32_t* best_r,
-                          const int* err, cudaStream_t s);
+                          int32_t* own_r, const int* err, cudaStream_t s);
 cudaError_t launch_best_T(const float* x, const int32_t* row_event, const int32_t* best_r,
                           int32_t n, int32_t xstride, uint8_t* T, cudaStream_t s);
 

@@ -175,3 +175,20 @@ def test_padded_run(variant, R, warm):
             g.replay()
             got = sb.sb_get_state(ctx)
             assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+def test_selection_of_the_best_replica_reads_no_caller_memory():
+    """best_r and T in one buffer: beyond the four bytes that they share, T is still the
+    best replica's."""
+    import torch
+    q = inputs.random_qubo(300, 9, 5)
+    ctx = sb.sb_create(q.n, q.rowptr, q.col, q.val, q.lin)
+    sb.sb_run(ctx, "bsb", 1.0, 0.3, 0.4, 20, 8, seed=3)
+    T, _, r = sb.sb_best(ctx)
+    assert r[0] != 0
+    buf = torch.zeros(512, dtype=torch.uint8, device="cuda")
+    for _ in range(20):
+        buf.zero_()
+        sb.sb_readout_device(ctx, None, None, buf[:4].view(torch.int32), buf[:300])
+        torch.cuda.synchronize()
+        assert np.array_equal(buf[4:300].cpu().numpy(), T[4:])
