@@ -12,6 +12,7 @@
 #include <new>
 #include <string>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "../../include/sb.h"
@@ -268,10 +269,9 @@ struct sb_ctx {
     int built = 0;           // 0: not tried, 1: tables ready, -1: does not fit
     int32_t nct = 0, nx = 0, max_ent = 0;
     size_t smem = 0;
+    char* d_mem = nullptr;   // one allocation for all of the following
     sbd::Run1Cta* d_cta = nullptr;
     int32_t *d_perm = nullptr, *d_deg = nullptr, *d_slice = nullptr, *d_ucol = nullptr;
-    int64_t ents = 0;            // entries, padding included
-    int32_t* d_pos = nullptr;    // CSR position of each entry (-1: padding)
     float* d_ej = nullptr;
     uint16_t* d_ei = nullptr;
     unsigned long long* d_word = nullptr;
@@ -454,18 +454,8 @@ void free_adj(sb_ctx* c) {
 }
 
 void free_run1(sb_ctx* c) {
-  sb_ctx::Run1& r = c->run1;
-  if (r.d_cta) cudaFree(r.d_cta);
-  r.d_cta = nullptr;
-  dfree(r.d_perm);
-  dfree(r.d_deg);
-  dfree(r.d_slice);
-  dfree(r.d_ucol);
-  dfree(r.d_pos);
-  dfree(r.d_ej);
-  dfree(r.d_ei);
-  dfree(r.d_word);
-  r.built = 0;
+  dfree(c->run1.d_mem);
+  c->run1 = sb_ctx::Run1();
 }
 
 void free_factor(sb_ctx* c) {
@@ -1967,12 +1957,14 @@ sbd::Tiling step_tiling(const sb_ctx* c) {
   return sbd::make_tiling(c->Rs);
 }
 
-// The entries of k_run_r1's tables from the current J, in place: a run that a caller
+// The couplings in k_run_r1's tables from the current J, in place: a run that a caller
 // has recorded keeps its addresses and takes the new couplings, as the step
-// kernels do, which read J itself.
-sb_status refill_run1(sb_ctx* c) {
-  if (c->run1.built <= 0) return SB_OK;
-  SB_CUDA(sbd::launch_fill_run1(c->d_J, c->jbf16, c->run1.d_pos, c->run1.ents, c->run1.d_ej, 0));
+// kernels do, which read J itself. With `all`, the entries' indices too.
+sb_status fill_run1(sb_ctx* c, bool all) {
+  const sb_ctx::Run1& r = c->run1;
+  if (r.built <= 0) return SB_OK;
+  SB_CUDA(sbd::launch_fill_run1(r.d_cta, r.nct, r.d_perm, r.d_deg, r.d_slice, r.d_ucol, c->d_rowptr,
+                                c->d_col, c->d_J, c->jbf16, r.d_ej, all ? r.d_ei : nullptr, 0));
   SB_CUDA(cudaStreamSynchronize(0));
   return SB_OK;
 }
@@ -1984,6 +1976,11 @@ sb_status refill_run1(sb_ctx* c) {
 // memory: the step kernels serve the run. CTAs: one per 1,024 nonzeros or 128
 // rows, at most one per SM (us per step with 16 / 48 / 152 CTAs: 1,721 rows 1.7 /
 // 1.8 / 1.7; 10,214 rows 1.7 / 1.5 / 1.5; 10,878 rows does not fit / 2.2 / 2.2).
+// The host orders the rows and collects the unions, which is all that it takes to
+// see whether they fit; the entries are filled in on the device, in one allocation.
+// What they add to the run that builds them, us (entries made on the host, eight
+// allocations / so): 1,879 rows, 28 k nonzeros, 2200 / 70; 10,999 rows, 221 k, 2300 / 460;
+// 39,445 rows, 1.8 M, 3600 / 850; 98,134 rows, 5.7 M, which do not fit, 5800 / 130.
 sb_status ensure_run1(sb_ctx* c) {
   sb_ctx::Run1& r = c->run1;
   if (r.built) return SB_OK;
@@ -2013,109 +2010,112 @@ sb_status ensure_run1(sb_ctx* c) {
                        std::min(at, lo + sbd::kRun1Threads));
   }
   if (n - row0[nct - 1] > sbd::kRun1Threads) return SB_OK;
+  std::vector<int32_t> perm((size_t)n), deg((size_t)n);
   struct Part {
-    std::vector<int32_t> perm, deg, slice, ucol, pos;
-    std::vector<uint16_t> ei;
-    bool ok = true;
+    std::vector<int32_t> slice, ucol;
+    int64_t nent = 0;
   };
   std::vector<Part> P((size_t)nct);
-  const int parts = std::min(nct, 32);
-  const bool built = parallel_parts(nct, parts, [&](int, int64_t b0, int64_t b1) {
-    std::vector<int32_t> local((size_t)n, -1);  // index in the union (-1 between CTAs)
-    for (int64_t b = b0; b < b1; ++b) {
+  std::atomic<bool> fits{true};
+  // host threads pay from about this many nonzeros on
+  const int parts = nnz < 600000 ? 1 : std::min(nct, 32);
+  auto chunks = [&](int, int64_t b0, int64_t b1) {
+    std::vector<uint64_t> seen(((size_t)n + 63) / 64, 0);  // columns of the chunk's union
+    std::vector<int32_t> first;                            // first slot of each degree, descending
+    for (int64_t b = b0; b < b1 && fits; ++b) {
       Part& q = P[(size_t)b];
       const int32_t r0 = row0[b], r1 = row0[b + 1];
-      for (int32_t i = r0; i < r1; ++i) q.perm.push_back(i);
-      std::stable_sort(q.perm.begin(), q.perm.end(), [&](int32_t i, int32_t j) {
-        return rp[i + 1] - rp[i] > rp[j + 1] - rp[j];
-      });
-      for (int32_t p = rp[r0]; p < rp[r1]; ++p)
-        if (local[col[p]] < 0) {
-          local[col[p]] = 0;
-          q.ucol.push_back(col[p]);
-        }
-      std::sort(q.ucol.begin(), q.ucol.end());
-      q.ok = q.ucol.size() <= 65535;
-      for (size_t u = 0; u < q.ucol.size(); ++u) local[q.ucol[u]] = (int32_t)u;
-      for (int32_t s = 0; s < r1 - r0; s += 32) {
-        const int32_t len = (rp[q.perm[s] + 1] - rp[q.perm[s]] + 7) / 8 * 8;
-        const size_t e0 = q.pos.size();
-        q.slice.push_back((int32_t)e0);
-        q.pos.resize(e0 + (size_t)len * 32, -1);
-        q.ei.resize(e0 + (size_t)len * 32, 0);
-        for (int32_t l = 0; l < 32 && s + l < r1 - r0; ++l) {
-          const int32_t row = q.perm[s + l], d = rp[row + 1] - rp[row];
-          q.deg.push_back(d);
-          for (int32_t k = 0; k < d; ++k) {
-            const int32_t p = rp[row] + k;
-            const size_t e = e0 + (size_t)(k / 4) * 128 + 4 * l + k % 4;
-            q.pos[e] = p;
-            q.ei[e] = (uint16_t)local[col[p]];
-          }
-        }
+      int32_t dmax = 0;
+      for (int32_t i = r0; i < r1; ++i) dmax = std::max(dmax, rp[i + 1] - rp[i]);
+      first.assign((size_t)dmax + 2, 0);
+      for (int32_t i = r0; i < r1; ++i) ++first[dmax - (rp[i + 1] - rp[i]) + 1];
+      for (int32_t d = 0; d <= dmax; ++d) first[d + 1] += first[d];
+      for (int32_t i = r0; i < r1; ++i) {
+        const int32_t d = rp[i + 1] - rp[i], k = r0 + first[dmax - d]++;
+        perm[k] = i;
+        deg[k] = d;
       }
-      for (int32_t u : q.ucol) local[u] = -1;
+      for (int32_t s = r0; s < r1; s += 32) {
+        q.slice.push_back((int32_t)q.nent);
+        q.nent += (deg[s] + 7) / 8 * 8 * 32;
+        if (q.nent * 6 > sbd::kRun1Smem) break;
+      }
+      if (q.nent * 6 > sbd::kRun1Smem) {
+        fits = false;
+        return;
+      }
+      int32_t w0 = (int32_t)seen.size(), w1 = -1;
+      for (int32_t p = rp[r0]; p < rp[r1]; ++p) {
+        const int32_t w = col[p] >> 6;
+        seen[w] |= 1ull << (col[p] & 63);
+        w0 = std::min(w0, w);
+        w1 = std::max(w1, w);
+      }
+      for (int32_t w = w0; w <= w1; ++w)
+        for (uint64_t m = std::exchange(seen[w], 0); m; m &= m - 1)
+          q.ucol.push_back(w * 64 + __builtin_ctzll(m));
+      if (q.ucol.size() > 65535 || q.nent * 6 + (int64_t)q.ucol.size() * 4 > sbd::kRun1Smem) fits = false;
     }
+  };
+  chunks(0, 0, 1);  // where the first chunk does not fit, no thread is started
+  if (!fits) return SB_OK;
+  const bool built = parallel_parts(nct - 1, parts, [&](int p, int64_t b0, int64_t b1) {
+    chunks(p, b0 + 1, b1 + 1);
   }, 1);
-  if (!built) return SB_OK;  // no host memory for the tables
+  if (!built || !fits) return SB_OK;  // no host memory, or no room in shared memory
   std::vector<sbd::Run1Cta> cta((size_t)nct);
-  std::vector<int32_t> perm, deg, slice, ucol;
-  size_t ents = 0, max_ent = 0, max_u = 0;
-  bool ok = true;
+  int64_t ents = 0, max_ent = 0, max_u = 0, nsl = 0, nu = 0;
   for (int32_t b = 0; b < nct; ++b) {
     const Part& q = P[(size_t)b];
-    ok = ok && q.ok;
-    cta[b] = {row0[b], row0[b + 1] - row0[b], (int32_t)ents, (int32_t)q.pos.size(),
-              (int32_t)slice.size(), (int32_t)ucol.size(), (int32_t)q.ucol.size(), 0};
-    ents += q.pos.size();
-    max_ent = std::max(max_ent, q.pos.size());
-    max_u = std::max(max_u, q.ucol.size());
-    perm.insert(perm.end(), q.perm.begin(), q.perm.end());
-    deg.insert(deg.end(), q.deg.begin(), q.deg.end());
-    slice.insert(slice.end(), q.slice.begin(), q.slice.end());
-    ucol.insert(ucol.end(), q.ucol.begin(), q.ucol.end());
+    cta[b] = {row0[b], row0[b + 1] - row0[b], (int32_t)ents, (int32_t)q.nent, (int32_t)nsl, (int32_t)nu,
+              (int32_t)q.ucol.size(), 0};
+    ents += q.nent;
+    nsl += (int64_t)q.slice.size();
+    nu += (int64_t)q.ucol.size();
+    max_ent = std::max(max_ent, q.nent);
+    max_u = std::max(max_u, (int64_t)q.ucol.size());
   }
   const int32_t nx = (int32_t)((max_u + 3) / 4 * 4);
-  const size_t smem = (size_t)nx * 4 + max_ent * 6 + 16;
-  if (!ok || ents > (size_t)INT32_MAX || smem > (size_t)sbd::kRun1Smem ||
+  const size_t smem = (size_t)nx * 4 + (size_t)max_ent * 6 + 16;
+  if (ents > INT32_MAX || nu > INT32_MAX || smem > (size_t)sbd::kRun1Smem ||
       sbd::run1_blocks_per_sm(smem) < 1)
     return SB_OK;
-  std::vector<int32_t> pos(std::max<size_t>(ents, 4), -1);
-  std::vector<uint16_t> ei(std::max<size_t>(ents, 4));
-  parallel_parts(nct, parts, [&](int, int64_t b0, int64_t b1) {
-    for (int64_t b = b0; b < b1; ++b) {
-      std::copy(P[b].pos.begin(), P[b].pos.end(), pos.begin() + cta[b].ent0);
-      std::copy(P[b].ei.begin(), P[b].ei.end(), ei.begin() + cta[b].ent0);
-    }
-  }, 1);
-  if (cudaMalloc(&r.d_cta, cta.size() * sizeof(sbd::Run1Cta)) != cudaSuccess) {
-    cudaGetLastError();
-    r.d_cta = nullptr;
-    return SB_OK;  // no memory for the tables: the step kernels serve the run
+  // [cta][perm][deg][slice][ucol], copied from the host, then [ej][ei][word]
+  size_t bytes = 0;
+  auto place = [&](size_t size) {
+    const size_t o = bytes;
+    bytes += (size + 255) / 256 * 256;
+    return o;
+  };
+  const size_t o_cta = place(cta.size() * sizeof(sbd::Run1Cta)), o_perm = place((size_t)n * 4),
+               o_deg = place((size_t)n * 4), o_slice = place((size_t)nsl * 4), o_ucol = place((size_t)nu * 4);
+  std::vector<char> host(bytes);
+  const size_t o_ej = place((size_t)ents * 4), o_ei = place((size_t)ents * 2),
+               o_word = place((size_t)n * 2 * sizeof(unsigned long long));
+  memcpy(&host[o_cta], cta.data(), cta.size() * sizeof(sbd::Run1Cta));
+  memcpy(&host[o_perm], perm.data(), (size_t)n * 4);
+  memcpy(&host[o_deg], deg.data(), (size_t)n * 4);
+  for (int32_t b = 0; b < nct; ++b) {
+    const Part& q = P[(size_t)b];
+    if (!q.slice.empty()) memcpy(&host[o_slice + (size_t)cta[b].slice0 * 4], q.slice.data(), q.slice.size() * 4);
+    if (!q.ucol.empty()) memcpy(&host[o_ucol + (size_t)cta[b].u0 * 4], q.ucol.data(), q.ucol.size() * 4);
   }
-  if (dalloc(&r.d_perm, perm.size()) || dalloc(&r.d_deg, deg.size()) ||
-      dalloc(&r.d_slice, std::max<size_t>(slice.size(), 1)) ||
-      dalloc(&r.d_ucol, std::max<size_t>(ucol.size(), 1)) || dalloc(&r.d_ej, pos.size()) ||
-      dalloc(&r.d_pos, pos.size()) || dalloc(&r.d_ei, ei.size()) || dalloc(&r.d_word, (size_t)2 * n)) {
-    free_run1(c);
-    r.built = -1;
-    return SB_OK;
-  }
-  SB_CUDA(cudaMemcpy(r.d_cta, cta.data(), cta.size() * sizeof(sbd::Run1Cta), cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_perm, perm.data(), perm.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_deg, deg.data(), deg.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_slice, slice.data(), slice.size() * 4, cudaMemcpyHostToDevice));
-  if (!ucol.empty())
-    SB_CUDA(cudaMemcpy(r.d_ucol, ucol.data(), ucol.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_pos, pos.data(), pos.size() * 4, cudaMemcpyHostToDevice));
-  SB_CUDA(cudaMemcpy(r.d_ei, ei.data(), ei.size() * 2, cudaMemcpyHostToDevice));
+  if (dalloc(&r.d_mem, bytes)) return SB_OK;  // no memory for the tables: the step kernels serve the run
+  r.d_cta = reinterpret_cast<sbd::Run1Cta*>(r.d_mem + o_cta);
+  r.d_perm = reinterpret_cast<int32_t*>(r.d_mem + o_perm);
+  r.d_deg = reinterpret_cast<int32_t*>(r.d_mem + o_deg);
+  r.d_slice = reinterpret_cast<int32_t*>(r.d_mem + o_slice);
+  r.d_ucol = reinterpret_cast<int32_t*>(r.d_mem + o_ucol);
+  r.d_ej = reinterpret_cast<float*>(r.d_mem + o_ej);
+  r.d_ei = reinterpret_cast<uint16_t*>(r.d_mem + o_ei);
+  r.d_word = reinterpret_cast<unsigned long long*>(r.d_mem + o_word);
+  SB_CUDA(cudaMemcpy(r.d_mem, host.data(), host.size(), cudaMemcpyHostToDevice));
   r.nct = nct;
   r.nx = nx;
   r.max_ent = (int32_t)max_ent;
   r.smem = smem;
-  r.ents = (int64_t)pos.size();
   r.built = 1;
-  const sb_status st = refill_run1(c);
+  const sb_status st = fill_run1(c, true);
   if (st) r.built = -1;
   return st;
 }
@@ -3292,7 +3292,7 @@ sb_status sb_set_weights(sb_ctx* ctx, const int8_t* cls, const double* quality, 
     // the factored form's weight and residual were formed for the old couplings
     free_factor(ctx);
     if ((st = refill_rw(ctx))) return st;
-    if ((st = refill_run1(ctx))) return st;
+    if ((st = fill_run1(ctx, false))) return st;
     SB_CUDA(cudaMemcpy(ctx->offset.data(), ctx->d_offset, 8, cudaMemcpyDeviceToHost));
     SB_CUDA(cudaMemcpy(ctx->sigma.data(), ctx->d_sigma, 8, cudaMemcpyDeviceToHost));
     SB_CUDA(cudaMemcpy(ctx->c0_auto.data(), ctx->d_c0auto, 8, cudaMemcpyDeviceToHost));

@@ -299,8 +299,11 @@ struct Run1Args {
 };
 cudaError_t run1_prepare();  // raise the kernels' shared-memory limit (once per device)
 int run1_blocks_per_sm(size_t smem);  // resident CTAs per SM (0: it does not fit)
-// ej[e] = J[pos[e]] (0 where pos[e] < 0)
-cudaError_t launch_fill_run1(const void* J, int jbf16, const int32_t* pos, int64_t count, float* ej,
+// the entries of nct CTAs: weights ej from J and, where ei is not NULL, each column's
+// index in its CTA's (ascending) union
+cudaError_t launch_fill_run1(const Run1Cta* cta, int nct, const int32_t* perm, const int32_t* deg,
+                             const int32_t* slice, const int32_t* ucol, const int32_t* rowptr,
+                             const int32_t* col, const void* J, int jbf16, float* ej, uint16_t* ei,
                              cudaStream_t s);
 cudaError_t launch_run_r1(int variant, const Run1Args& a, size_t smem, cudaStream_t s);
 

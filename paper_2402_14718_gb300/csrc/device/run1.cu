@@ -190,12 +190,40 @@ __global__ void __launch_bounds__(kRun1Threads, 1) k_run_r1(const Run1Args a) {
   }
 }
 
+// A warp fills one slot's entries, padding included (weight 0, index 0).
 template <typename JT>
-__global__ void k_fill_run1(const JT* J, const int32_t* pos, int64_t count, float* ej) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t p = pos[i];
-    ej[i] = p >= 0 ? (float)J[p] : 0.f;
+__global__ void __launch_bounds__(256) k_fill_run1(const Run1Cta* cta, const int32_t* perm, const int32_t* deg,
+                                                   const int32_t* slice, const int32_t* ucol,
+                                                   const int32_t* rowptr, const int32_t* col, const JT* J,
+                                                   float* ej, uint16_t* ei) {
+  const Run1Cta c = cta[blockIdx.x];
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.y * 8 + (threadIdx.x >> 5); t < c.nrows; t += 8 * gridDim.y) {
+    const int row = perm[c.row0 + t], d = deg[c.row0 + t];
+    const int len = (deg[c.row0 + t - t % 32] + 7) / 8 * 8;  // of the slice's longest row, its first
+    const size_t e0 = (size_t)c.ent0 + slice[c.slice0 + t / 32] + 4 * (t % 32);
+    for (int k = lane; k < len; k += 32) {
+      float w = 0.f;
+      int u = 0;
+      if (k < d) {
+        const int p = rowptr[row] + k;
+        w = (float)J[p];
+        if (ei) {  // binary search: every column of the row is there
+          const int j = col[p];
+          int hi = c.nu - 1;
+          while (u < hi) {
+            const int m = (u + hi) / 2;
+            if (ucol[c.u0 + m] < j)
+              u = m + 1;
+            else
+              hi = m;
+          }
+        }
+      }
+      const size_t e = e0 + (size_t)(k / 4) * 128 + k % 4;
+      ej[e] = w;
+      if (ei) ei[e] = (uint16_t)u;
+    }
   }
 }
 
@@ -234,14 +262,17 @@ int run1_blocks_per_sm(size_t smem) {
   return n;
 }
 
-cudaError_t launch_fill_run1(const void* J, int jbf16, const int32_t* pos, int64_t count, float* ej,
+cudaError_t launch_fill_run1(const Run1Cta* cta, int nct, const int32_t* perm, const int32_t* deg,
+                             const int32_t* slice, const int32_t* ucol, const int32_t* rowptr,
+                             const int32_t* col, const void* J, int jbf16, float* ej, uint16_t* ei,
                              cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  const int grid = (int)std::min<int64_t>((count + 255) / 256, 4096);
+  const dim3 grid(nct, 16);
   if (jbf16)
-    k_fill_run1<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(J), pos, count, ej);
+    k_fill_run1<<<grid, 256, 0, s>>>(cta, perm, deg, slice, ucol, rowptr, col,
+                                     static_cast<const __nv_bfloat16*>(J), ej, ei);
   else
-    k_fill_run1<<<grid, 256, 0, s>>>(static_cast<const float*>(J), pos, count, ej);
+    k_fill_run1<<<grid, 256, 0, s>>>(cta, perm, deg, slice, ucol, rowptr, col, static_cast<const float*>(J),
+                                     ej, ei);
   return cudaGetLastError();
 }
 
