@@ -509,9 +509,10 @@ sb_status sb_energy_noalloc(int32_t n, const int32_t* rowptr, const int32_t* col
  * does (same states). 0: one thread per row. -1 (default): the widest group
  * for which rows x lanes fit in the SMs' resident threads, else 0; and runs of 16
  * steps or more whose couplings fit in the SMs' shared memory take one launch
- * for all steps (same states; its waits are bounded by SB_OPT_WAIT_NS, after
- * which the next synchronising call returns SB_ERR_TIMEOUT, as for
- * SB_OPT_STREAM). */
+ * for all steps, from the run on with which the context's one-replica steps have
+ * paid for the tables that this needs, a few hundred at most (same states; its
+ * waits are bounded by SB_OPT_WAIT_NS, after which the next synchronising call
+ * returns SB_ERR_TIMEOUT, as for SB_OPT_STREAM). */
 #define SB_OPT_R1_LANES 11
 /* SB_OPT_WAIT_NS (12): limit, in nanoseconds of the GPU's global timer, of
  * every wait of the streamed step kernel (SB_OPT_STREAM) on its shared-memory

@@ -30,7 +30,7 @@ using sbh::set_error;
 namespace {
 
 const int kEnergyRowsMin = 64;
-// shortest one-replica run that is worth k_run_r1 and, the first time, its tables
+// shortest one-replica run that is worth k_run_r1 once it has its tables
 const int kRun1Steps = 16;
 
 // A run of steps is captured into a CUDA graph the second time the same run
@@ -267,6 +267,7 @@ struct sb_ctx {
   // one-replica run in one launch (k_run_r1): tables for this context's rows
   struct Run1 {
     int built = 0;           // 0: not tried, 1: tables ready, -1: does not fit
+    int64_t steps = 0;       // one-replica steps run without them
     int32_t nct = 0, nx = 0, max_ent = 0;
     size_t smem = 0;
     char* d_mem = nullptr;   // one allocation for all of the following
@@ -2120,6 +2121,21 @@ sb_status ensure_run1(sb_ctx* c) {
   return st;
 }
 
+// Steps after which k_run_r1's tables have paid for themselves, by what they cost
+// and what they save a step, us: a context builds them for the run that brings its
+// one-replica steps to this number, so a short run or a few of them cost no more than
+// with the step kernels alone, and a long one gains from its first step on. Cost by
+// rows and nonzeros (up to 600,000, on one thread; about 1,100 beyond), saving by
+// nonzeros (the heaviest row sets the step kernels' time), and a third on top for the
+// spread. Measured, steps to break even / by this: 564 rows, 4 k nonzeros 7 / 26; 1,879,
+// 28 k 26 / 46; 4,208, 104 k 66 / 91; 10,152, 37 k 31 / 78; 10,999, 221 k 80 / 149; 39,484,
+// 293 k 180 / 231; 67,374, 772 k 205 / 207; 39,445, 1.8 M 45 / 121; 108,750, 1.8 M 145 / 122.
+int64_t run1_break_even(const sb_ctx* c) {
+  const double nnz = (double)c->nnz;
+  const double cost = nnz < 600000 ? 15.0 + 1.5e-3 * nnz + 8e-3 * c->n : 1100.0;
+  return (int64_t)(1.33 * cost / (3.0 + 6e-6 * nnz)) + 16;
+}
+
 sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, int32_t steps,
                                   const float* sched, cudaStream_t stream) {
   if (steps <= 0) return SB_OK;
@@ -2131,7 +2147,8 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
     // which need none, are recorded
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (!c->run1.built) SB_CUDA(cudaStreamIsCapturing(stream, &cap));
-    if (cap == cudaStreamCaptureStatusNone) {
+    if (cap == cudaStreamCaptureStatusNone && !c->run1.built &&
+        (c->run1.steps += steps) >= run1_break_even(c)) {
       try {
         if (sb_status st0 = ensure_run1(c)) return st0;
       } catch (const std::bad_alloc&) {
