@@ -2121,6 +2121,17 @@ sb_status ensure_run1(sb_ctx* c) {
   return st;
 }
 
+// ensure_run1, or the step kernels where the host has no memory for it
+sb_status try_run1(sb_ctx* c) {
+  try {
+    return ensure_run1(c);
+  } catch (const std::bad_alloc&) {
+    free_run1(c);
+    c->run1.built = -1;
+    return SB_OK;
+  }
+}
+
 // Steps after which k_run_r1's tables have paid for themselves, by what they cost
 // and what they save a step, us: a context builds them for the run that brings its
 // one-replica steps to this number, so a short run or a few of them cost no more than
@@ -2148,14 +2159,8 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (!c->run1.built) SB_CUDA(cudaStreamIsCapturing(stream, &cap));
     if (cap == cudaStreamCaptureStatusNone && !c->run1.built &&
-        (c->run1.steps += steps) >= run1_break_even(c)) {
-      try {
-        if (sb_status st0 = ensure_run1(c)) return st0;
-      } catch (const std::bad_alloc&) {
-        free_run1(c);
-        c->run1.built = -1;
-      }
-    }
+        (c->run1.steps += steps) >= run1_break_even(c))
+      if (sb_status st0 = try_run1(c)) return st0;
     const sb_ctx::Run1& r = c->run1;
     if (r.built > 0) {
       sbd::Run1Args ua{};
@@ -3562,17 +3567,22 @@ sb_status sb_autotune(sb_ctx* ctx, sb_variant variant, int32_t replicas, int32_t
       cands.insert(cands.begin(), Cand{0, 0, 0, 4, 1, 0, 0, 1});
       cands.insert(cands.begin(), Cand{0, 0, 0, 4, 1, 0, -1, 1});
     }
+    if ((st = ensure_state(ctx, replicas))) return st;
+    // one replica: the one-launch run is timed with its tables in place, over no fewer
+    // steps than it serves
+    const int32_t timed = replicas == 1 ? std::max(trial_steps, kRun1Steps) : trial_steps;
+    const int32_t warm = replicas == 1 ? kRun1Steps : std::min(trial_steps, 4);
+    if (replicas == 1 && ctx->r1_lanes < 0 && !SB_CHECKED && (st = try_run1(ctx))) return st;
+    float* sched = nullptr;
+    if ((st = dalloc(&sched, (size_t)timed))) return st;
     const int keep_graph = ctx->use_graph;
     ctx->use_graph = 0;
-    if ((st = ensure_state(ctx, replicas))) return st;
-    float* sched = nullptr;
-    if ((st = dalloc(&sched, (size_t)trial_steps))) return st;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     float best_us = 3.0e38f;
     int best = 0;
     cudaError_t err = cudaEventCreate(&e0);
     if (err == cudaSuccess) err = cudaEventCreate(&e1);
-    if (err == cudaSuccess) err = sbd::launch_linear_schedule(sched, trial_steps, 1.0, s);
+    if (err == cudaSuccess) err = sbd::launch_linear_schedule(sched, timed, 1.0, s);
     for (size_t k = 0; k < cands.size() && err == cudaSuccess; ++k) {
       const Cand& c = cands[k];
       if (c.tiled) {
@@ -3597,15 +3607,15 @@ sb_status sb_autotune(sb_ctx* ctx, sb_variant variant, int32_t replicas, int32_t
       ctx->l2_persist = c.l2;
       ctx->graph.reset();
       if ((st = sb_run(ctx, variant, 1.0, 0.0, 0.5, 0, replicas, 12345, nullptr, stream))) break;
-      if ((st = enqueue_steps(ctx, variant, 1.0, 0.5, std::min(trial_steps, 4), sched, s))) break;
+      if ((st = enqueue_steps(ctx, variant, 1.0, 0.5, warm, sched, s))) break;
       err = cudaEventRecord(e0, s);
       if (err != cudaSuccess) break;
-      if ((st = enqueue_steps(ctx, variant, 1.0, 0.5, trial_steps, sched, s))) break;
+      if ((st = enqueue_steps(ctx, variant, 1.0, 0.5, timed, sched, s))) break;
       err = cudaEventRecord(e1, s);
       if (err == cudaSuccess) err = cudaEventSynchronize(e1);
       float ms = 0.f;
       if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-      const float us = ms * 1000.f / trial_steps;
+      const float us = ms * 1000.f / timed;
       if (err == cudaSuccess && us < best_us) {
         best_us = us;
         best = (int)k;
