@@ -196,27 +196,6 @@ def make_ctx(sb, qs, prec, factor=True):
     return ctx
 
 
-def step_kernels(cfg, variant, R, info):
-    """Names of the kernels one SB step launches with autotuned configuration cfg."""
-    if cfg.get("factor"):
-        if variant != "dsb" and R % 128 == 0 and cfg.get("rows_per_warp", 0) != 0 \
-                and cfg.get("tile", 0) == 0:
-            return ["k_fac_sum", "k_step_rw"]
-        return ["k_fac_sum", "k_step_fac"]
-    if cfg["rows_per_warp"] and R % 128 == 0:
-        return ["k_step_rw"]
-    if cfg["tiled"] and R % 32 == 0:
-        return ["k_step_tiled"]
-    if variant == "dsb" and cfg["tile"] == 0 and cfg["groups"] == 1 and R % 16 == 0 \
-            and R // 16 <= 32 and (R // 16) & (R // 16 - 1) == 0:
-        return ["k_step_dsb16"]
-    if R == 1:  # all steps of a run in one launch unless a step option is set
-        one = cfg["tile"] == 0 and cfg["groups"] == 1 and not cfg["rows_per_cta"] \
-            and not cfg["l2_persist"]
-        return ["k_run_r1"] if one else ["k_step_r1"]
-    return ["k_step"]
-
-
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one SB step (all
 # its launches) from an ncu capture of the step's kernels, keyed by workload,
 # variant, kernels and those kernels' sources (sha256 prefix, kernel_source_hash);
@@ -248,10 +227,24 @@ MEASURED_TRAFFIC = {
         "source": _CAPTURE.format(step="k_step_rw", args=" --workload event1000")},
 }
 
-KERNEL_SOURCES = {"k_step_rw": ("rw.cu", "kernels.cuh", "signs.cuh"),
+_FACTOR = ("factor.cu", "kernels.cuh", "signs.cuh", "pdl.cuh")
+KERNEL_SOURCES = {"k_step_rw": ("rw.cu", "kernels.cuh", "signs.cuh", "pdl.cuh"),
                   "k_step_stream": ("stream.cu", "kernels.cuh", "signs.cuh"),
-                  "k_fac_sum": ("factor.cu", "kernels.cuh", "signs.cuh"),
-                  "k_step_fac": ("factor.cu", "kernels.cuh", "signs.cuh")}
+                  "k_run_r1": ("run1.cu", "kernels.cuh", "signs.cuh"),
+                  "k_fac_sum": _FACTOR, "k_step_fac": _FACTOR,
+                  "k_fac_sum_sgn": _FACTOR, "k_step_fac_sgn": _FACTOR}
+
+
+def launches_per_run(knames, variant, R, S, qs):
+    """Kernels of a timed run: c0, start and c0 again, the steps (dSB with sign bytes
+    first writes those of the start), and the readout: selection bits and their sums
+    where every coupling is a whole number of 2^-8, else the FP64 sums, then block
+    sums, arg-min and selection."""
+    signs = variant == "dsb" and (R + 3) // 4 * 4 == R and knames[0] not in (
+        "k_run_r1", "k_step_stream", "k_step_tiled")
+    whole = all(bool(np.all(q.val * 256 == np.rint(q.val * 256))) for q in qs)
+    steps = 1 if knames == ["k_run_r1"] else S * len(knames)
+    return 3 + (1 if signs else 0) + steps + (5 if whole else 4)
 
 
 def kernel_source_hash(knames):
@@ -260,7 +253,7 @@ def kernel_source_hash(knames):
     h = hashlib.sha256()
     files = []
     for k in knames:
-        for f in KERNEL_SOURCES.get(k, ("kernels.cu", "kernels.cuh", "signs.cuh")):
+        for f in KERNEL_SOURCES.get(k, ("kernels.cu", "kernels.cuh", "signs.cuh", "pdl.cuh")):
             if f not in files:
                 files.append(f)
     for f in files:
@@ -829,7 +822,6 @@ def run_ours(args):
         print(json.dumps({"profile_steps": args.profile_steps, "N": N, "nnz": nnz, "R": R}))
         return 0
     cfg, tune_us = sb.sb_autotune(ctx, variant, R, trial_steps=20 if E > 1 else 30)   # untimed set-up
-    knames = step_kernels(cfg, variant, R, finfo)
     sched = torch.tensor(np.array([a0 * k / (S - 1) for k in range(S)], np.float32), device=dev)
     d_E = torch.empty(E * R, dtype=torch.float64, device=dev)
     d_bE = torch.empty(E, dtype=torch.float64, device=dev)
@@ -870,6 +862,7 @@ def run_ours(args):
         dist.barrier()
     t_wall = time.perf_counter() - t_wall
     clk = clocks.stop()
+    knames = sb.sb_step_kernels(ctx).split(" + ")   # of the steps just timed
     step_ms = [m[0].elapsed_time(m[3]) for m in marks]
     sweep_ms = [m[1].elapsed_time(m[2]) for m in marks]
     ms = reduce_step_ms(float(np.sum(step_ms)) / args.steps, ws, dist if ws > 1 else None, dev)
@@ -977,8 +970,7 @@ def run_ours(args):
                        "autotune": cfg, "autotune_us_per_step": tune_us,
                        "host_build_s": t_build},
             "roofline": roofline, "e2e": e2e,
-            "gpu_launches": (3 + (1 if variant == "dsb" else 0) + (1 if knames == ["k_run_r1"] else S * len(knames)) + 4)
-            * args.steps,
+            "gpu_launches": launches_per_run(knames, variant, R, S, qs) * args.steps,
             "clocks": clk, "wall_s_timed": t_wall}
     if ws > 1:
         # the job's best of every event over all ranks' replicas
