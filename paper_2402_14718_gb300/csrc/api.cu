@@ -2191,10 +2191,16 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
       ua.err = c->d_err;
       ua.wait_ns = c->wait_ns;
       ua.skip_step = c->skip_stage;
-      SB_CUDA(sbd::launch_run_r1(variant, ua, r.smem, stream));
-      c->step_kernels = "k_run_r1";
-      if (steps & 1) c->cur ^= 1;
-      return SB_OK;
+      const cudaError_t e = sbd::launch_run_r1(variant, ua, r.smem, stream);
+      // a stream of a part of the device (a green context) may hold too few SMs for
+      // the grid to be resident at once: the step kernels serve the run there
+      if (e != cudaErrorCooperativeLaunchTooLarge) {
+        SB_CUDA(e);
+        c->step_kernels = "k_run_r1";
+        if (steps & 1) c->cur ^= 1;
+        return SB_OK;
+      }
+      cudaGetLastError();
     }
   }
   // A run of padded rows that the caller records reads the CSR in place: the tables
