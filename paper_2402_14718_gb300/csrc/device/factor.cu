@@ -162,7 +162,7 @@ struct FacMinBlocks {
   static constexpr int sum = NCH == 2 ? 7 : B, step = NCH == 2 ? 8 : B;
 };
 // Nine CTAs leave 56 registers and spill up to 52 bytes since x and U come by plain
-// loads (pdl.cuh); eight fit. Nine stay the better choice where there are lanes
+// loads (pdl.cuh); eight spill nothing, or at most 16. Nine stay the better choice where there are lanes
 // enough to use the warps. bSB, us per step with nine / eight, and with __ldg and
 // nine, launch by launch, that came before:
 //   R = 16: 39,445 rows (158 k lanes) 21.2 / 17.4, 18.3; 98,134 rows (393 k) 28.6 /
@@ -172,7 +172,7 @@ struct FacMinBlocks {
 //   108,750 rows (1.7 M) 58.2 / 61.0, 59.4.
 //   R = 8 (two lanes a row): 39,445 rows (79 k) 26.4 / 25.5, 26.4; 67,374 rows (135 k)
 //   19.2 / 20.8, 19.6; 98,134 rows (196 k) 31.9 / 31.1, 31.0; 242,044 rows 40.8 / 41.4, 40.9.
-//   R = 4: 39,165 rows 33.0 / 32.2, 32.7; 472,812 rows 77.4 / 73.0, 71.8.
+//   R = 4: 39,445 rows 33.0 / 32.2, 32.7; 472,676 rows 77.4 / 73.0, 71.8.
 inline int fac_blocks(int64_t n, int R, int G) {
   const int64_t lanes = n * R / 4;
   return G >= 2 && lanes >= (G == 2 ? 100000 : 800000) ? 9 : 8;

@@ -309,9 +309,9 @@ cudaError_t launch_step_u(int jbf16, const Tiling& t, const StepArgs& a, cudaStr
 //  two chunks per lane, 2 / 4 in flight: 10,878 rows R = 100 12.9 / 11.4, R = 192
 //  16.2 / 17.1; 109,775 rows R = 100 88 / 105. So 2 from 1.5 M spins on (4 with
 //  sign bytes, which hold a quarter of the registers: 89 / 84);
-//  sign bytes, two chunks, two / three CTAs per SM: 67,445 rows R = 192 110 / 82 (107
-//  with the shuffled walk that came before), R = 20 14.9 / 13.2; 39,165 rows R = 160
-//  111 / 91, R = 12 27.9 / 31.4; 10,878 rows R = 160 18.2 / 16.2, R = 96 FP32 11.7 / 12.2,
+//  sign bytes, two chunks, two / three CTAs per SM: 67,374 rows R = 192 110 / 82 (107
+//  with the shuffled walk that came before), R = 20 14.9 / 13.2; 39,445 rows R = 160
+//  111 / 91, R = 12 27.9 / 31.4; 10,999 rows R = 160 18.2 / 16.2, R = 96 FP32 11.7 / 12.2,
 //  R = 33 8.2 / 9.5. So three from 1.5 M spins on as well.
 template <int V, int NCH, int MODE>
 cudaError_t launch_step_t(int jbf16, const Tiling& t, const StepArgs& a, cudaStream_t s) {
@@ -490,8 +490,8 @@ __global__ void __launch_bounds__(kBlock) k_step_r1g(const StepArgs a) {
 // same walk: each lane reads the (col, J) pairs itself, four neighbours in
 // flight without a predicate, the next four pairs on their way. Pairs loaded G
 // at a time and broadcast by shuffles left G = 1 .. 4 with as many neighbours in
-// flight: us per step before / now, 39,165 rows R = 16 81 / 21, R = 64 37 / 24.5,
-// R = 128 40.5 / 36; 67,445 rows R = 64 24.8 / 20.8; 109,775 rows R = 256 equal.
+// flight: us per step before / now, 39,445 rows R = 64 47.3 / 31.5, R = 128 45.7 / 37.4;
+// 67,374 rows R = 64 24.5 / 18.8, R = 256 68.6 / 67.5; 472,676 rows R = 16 266 / 112.
 
 #ifndef SB_DSB_BLOCK
 #define SB_DSB_BLOCK 128
@@ -499,10 +499,10 @@ __global__ void __launch_bounds__(kBlock) k_step_r1g(const StepArgs a) {
 // seven CTAs of 128 threads per SM: with the sign bytes, x and y in plain loads
 // (pdl.cuh) eight leave the compiler too few registers to keep the loads together.
 // us per step with eight / seven, and with the shuffled walk and nine CTAs that came
-// before: 10,878 rows R = 256 17.9 / 14.9, 17.4; 39,165 rows R = 64 47.7 / 31.5, 47.3,
-// R = 512 124.5 / 119, 121; 91,504 rows R = 256 200 / 188, 199; 472,812 rows R = 128
-// 458 / 424, 486. Six: R = 512 122, 91,504 rows 194; asking for all own values before
-// the first store, with seven: R = 512 123.5, 91,504 rows 198.
+// before: 10,999 rows R = 256 17.9 / 14.9, 17.4; 39,445 rows R = 64 47.7 / 31.5, 47.3,
+// R = 512 124.5 / 119, 121; 98,134 rows R = 256 200 / 188, 199; 472,676 rows R = 128
+// 458 / 424, 486. Six: R = 512 122, 98,134 rows 194; asking for all own values before
+// the first store, with seven: R = 512 123.5, 98,134 rows 198.
 #ifndef SB_DSB_MINB
 #define SB_DSB_MINB 7
 #endif
@@ -1638,7 +1638,7 @@ cudaError_t launch_signs(const float* x, uint8_t* s, size_t count, cudaStream_t 
 // A warp walks rows (32 / opitch at a time where they are short), 32 values of
 // each, four rows and both arrays in flight, no division in the loop. Bound by
 // launch and latency below a few MB, by L2 above. sb_set_state of a device state of
-// 67,445 rows, us: R = 50 28, R = 99 43, its wait of about 6 included (one launch
+// 67,374 rows, us: R = 50 28, R = 99 43, its wait of about 6 included (one launch
 // per array with a 64-bit division per value, without the wait, 32 / 62; the two
 // copies of an unpadded state, without it, 27 / 38).
 __global__ void __launch_bounds__(kBlock) k_repitch(const float* x, const float* y, int32_t ipitch,

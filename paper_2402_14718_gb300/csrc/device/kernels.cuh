@@ -25,9 +25,10 @@ Tiling make_tiling_rt(int R, int RT);
 bool dsb16_ok(int R);
 // Above this many spins dSB takes that kernel, below it k_step with sign bytes
 // (4 replicas per lane: four times the lanes, a quarter of the bytes per load).
-// us per step, 16 per lane / 4 per lane: 39,165 rows R = 32 (1.25 M spins) 23.5 /
-// 18.8, R = 64 (2.5 M) 24.5 / 29.1; 67,445 rows R = 32 (2.2 M) 14.0 / 13.9, R = 64
-// (4.3 M) 20.8 / 22.5; 10,878 rows R = 64 (0.7 M) 13.0 / 7.9, R = 512 (5.6 M) 25 / 30.
+// us per step, 16 per lane / 4 per lane: 39,445 rows R = 32 (1.26 M spins) 30.9 /
+// 24.4, R = 64 (2.52 M) 31.5 / 34.4; 67,374 rows R = 32 (2.16 M) 17.2 / 13.4, R = 64
+// (4.31 M) 18.8 / 22.3; 10,999 rows R = 128 (1.41 M) 14.5 / 10.9, R = 256 (2.82 M) 14.9 /
+// 18.3; 98,134 rows R = 16 (1.57 M) 62.6 / 41.3, R = 32 (3.14 M) 49.3 / 56.3.
 constexpr int64_t kDsb16Spins = 2400000;
 // rows per CTA of k_step_dsb16 for a step's rows-per-CTA setting rpc
 int dsb16_rows_per_cta(int rpc);

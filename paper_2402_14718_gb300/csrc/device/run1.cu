@@ -21,11 +21,12 @@
 // lane together (a warp's reads of weights and indices have no bank conflicts),
 // in CSR order: the sum is the one FMA chain of the other one-replica kernels, bit
 // for bit, with eight positions in flight and the next indices on their way.
-// Measured, us per step before / now: 1,721 rows 2.9 / 1.7; 10,214 rows (35,860
-// nonzeros) 3.0 / 1.5; 10,878 rows 5.5 / 2.2; 39,165 rows 14 to 20.6 / 3.0; 67,445
-// rows 6.5 / 2.4. A cluster of 16 CTAs that wrote its positions into each other's
-// shared memory took 1.45 us for 1,721 rows with the cluster's barrier, 2.9 us for
-// 10,214 rows, and 5 to 9 us when its threads polled shared memory instead.
+// Measured in runs of 256 to 512 steps, us per step, step kernels in a graph / now:
+// 1,879 rows 5.0 / 1.55; 10,152 rows (37,322 nonzeros) 5.3 / 1.5; 10,999 rows 7.5 / 1.9;
+// 39,445 rows 22.5 / 3.7; 67,374 rows 8.2 / 2.3. A cluster of 16 CTAs that wrote its
+// positions into each other's shared memory took 1.45 us for 1,721 rows with the
+// cluster's barrier, where this form then took 1.7, but 2.9 us for 10,214 rows, and 5
+// to 9 us when its threads polled shared memory instead.
 #include <cuda_bf16.h>
 
 #include <algorithm>
