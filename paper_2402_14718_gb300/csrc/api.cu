@@ -3105,11 +3105,11 @@ sb_status sb_set_state(sb_ctx* ctx, const float* x, const float* y, int32_t repl
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     SB_CUDA(cudaDeviceSynchronize());
     ctx->cur = 0;
-    if (ctx->Rs == replicas) {
+    if (on_device && own_memory(ctx, x, bytes, 4) && own_memory(ctx, y, bytes, 4)) {
+      SB_CUDA(sbd::launch_repitch(x, y, replicas, ctx->d_x[0], ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
+    } else if (ctx->Rs == replicas) {
       SB_CUDA(cudaMemcpy(ctx->d_x[0], x, bytes, k));
       SB_CUDA(cudaMemcpy(ctx->d_y, y, bytes, k));
-    } else if (on_device && own_memory(ctx, x, bytes, 4) && own_memory(ctx, y, bytes, 4)) {
-      SB_CUDA(sbd::launch_repitch(x, y, replicas, ctx->d_x[0], ctx->d_y, ctx->Rs, ctx->n, replicas, 0));
     } else {  // both through the x buffers, then into the padded rows
       SB_CUDA(cudaMemcpy(ctx->d_x[0], y, bytes, k));
       SB_CUDA(cudaMemcpy(ctx->d_x[1], x, bytes, k));
@@ -3141,7 +3141,7 @@ sb_status sb_get_state(const sb_ctx* ctx, float* x, float* y, int32_t on_device)
   const float *const sx = ctx->d_x[ctx->cur], *const sy = ctx->d_y;
   const bool padded = ctx->Rs != ctx->R;
   std::unique_lock<std::mutex> one_at_a_time(ctx->get_mutex, std::defer_lock);
-  if (padded && on_device && (!x || own_memory(ctx, x, bytes, 4)) &&
+  if (on_device && (!x || own_memory(ctx, x, bytes, 4)) &&
       (!y || own_memory(ctx, y, bytes, 4))) {
     SB_CUDA(sbd::launch_repitch(x ? sx : sy, x && y ? sy : nullptr, ctx->Rs, x ? x : y, y, ctx->R,
                                 ctx->n, ctx->R, 0));

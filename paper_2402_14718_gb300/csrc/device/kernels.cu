@@ -1669,9 +1669,42 @@ __global__ void __launch_bounds__(kBlock) k_repitch(const float* x, const float*
     }
 }
 
+// The same of rows that lie alike: x and y in one launch, by 16 bytes. sb_set_state /
+// sb_get_state of a device state, us, two copies without the wait / so, with it: 1,879
+// rows R = 64 17 / 19, 25 / 21; 10,999 rows R = 64 22 / 20, 30 / 23; 67,374 rows R = 64
+// 28 / 25, 36 / 32.
+__global__ void __launch_bounds__(kBlock) k_copy2(const float4* x, const float4* y, float4* xo, float4* yo,
+                                                  int64_t count) {
+  const int64_t step = (int64_t)gridDim.x * kBlock;
+  for (int64_t i0 = (int64_t)blockIdx.x * kBlock + threadIdx.x; i0 < count; i0 += 4 * step) {
+    float4 v[4], w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * step < count) {
+        v[u] = __ldg(x + i0 + u * step);
+        w[u] = __ldg(y + i0 + u * step);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * step < count) {
+        xo[i0 + u * step] = v[u];
+        yo[i0 + u * step] = w[u];
+      }
+  }
+}
+
 cudaError_t launch_repitch(const float* x, const float* y, int32_t ipitch, float* xo, float* yo,
                            int32_t opitch, int32_t n, int32_t cols, cudaStream_t s) {
   if (n <= 0 || opitch <= 0) return cudaSuccess;
+  const auto aligned = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  const int64_t values = (int64_t)n * cols;
+  if (ipitch == cols && opitch == cols && y && values % 4 == 0 && aligned(x) && aligned(y) && aligned(xo) &&
+      aligned(yo)) {
+    const int grid = (int)std::min<int64_t>((values / 4 + kBlock - 1) / kBlock, 4096);
+    k_copy2<<<grid, kBlock, 0, s>>>(reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(y),
+                                    reinterpret_cast<float4*>(xo), reinterpret_cast<float4*>(yo), values / 4);
+    return cudaGetLastError();
+  }
   const int64_t rows = (int64_t)(kBlock / 32) * (opitch < 32 ? 32 / opitch : 1);  // of a block at a time
   const int grid = (int)std::min<int64_t>((n + rows - 1) / rows, 4096);
   k_repitch<<<grid, kBlock, 0, s>>>(x, y, ipitch, xo, yo, opitch, n, cols);
