@@ -200,31 +200,31 @@ def make_ctx(sb, qs, prec, factor=True):
 # its launches) from an ncu capture of the step's kernels, keyed by workload,
 # variant, kernels and those kernels' sources (sha256 prefix, kernel_source_hash);
 # any other combination reports null. Each capture is one ncu pass of the
-# third step of the profiling driver (`--profile-steps 4`, the workload's own
+# second step of the profiling driver (`--profile-steps 4`, the workload's own
 # size), early in the schedule where no spin is pinned yet, so the writes are
 # at their largest.
 _CAPTURE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none "
-            "-k regex:\"k_fac_sum|{step}\" -s 2 -c 2 python bench.py{args} --profile-steps 4")
+            "-k regex:\"k_fac_sum|k_step_fac|k_step_rw\" -s 2 -c 2 python bench.py{args} "
+            "--profile-steps 4")
 MEASURED_TRAFFIC = {
     # the full batch holds ~8 GB on the device: counters are taken on every 4th
-    # event (128 events, sum N = 1,120,853; 1,531,240,704 B per step) and scaled
+    # event (128 events, sum N = 1,120,853; 1,511,852,544 B per step) and scaled
     # by the spin-updates (x 5,677,517 / 1,120,853). Per spin-update the traffic
-    # rises with the working set (20.7 / 21.3 B at 64 / 128 events; 22.4 B in an
-    # earlier capture of the whole batch with the same kernel code), so this is
-    # a lower bound by about 5 %.
-    ("batch512", "dsb", ("k_fac_sum", "k_step_fac"), "9ffffff132286b78"): {
-        "bytes_per_step": 7756275915,
-        "source": _CAPTURE.format(step="k_step_fac", args=" --events 128") +
+    # rises with the working set (20.7 / 21.3 / 22.4 B at 64 / 128 / 512 events with
+    # an earlier form of the kernels), so this is a lower bound by about 5 %.
+    ("batch512", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
+        "bytes_per_step": 7658068025,
+        "source": _CAPTURE.format(args=" --events 128") +
         " (every 4th event; scaled to the 512 events by the spin-updates)"},
-    ("event10k", "dsb", ("k_fac_sum", "k_step_fac"), "9ffffff132286b78"): {
-        "bytes_per_step": 78817024 + 22779136 + 717631232 + 497986304,
-        "source": _CAPTURE.format(step="k_step_fac", args=" --workload event10k --variant dsb")},
-    ("event10k_1m", "dsb", ("k_fac_sum", "k_step_fac"), "9ffffff132286b78"): {
-        "bytes_per_step": 255639040 + 96422912 + 1643463936 + 1169588992,
-        "source": _CAPTURE.format(step="k_step_fac", args=" --workload event10k_1m --variant dsb")},
-    ("event1000", "bsb", ("k_fac_sum", "k_step_rw"), "b5333c45d2b32b72"): {
-        "bytes_per_step": 40304896 + 1613056 + 101010688 + 33296128,
-        "source": _CAPTURE.format(step="k_step_rw", args=" --workload event1000")},
+    ("event10k", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
+        "bytes_per_step": 74019328 + 19165696 + 708126720 + 485044480,
+        "source": _CAPTURE.format(args=" --workload event10k --variant dsb")},
+    ("event10k_1m", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
+        "bytes_per_step": 238134272 + 81408512 + 1648426752 + 1191499776,
+        "source": _CAPTURE.format(args=" --workload event10k_1m --variant dsb")},
+    ("event1000", "bsb", ("k_fac_sum", "k_step_rw"), "babe6105eba29716"): {
+        "bytes_per_step": 40308992 + 1826304 + 101010944 + 35682048,
+        "source": _CAPTURE.format(args=" --workload event1000")},
 }
 
 _FACTOR = ("factor.cu", "kernels.cuh", "signs.cuh", "pdl.cuh")

@@ -309,7 +309,10 @@ sb_status sb_gather_probe(int64_t array_bytes, int32_t row_bytes, int32_t repeat
  * value, per event). a_sched: device FP32 array of `steps`
  * values a_k, or NULL for the linear ramp a_k = a0 k / (steps - 1).
  * Allocates the N x R state on first use (kept for later calls with the same
- * R). 1 <= replicas <= 65535, 0 <= steps. Asynchronous on `stream`.
+ * R). Replica counts that are no multiple of 4 are stored in padded rows (50 as
+ * 64, 7 as 8; unpadded where device memory is short); where an option or a
+ * factored form below asks for a multiple, the count as stored decides.
+ * 1 <= replicas <= 65535, 0 <= steps. Asynchronous on `stream`.
  */
 sb_status sb_run(sb_ctx* ctx, sb_variant variant, double a0, double c0, double dt,
                  int32_t steps, int32_t replicas, uint64_t seed, const float* a_sched,
@@ -565,7 +568,8 @@ sb_status sb_autotune(sb_ctx* ctx, sb_variant variant, int32_t replicas, int32_t
  * nothing traps; a row-pointer pair outside [0, nnz] reads as an empty row.
  * Results are then wrong but the device stays usable. Not covered: the
  * tiled and streamed step options, the adjoint kernels and the device QUBO
- * builder. The release build compiles the tests away.
+ * builder. One replica takes the step kernels there, which are covered, instead
+ * of the one launch for all steps. The release build compiles the tests away.
  *
  * sb_checked_build: 1 in the bounds-checked build, 0 in the release build.
  *

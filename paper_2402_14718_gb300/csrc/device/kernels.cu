@@ -1272,10 +1272,12 @@ __global__ void __launch_bounds__(kBlock) k_energy_partial(const EnergyArgs a) {
 // sum_j b_ij T_j is a whole number too: it is summed exactly in integers, in any
 // order, from the selections as bits, and only the linear terms (n x R) and the
 // block sums stay in FP64. Bits also cut the gather: a neighbour's 256 replicas
-// are one 32-byte sector instead of 1 KB of positions. Bound by integer issue
-// (about two instructions per nonzero and replica). Whole readout of the
-// 39,165-row event at R = 256: 1791 us with k_energy_partial and serial block
-// sums, 273 us here; the error against 64-bit sums falls from 7e-16 to 2e-16.
+// are one 32-byte sector instead of 1 KB of positions. Bound by instruction issue
+// (about two instructions per nonzero and replica: issue slots 63 % busy and the
+// integer pipe 59 %, with a third of the warps active and hardly a stall on
+// memory). Whole readout of 39,445 rows at R = 256: 1790 us with k_energy_partial and
+// serial block sums, 246 us here, 178 of them k_energy_bits; the error against
+// 64-bit sums falls from 7e-16 to 2e-16.
 
 // Bits of one row's selections: a warp takes 32 replicas of a row at a time
 // (one coalesced 128-byte load, one ballot) when R >= 16, a thread a whole row
@@ -1316,8 +1318,8 @@ __device__ __forceinline__ int whole_b(float j) {
 
 // A team of L x S lanes owns a row: lane l of slice s holds the replicas 8 l ..
 // 8 l + 7 (one byte of bits per neighbour) of every S-th nonzero, eight in flight
-// (39,165 rows R = 256, whole readout: 180 us with eight and three CTAs per SM, 198
-// with four and four CTAs). Few replicas leave few bytes per row, so the slices then share a
+// (39,165 rows R = 256, by itself: 180 us with eight and three CTAs per SM, at 80
+// registers with 76 bytes spilled, 198 with four and four CTAs). Few replicas leave few bytes per row, so the slices then share a
 // row's nonzeros (whole-number sums: any split gives the same value).
 template <typename JT>
 __global__ void __launch_bounds__(kBlock, 3) k_energy_bits(const EnergyBitArgs a, int L, int S) {
