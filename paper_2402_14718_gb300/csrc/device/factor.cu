@@ -633,6 +633,11 @@ __global__ void __launch_bounds__(kFacBlock, (FacMinBlocks<NCH, B>::step)) k_ste
 // Bound by latency and issue. Ten CTAs per SM (48 registers); with eight (64,
 // U rows first) the 64-event batch takes 216 us a step late in the run, with
 // twelve (spills) 218, with ten 197; requesting the own x and y first took 216.
+// FP32 U rows (UF32) hold 24 registers in flight and lie in HBM: they are asked for
+// in L2 with the head's neighbours and read one after the other at the end.
+// 1,031,640 rows, us per step, in flight as the BF16 ones (52 bytes spilled) / so, and
+// with the shuffled walk that came before: R = 128 851 / 737, 786; R = 64 501 / 438,
+// 454; R = 16 233 / 216, 293. Eight CTAs, in flight 830, one by one 812; nine 794.
 template <bool UF32, int K, typename JT>
 __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArgs a) {
   constexpr int P = kSgnPer;
@@ -671,6 +676,12 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
     for (int u = 0; u < 4; ++u) s1[u] = gather(cb[u]);
   }
   const uint32_t uw[4] = {hu.x, hu.y, hu.z, hu.w};
+  if (UF32) {
+#pragma unroll
+    for (int s = 0; s < K; ++s)
+      if ((int)uw[s] >= 0)
+        prefetch_l2(static_cast<const float*>(a.U) + (size_t)chk_idx((int)uw[s], a.urows, kChkURow) * R + off);
+  }
   const float c0 = a.c0_ev[ev];
   const float pa = a.a0 - __ldg(a.sched + a.k);
 
@@ -701,7 +712,7 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
   URow<1, NCH> ur[K];
 #pragma unroll
   for (int s = 0; s < K; ++s)
-    if ((int)uw[s] >= 0)
+    if (!UF32 && (int)uw[s] >= 0)
       ur[s].load(a.U, (size_t)chk_idx((int)uw[s], a.urows, kChkURow) * R + off, G);
   if (L > kFacHead) {
     const JT* J = static_cast<const JT*>(a.rJ);
@@ -735,6 +746,7 @@ __global__ void __launch_bounds__(kFacBlock, 10) k_step_fac_sgn(const FacStepArg
   for (int s = 0; s < K; ++s)
     if ((int)uw[s] >= 0) {
       any = true;
+      if (UF32) ur[s].load(a.U, (size_t)chk_idx((int)uw[s], a.urows, kChkURow) * R + off, G);
       ur[s].add_to(fu);
     }
   if (any) {

@@ -129,3 +129,20 @@ def test_buffers_that_end_with_their_memory(pieces):
     r = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("R", [1, 50, 64])
+@pytest.mark.parametrize("shift", [1, 2, 4])
+def test_buffers_off_the_16_byte_boundary(R, shift):
+    import torch
+    n = 5000
+    ctx = sb.sb_create(n, np.zeros(n + 1, np.int32), np.zeros(0, np.int32), np.zeros(0), np.zeros(n))
+    g = torch.Generator(device="cuda").manual_seed(R)
+    base = torch.rand(2 * n * R + 16, generator=g, device="cuda")
+    x, y = base[shift:shift + n * R].view(n, R), base[n * R + 8:2 * n * R + 8].view(n, R)
+    sb.sb_set_state(ctx, x, y)
+    out = torch.zeros(2 * n * R + 16, device="cuda")
+    a, b = out[shift:shift + n * R].view(n, R), out[n * R + 8:2 * n * R + 8].view(n, R)
+    sb._lib.check(sb.lib.sb_get_state(ctx.handle, a.data_ptr(), b.data_ptr(), 1))
+    assert torch.equal(a, x) and torch.equal(b, y)
+    assert out[:shift].sum() == 0 and out[2 * n * R + 8:].sum() == 0
