@@ -105,6 +105,17 @@ struct JPack<2, float> {
 };
 
 
+// Groups of two overlap the launch before them and load x plainly (pdl.cuh). Groups
+// of four hold twice the sums, and with plain loads the compiler found no order for
+// them (us per step, dependent / plain launches: 39,445 rows, R = 256, BF16 bSB 109 /
+// 91.6, dSB 126 / 109; 10,999 rows, R = 128, bSB 14.1 / 13.6; 1,879 rows 8.0 / 9.3): they are launched one after the
+// other, read x as read-only data, and take their rows one at a time.
+template <int RW, typename T>
+__device__ __forceinline__ T ld_x(const T* p) {
+  if constexpr (RW == 2) return *p;
+  return __ldg(p);
+}
+
 // MODE: 0 aSB, 1 bSB, 2 dSB gathering x (sgn at use), 3 dSB gathering the
 // sign bytes written by the previous step (4 bytes per lane chunk)
 // Residency (CTAs of 128 threads per SM): with two chunks per lane nine (BF16 J)
@@ -151,7 +162,7 @@ __global__ void __launch_bounds__(kRwBlock, (rw_blocks<RW, NCH>(sizeof(JT)))) k_
       pk = __ldg(a.ent + e0 + lane);
       jp.ld(a.ejv, e0 + lane);
     }
-    pdl_wait();  // from here on: what earlier launches write
+    if (RW == 2) pdl_wait();  // from here on: what earlier launches write
     const float pa = a.a0 - __ldg(a.sched + a.k);
     for (int eb = e0; eb < e1; eb += 32) {
       const int cnt = min(32, e1 - eb);
@@ -176,7 +187,7 @@ __global__ void __launch_bounds__(kRwBlock, (rw_blocks<RW, NCH>(sizeof(JT)))) k_
             const uint32_t* ps = reinterpret_cast<const uint32_t*>(xl + (size_t)cu * rb);
 #pragma unroll
             for (int j = 0; j < NCH; ++j) {
-              const uint32_t t = ps[32 * j];
+              const uint32_t t = ld_x<RW>(ps + 32 * j);
 #pragma unroll
               for (int k = 0; k < 4; ++k) xv[u][j][k] = scaled_sign_of_byte(t, k);
             }
@@ -184,7 +195,7 @@ __global__ void __launch_bounds__(kRwBlock, (rw_blocks<RW, NCH>(sizeof(JT)))) k_
             const float4* px = reinterpret_cast<const float4*>(xl + (size_t)cu * rb);
 #pragma unroll
             for (int j = 0; j < NCH; ++j) {
-              const float4 t = px[32 * j];
+              const float4 t = ld_x<RW>(px + 32 * j);
               xv[u][j][0] = t.x;
               xv[u][j][1] = t.y;
               xv[u][j][2] = t.z;
@@ -217,69 +228,79 @@ __global__ void __launch_bounds__(kRwBlock, (rw_blocks<RW, NCH>(sizeof(JT)))) k_
     }
 
     // symplectic Euler: momentum with the old position, then position, then wall.
-    // The own values of all rows are asked for before the first store: x is a plain
-    // load (pdl.cuh) that the compiler must keep behind a store that may alias it,
-    // and row by row the second row's latency came on top of the first's (per step,
+    // Groups of two ask for the own values of both rows before the first store: x is a
+    // plain load (pdl.cuh) that the compiler must keep behind a store that may alias
+    // it, and row by row the second row's latency came on top of the first's (per step,
     // row by row / now: 39,165 rows, R = 256, factored 55.6 / 54.2 us; 472,812 rows,
     // R = 128, factored 452 / 439).
-    int row[RW];
-    float c0[RW], hi[RW];
+    constexpr int QB = RW == 2 ? 2 : 1;  // rows at a time
 #pragma unroll
-    for (int q = 0; q < RW; ++q) {
-      row[q] = __ldg(a.grows + (size_t)grp * RW + q);
-      const int ev = a.row_event && row[q] >= 0 ? __ldg(a.row_event + row[q]) : 0;
-      c0[q] = a.c0_ev[ev];
-      hi[q] = row[q] >= 0 ? __ldg(a.h + row[q]) : 0.f;
-    }
+    for (int q0 = 0; q0 < RW; q0 += QB) {
+      int row[QB];
+      float c0[QB], hi[QB];
 #pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      float4 xo[RW], yo[RW];
-#pragma unroll
-      for (int q = 0; q < RW; ++q) {
-        // a group's missing row reads its first one (no predicate: it spills)
-        const size_t idx = (size_t)(row[q] >= 0 ? row[q] : max(row[0], 0)) * R + rep0 + 128 * j;
-        xo[q] = *reinterpret_cast<const float4*>(a.xin + idx);
-        yo[q] = *reinterpret_cast<const float4*>(a.y + idx);
+      for (int q = 0; q < QB; ++q) {
+        row[q] = __ldg(a.grows + (size_t)grp * RW + q0 + q);
+        const int ev = a.row_event && row[q] >= 0 ? __ldg(a.row_event + row[q]) : 0;
+        c0[q] = a.c0_ev[ev];
+        hi[q] = row[q] >= 0 ? __ldg(a.h + row[q]) : 0.f;
       }
+      if (QB == 1 && row[0] < 0) continue;
 #pragma unroll
-      for (int q = 0; q < RW; ++q) {
-        if (row[q] < 0) continue;
-        const size_t idx = (size_t)row[q] * R + rep0 + 128 * j;
-        float xs[4] = {xo[q].x, xo[q].y, xo[q].z, xo[q].w}, ys[4] = {yo[q].x, yo[q].y, yo[q].z, yo[q].w};
-        uint32_t sw = 0u;
+      for (int j = 0; j < NCH; ++j) {
+        float4 xo[QB], yo[QB];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          float x = xs[v], y = ys[v];
-          float force = -pa * x + c0[q] * (acc[q][j][v] + hi[q]);
-          if (VARIANT == 0) force -= x * x * x;
-          y = y + a.dt * force;
-          x = x + a.dta0 * y;
-          if (VARIANT != 0 && fabsf(x) > 1.f) {
-            x = copysignf(1.f, x);
-            y = 0.f;
-          }
-          xs[v] = x;
-          ys[v] = y;
-          if (use_sgn) sw |= sign_byte(x) << (8 * v);
+        for (int q = 0; q < QB; ++q) {
+          // a group's missing row reads its first one (no predicate: it spills)
+          const size_t idx = (size_t)(row[q] >= 0 ? row[q] : max(row[0], 0)) * R + rep0 + 128 * j;
+          xo[q] = ld_x<RW>(reinterpret_cast<const float4*>(a.xin + idx));
+          yo[q] = *reinterpret_cast<const float4*>(a.y + idx);
         }
-        if (use_sgn) *reinterpret_cast<uint32_t*>(a.sgn_out + idx) = sw;
-        *reinterpret_cast<float4*>(a.xout + idx) = make_float4(xs[0], xs[1], xs[2], xs[3]);
-        *reinterpret_cast<float4*>(a.y + idx) = make_float4(ys[0], ys[1], ys[2], ys[3]);
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+          if (row[q] < 0) continue;
+          const size_t idx = (size_t)row[q] * R + rep0 + 128 * j;
+          float xs[4] = {xo[q].x, xo[q].y, xo[q].z, xo[q].w}, ys[4] = {yo[q].x, yo[q].y, yo[q].z, yo[q].w};
+          uint32_t sw = 0u;
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            float x = xs[v], y = ys[v];
+            float force = -pa * x + c0[q] * (acc[q0 + q][j][v] + hi[q]);
+            if (VARIANT == 0) force -= x * x * x;
+            y = y + a.dt * force;
+            x = x + a.dta0 * y;
+            if (VARIANT != 0 && fabsf(x) > 1.f) {
+              x = copysignf(1.f, x);
+              y = 0.f;
+            }
+            xs[v] = x;
+            ys[v] = y;
+            if (use_sgn) sw |= sign_byte(x) << (8 * v);
+          }
+          if (use_sgn) *reinterpret_cast<uint32_t*>(a.sgn_out + idx) = sw;
+          *reinterpret_cast<float4*>(a.xout + idx) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+          *reinterpret_cast<float4*>(a.y + idx) = make_float4(ys[0], ys[1], ys[2], ys[3]);
+        }
       }
     }
   }
+}
+
+template <int RW, int NCH, int MODE, typename JT>
+cudaError_t launch_m(dim3 grid, const RwArgs& a, cudaStream_t s) {
+  if constexpr (RW == 2) return launch_pdl(k_step_rw<RW, NCH, MODE, JT>, grid, kRwBlock, a, s);
+  k_step_rw<RW, NCH, MODE, JT><<<grid, kRwBlock, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 template <int RW, int NCH, typename JT>
 cudaError_t launch_t(int variant, const RwArgs& a, cudaStream_t s) {
   dim3 grid((a.ngroups + a.gpc - 1) / a.gpc, a.R / (128 * NCH));
   switch (variant) {
-    case 0: return launch_pdl(k_step_rw<RW, NCH, 0, JT>, grid, kRwBlock, a, s);
-    case 1: return launch_pdl(k_step_rw<RW, NCH, 1, JT>, grid, kRwBlock, a, s);
+    case 0: return launch_m<RW, NCH, 0, JT>(grid, a, s);
+    case 1: return launch_m<RW, NCH, 1, JT>(grid, a, s);
     default:
-      if (a.sgn_in)
-        return launch_pdl(k_step_rw<RW, NCH, 3, JT>, grid, kRwBlock, a, s);
-      return launch_pdl(k_step_rw<RW, NCH, 2, JT>, grid, kRwBlock, a, s);
+      return a.sgn_in ? launch_m<RW, NCH, 3, JT>(grid, a, s) : launch_m<RW, NCH, 2, JT>(grid, a, s);
   }
 }
 
