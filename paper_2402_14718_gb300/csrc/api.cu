@@ -2431,7 +2431,9 @@ sb_status enqueue_steps_as_stored(sb_ctx* c, int variant, double a0, double dt, 
   // byte condition below must agree
   const bool dsb16 = !fac && !streamed && !rw && variant == SB_DSB && dsb_signs &&
                      c->step_rt == 0 &&
-                     c->groups == 1 && sbd::dsb16_ok(c->Rs) && (int64_t)c->n * c->Rs > sbd::kDsb16Spins &&
+                     c->groups == 1 && sbd::dsb16_ok(c->Rs) &&
+                     ((int64_t)c->n * c->Rs > sbd::kDsb16Spins ||
+                      c->step_rpc > 2 * (256 / sbd::make_tiling(c->Rs).G)) &&
                      !(c->tiled_ok && use_tiled && c->Rs % sbd::kTileRT == 0);
   const sbd::Tiling t = dsb16 ? sbd::make_tiling_dsb16(c->Rs) : step_tiling(c);
   sbd::StepArgs a;

@@ -29,6 +29,11 @@ bool dsb16_ok(int R);
 // 24.4, R = 64 (2.52 M) 31.5 / 34.4; 67,374 rows R = 32 (2.16 M) 17.2 / 13.4, R = 64
 // (4.31 M) 18.8 / 22.3; 10,999 rows R = 128 (1.41 M) 14.5 / 10.9, R = 256 (2.82 M) 14.9 /
 // 18.3; 98,134 rows R = 16 (1.57 M) 62.6 / 41.3, R = 32 (3.14 M) 49.3 / 56.3.
+// Rows per CTA set by option (SB_OPT_STEP_RPC): more than two rows for each of
+// k_step's lane groups queue there, and the other kernel, with a quarter of the lanes
+// to a row, holds more of them at once. 10,999 rows, 32 rows per CTA, R = 128: 14.7 /
+// 20.4; 64, R = 64: 9.6 / 14.5; 32, R = 64 (two a group): 9.6 / 12.2; 64, R = 32: 9.0 /
+// 8.6, and 67,374 rows 17.2 / 14.7.
 constexpr int64_t kDsb16Spins = 2400000;
 // rows per CTA of k_step_dsb16 for a step's rows-per-CTA setting rpc
 int dsb16_rows_per_cta(int rpc);

@@ -51,3 +51,19 @@ def test_replica_counts_and_options():
     ctx = sb.sb_create(big, *run1._sparse(big, 4, 3), sb.SB_J_BF16)
     sb.sb_run(ctx, "dsb", 1.0, 0.05, 0.5, 3, 64, seed=1)
     assert sb.sb_step_kernels(ctx) == "k_step_dsb16"
+
+
+@pytest.mark.parametrize("rpc,R,kernel", [(0, 128, "k_step"), (32, 128, "k_step_dsb16"), (32, 64, "k_step"),
+                                          (64, 64, "k_step_dsb16"), (64, 32, "k_step"), (0, 256, "k_step_dsb16")])
+def test_dsb_rows_per_cta(rpc, R, kernel):
+    """1.4 M spins at R = 128: more than two rows to a lane group take the other kernel."""
+    n = 11000
+    q = run1._sparse(n, 8, 3)
+    ctx = sb.sb_create(n, *q, sb.SB_J_BF16)
+    out = []
+    for v in (rpc, 0):
+        sb.sb_set_option(ctx, sb.SB_OPT_STEP_RPC, v)
+        sb.sb_run(ctx, "dsb", 1.0, 0.4, 0.3, 5, R, seed=2)
+        out.append((sb.sb_step_kernels(ctx),) + sb.sb_get_state(ctx))
+    assert out[0][0] == kernel
+    assert np.array_equal(out[0][1], out[1][1]) and np.array_equal(out[0][2], out[1][2])
