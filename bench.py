@@ -208,22 +208,22 @@ _CAPTURE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-co
             "--profile-steps 4")
 MEASURED_TRAFFIC = {
     # the full batch holds ~8 GB on the device: counters are taken on every 4th
-    # event (128 events, sum N = 1,120,853; 1,511,852,544 B per step) and scaled
+    # event (128 events, sum N = 1,120,853; 1,511,849,472 B per step) and scaled
     # by the spin-updates (x 5,677,517 / 1,120,853). Per spin-update the traffic
     # rises with the working set (20.7 / 21.3 / 22.4 B at 64 / 128 / 512 events with
     # an earlier form of the kernels), so this is a lower bound by about 5 %.
-    ("batch512", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
-        "bytes_per_step": 7658068025,
+    ("batch512", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "41550960397f40af"): {
+        "bytes_per_step": 7658052464,
         "source": _CAPTURE.format(args=" --events 128") +
         " (every 4th event; scaled to the 512 events by the spin-updates)"},
-    ("event10k", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
-        "bytes_per_step": 74019328 + 19165696 + 708126720 + 485044480,
+    ("event10k", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "41550960397f40af"): {
+        "bytes_per_step": 74062336 + 19192576 + 707954688 + 485044480,
         "source": _CAPTURE.format(args=" --workload event10k --variant dsb")},
-    ("event10k_1m", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "ed6ae3d84307a3da"): {
-        "bytes_per_step": 238134272 + 81408512 + 1648426752 + 1191499776,
+    ("event10k_1m", "dsb", ("k_fac_sum_sgn", "k_step_fac_sgn"), "41550960397f40af"): {
+        "bytes_per_step": 238162944 + 81656320 + 1641257984 + 1135402496,
         "source": _CAPTURE.format(args=" --workload event10k_1m --variant dsb")},
-    ("event1000", "bsb", ("k_fac_sum", "k_step_rw"), "babe6105eba29716"): {
-        "bytes_per_step": 40308992 + 1826304 + 101010944 + 35682048,
+    ("event1000", "bsb", ("k_fac_sum", "k_step_rw"), "61e06dcbab9b592a"): {
+        "bytes_per_step": 40312832 + 1972480 + 101012736 + 35805184,
         "source": _CAPTURE.format(args=" --workload event1000")},
 }
 
