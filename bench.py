@@ -548,8 +548,9 @@ def time_to_target(sb, w, pairs, ctx, stream, dev, plain_events, plain_runs=64, 
     e's replicas at or below its target at checkpoint k; one batched run of
     R_b replicas succeeds for event e with P_e(k) = 1 - (1 - p_e(k))^R_b.
 
-    Plain FP32 form (FP32 J, one replica, one event, one kernel launch per
-    step, no graph): `plain_runs` runs of each sampled event and configuration
+    Plain FP32 form (FP32 J, one replica, one event, no graph: all steps in
+    one launch where the couplings fit in the SMs' shared memory, else one
+    kernel launch per step): `plain_runs` runs of each sampled event and configuration
     with checkpoints give its own p_e(k); a plain run is timed without
     checkpoints and t_e(k) = t_run,e k / (m S). Events are solved one after
     another, each with its own best round; the workload's plain TTT is E times
