@@ -128,7 +128,7 @@ struct sb_ctx {
   // readout (sized for eR replicas, independent of the state's R)
   int32_t eR = 0;
   // blocks of rows whose energies are summed first, and their sums for eR
-  // replicas: in FP64 ([0], always there) and from selection bits ([1])
+  // replicas: in FP64 ([0]) and from selection bits ([1])
   struct EnergyBlocks {
     int32_t rows = 0, nblk = 0;
     int32_t* d_row = nullptr;
@@ -664,28 +664,30 @@ sb_status ensure_state(sb_ctx* c, int32_t R) {
 }
 
 // Nothing here is freed while the replica count stays, whatever the weights become:
-// a readout that a caller has recorded keeps its buffers. And nothing new is made for
-// the bits while one is being recorded: it takes the FP64 sums.
+// a readout that a caller has recorded keeps its buffers. And nothing new is made while
+// one is being recorded if the buffers of the other sums are there: it takes those.
 sb_status ensure_readout(sb_ctx* c, int32_t R, bool recording) {
   sb_status st;
-  if (c->eR != R || !c->eb[0].d_partial || !c->d_Eall) {
+  if (c->eR != R || !c->d_Eall) {
     free_readout(c);
-    if ((st = ensure_energy_blocks(c, c->eb[0], std::max(kEnergyRowsMin, 256 / sbd::make_tiling(R).G), R)) ||
-        (st = dalloc(&c->d_Eall, (size_t)c->E * R)))
-      return st;
+    if ((st = dalloc(&c->d_Eall, (size_t)c->E * R))) return st;
     c->eR = R;
   }
-  if (!c->b_whole || c->d_bits || c->bits_oom || recording) return SB_OK;
-  // whole-number couplings: larger blocks where that still leaves eight CTAs
-  // per SM (fewer partial sums to add; the 472,812-row event: 2 ms of block sums)
-  if (!c->sms) SB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
-  const int32_t rows = std::min(sbd::kEnergyBitRows, std::max(kEnergyRowsMin, c->n / (c->sms * 8) / 64 * 64));
-  st = ensure_energy_blocks(c, c->eb[1], rows, R);
-  if (!st) st = dalloc(&c->d_bits, (size_t)c->n * sbd::energy_bit_stride(R));
-  if (st != SB_ERR_OOM) return st;
-  dfree(c->eb[1].d_partial);  // the FP64 sums need none of it
-  c->bits_oom = true;
-  return SB_OK;
+  if (c->b_whole && !c->d_bits && !c->bits_oom && !(recording && c->eb[0].d_partial)) {
+    // whole-number couplings: larger blocks where that still leaves eight CTAs
+    // per SM (fewer partial sums to add; the 472,812-row event: 2 ms of block sums)
+    if (!c->sms) SB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+    const int32_t rows = std::min(sbd::kEnergyBitRows, std::max(kEnergyRowsMin, c->n / (c->sms * 8) / 64 * 64));
+    st = ensure_energy_blocks(c, c->eb[1], rows, R);
+    if (!st) st = dalloc(&c->d_bits, (size_t)c->n * sbd::energy_bit_stride(R));
+    if (st && st != SB_ERR_OOM) return st;
+    if (st) {  // the FP64 sums need less
+      dfree(c->eb[1].d_partial);
+      c->bits_oom = true;
+    }
+  }
+  if ((c->b_whole && c->d_bits) || c->eb[0].d_partial || (recording && c->eb[1].d_partial)) return SB_OK;
+  return ensure_energy_blocks(c, c->eb[0], std::max(kEnergyRowsMin, 256 / sbd::make_tiling(R).G), R);
 }
 
 // Cut rows into blocks (in row order) whose union of neighbour rows plus own
@@ -2709,6 +2711,7 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   // k_convert's verdict on the weights of the day picks one on the device.
   const bool bits = c->b_whole && c->d_bits;
   const int32_t* const gate = bits && recording ? c->d_inexact : nullptr;
+  const sb_ctx::EnergyBlocks& blk = bits || !c->eb[0].d_partial ? c->eb[1] : c->eb[0];
   if (bits) {
     sbd::EnergyBitArgs b;
     b.rowptr = c->d_rowptr;
@@ -2718,21 +2721,16 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
     b.qlin = c->d_qlin;
     b.bits = c->d_bits;
     b.bstride = sbd::energy_bit_stride(R);
-    b.blk_row = c->eb[1].d_row;
-    b.nblk = c->eb[1].nblk;
+    b.blk_row = blk.d_row;
+    b.nblk = blk.nblk;
     b.n = c->n;
     b.R = R;
-    b.partial = c->eb[1].d_partial;
+    b.partial = blk.d_partial;
     b.gate = gate;
     b.nnz = c->nnz;
     SB_CUDA(sbd::launch_select_bits(d_spins ? nullptr : c->d_x[c->cur], c->Rs, d_spins, c->n, R,
                                     c->d_bits, s));
     SB_CUDA(sbd::launch_energy_bits(b, s));
-    SB_CUDA(sbd::launch_energy_reduce(b.partial, c->eb[1].d_ev0, c->E, R, E_all, gate, 0, s));
-  }
-  if (bits && !gate) {
-    SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, c->d_bestr, err, s));
-    return SB_OK;
   }
   const sbd::Tiling t = sbd::make_tiling(R);
   sbd::EnergyArgs a;
@@ -2743,16 +2741,16 @@ sb_status readout(sb_ctx* c, const int8_t* d_spins, int32_t R, cudaStream_t s,
   a.x = d_spins ? nullptr : c->d_x[c->cur];
   a.xstride = c->Rs;
   a.spins = d_spins;
-  a.blk_row = c->eb[0].d_row;
-  a.nblk = c->eb[0].nblk;
+  a.blk_row = blk.d_row;
+  a.nblk = blk.nblk;
   a.n = c->n;
   a.R = R;
   a.G = t.G;
-  a.partial = c->eb[0].d_partial;
+  a.partial = blk.d_partial;
   a.gate = gate;
   a.nnz = c->nnz;
-  SB_CUDA(sbd::launch_energy_partial(t, a, s));
-  SB_CUDA(sbd::launch_energy_reduce(a.partial, c->eb[0].d_ev0, c->E, R, E_all, gate, 1, s));
+  if (!bits || gate) SB_CUDA(sbd::launch_energy_partial(t, a, s));
+  SB_CUDA(sbd::launch_energy_reduce(blk.d_partial, blk.d_ev0, c->E, R, E_all, s));
   SB_CUDA(sbd::launch_argmin(E_all, c->E, R, best_E, best_r, c->d_bestr, err, s));
   return SB_OK;
 }

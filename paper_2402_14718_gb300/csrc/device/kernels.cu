@@ -1430,10 +1430,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_energy_bits(const EnergyBitArgs a
 constexpr int kReduceWarps = 32;
 __global__ void __launch_bounds__(32 * kReduceWarps) k_energy_reduce(const double* partial,
                                                                      const int32_t* ev_blk0,
-                                                                     int32_t R, double* out,
-                                                                     const int32_t* gate, int want) {
+                                                                     int32_t R, double* out) {
   __shared__ double sm[kReduceWarps][32];
-  if (gate && (*gate != 0) != (want != 0)) return;
   const int e = blockIdx.y;
   const int b0 = ev_blk0[e], b1 = ev_blk0[e + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1817,11 +1815,10 @@ cudaError_t launch_energy_partial(const Tiling& t, const EnergyArgs& a, cudaStre
 }
 
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
-                                 int32_t R, double* E_out, const int32_t* gate, int want,
-                                 cudaStream_t s) {
+                                 int32_t R, double* E_out, cudaStream_t s) {
   if (E <= 0 || R <= 0) return cudaSuccess;
   dim3 grid((R + 31) / 32, E);
-  k_energy_reduce<<<grid, 32 * kReduceWarps, 0, s>>>(partial, ev_blk0, R, E_out, gate, want);
+  k_energy_reduce<<<grid, 32 * kReduceWarps, 0, s>>>(partial, ev_blk0, R, E_out);
   return cudaGetLastError();
 }
 

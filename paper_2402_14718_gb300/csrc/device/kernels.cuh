@@ -172,11 +172,9 @@ inline int32_t energy_bit_stride(int R) { return (R + 31) / 32 * 4; }
 cudaError_t launch_select_bits(const float* x, int32_t xstride, const int8_t* spins, int32_t n,
                                int32_t R, uint8_t* bits, cudaStream_t s);
 cudaError_t launch_energy_bits(const EnergyBitArgs& a, cudaStream_t s);
-// E[e*R + r] = sum of the event's block partials, in a fixed order. gate (device, may
-// be NULL): does nothing unless (*gate != 0) == want.
+// E[e*R + r] = sum of the event's block partials, in a fixed order.
 cudaError_t launch_energy_reduce(const double* partial, const int32_t* ev_blk0, int32_t E,
-                                 int32_t R, double* E_out, const int32_t* gate, int want,
-                                 cudaStream_t s);
+                                 int32_t R, double* E_out, cudaStream_t s);
 // arg-min over replicas per event (ties -> lowest index).
 // own_r (device, may be NULL): best_r once more; err (device, may be NULL): where it
 // is set, every energy becomes NaN

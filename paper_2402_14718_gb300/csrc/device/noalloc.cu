@@ -191,7 +191,7 @@ extern "C" sb_status sb_energy_noalloc(int32_t n, const int32_t* d_rowptr, const
     a.partial = partial;  // every (block, replica) entry is written before it is read
     e = sbd::launch_energy_partial(t, a, cs);
   }
-  if (e == cudaSuccess) e = sbd::launch_energy_reduce(partial, ev_blk0, 1, replicas, d_E, nullptr, 0, cs);
+  if (e == cudaSuccess) e = sbd::launch_energy_reduce(partial, ev_blk0, 1, replicas, d_E, cs);
   if (e == cudaSuccess && d_best_E) e = sbd::launch_argmin(d_E, 1, replicas, d_best_E, d_best_r, nullptr, nullptr, cs);
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -107,7 +107,8 @@ def test_readout(n, R, first):
         assert b.item() == E.min().item() and r.item() == E.argmin().item()
 
 
-def test_readout_recorded_right_after_the_weights_became_whole():
+@pytest.mark.parametrize("before,then", [(0.6, 1.0), (1.0, 0.6), (1.0, 1.0)])
+def test_readout_recorded_right_after_new_weights(before, then):
     """Buffers made for other weights serve the recording: it makes none of its own."""
     import torch
     n, R = 3000, 8
@@ -116,12 +117,12 @@ def test_readout_recorded_right_after_the_weights_became_whole():
     x = np.random.default_rng(1).uniform(-1, 1, size=(n, R)).astype(np.float32)
     E = torch.zeros((1, R), dtype=torch.float64, device="cuda")
     stream = torch.cuda.Stream()
-    _weights(ctx, q, 0.6)
+    _weights(ctx, q, before)
     sb.sb_set_state(ctx, x, x)
     sb.sb_readout_device(ctx, E, stream=stream)
-    _weights(ctx, q, 1.0)
+    _weights(ctx, q, then)
     g = _record(stream, lambda: sb.sb_readout_device(ctx, E, stream=stream))
-    for w_c in (1.0, 0.6):
+    for w_c in (then, 1.0, 0.6, 1.0):
         _weights(ctx, q, w_c)
         g.replay()
         torch.cuda.synchronize()
