@@ -1629,23 +1629,27 @@ sb_status set_factor(sb_ctx* c, int32_t n_ids, int32_t K, const int32_t* member,
   // kernel's time). dSB: whole blocks, their members in words of four (row and
   // slot), the large ones spread over a CTA (ensure_fac_ctas).
   constexpr int64_t kChunk = 16;
-  std::vector<int4> items, items1;
-  std::vector<uint32_t> gword;
-  std::vector<int32_t> bcnt((size_t)ng), bev((size_t)ng, 0);
-  items1.reserve((size_t)ng);
-  gword.reserve(gmem.size() + (size_t)ng * 2);
+  std::vector<int4> items, items1((size_t)ng);
+  std::vector<int32_t> bcnt((size_t)ng), bev((size_t)ng, 0), word0((size_t)ng + 1, 0);
   for (int32_t ga = 0; ga < ng; ++ga) {
-    const int32_t w0 = (int32_t)(gword.size() / 4);
-    for (int s = 0; s < K; ++s)
-      for (int32_t t = gseg[(size_t)ga * K + s]; t < gseg[(size_t)ga * K + s + 1]; ++t)
-        gword.push_back((uint32_t)gmem[t] | (uint32_t)s << 28);
-    while (gword.size() % 4) gword.push_back(sbd::kFacPad);
-    items1.push_back(make_int4(ga, w0, (int32_t)(gword.size() / 4), 0));
     bcnt[ga] = gseg[(size_t)ga * K + K] - gseg[(size_t)ga * K];
-    if (c->E > 1 && bcnt[ga] > 0)
-      bev[ga] = (int32_t)(std::upper_bound(c->ev_row0.begin(), c->ev_row0.end(),
-                                           gmem[gseg[(size_t)ga * K]]) - c->ev_row0.begin()) - 1;
+    word0[ga + 1] = word0[ga] + (bcnt[ga] + 3) / 4;
   }
+  std::vector<uint32_t> gword((size_t)word0[ng] * 4);
+  // on host threads where there is enough to fill to pay for them
+  parallel_parts(ng, 64, [&](int, int64_t b0, int64_t b1) {
+    for (int64_t ga = b0; ga < b1; ++ga) {
+      uint32_t* w = gword.data() + (size_t)word0[ga] * 4;
+      for (int s = 0; s < K; ++s)
+        for (int32_t t = gseg[(size_t)ga * K + s]; t < gseg[(size_t)ga * K + s + 1]; ++t)
+          *w++ = (uint32_t)gmem[t] | (uint32_t)s << 28;
+      for (uint32_t* const end = gword.data() + (size_t)word0[ga + 1] * 4; w < end;) *w++ = sbd::kFacPad;
+      items1[ga] = make_int4((int32_t)ga, word0[ga], word0[ga + 1], 0);
+      if (c->E > 1 && bcnt[ga] > 0)
+        bev[ga] = (int32_t)(std::upper_bound(c->ev_row0.begin(), c->ev_row0.end(),
+                                             gmem[gseg[(size_t)ga * K]]) - c->ev_row0.begin()) - 1;
+    }
+  }, gmem.size() < 500000 ? INT64_MAX : 1);
   std::vector<int32_t> gnc(ng), gscr0(ng, -1);
   int32_t nslots = 0;
   for (int32_t ga = 0; ga < ng; ++ga) {
